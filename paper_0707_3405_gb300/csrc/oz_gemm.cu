@@ -39,21 +39,32 @@
 // Data path: a split kernel writes each operand's digits once, as 64-byte-swizzled
 // K-major BF16 tiles in the exact order one pipeline stage needs them (six slices
 // of a 128- or 64-row tile x 32 K values, contiguous), plus the chunk scales.
-// The product kernel (one CTA per output tile and K split, 10 warps) streams the
-// stages with one bulk copy per operand (cp.async.bulk into a 3-stage ring,
-// mbarrier transaction counts), one thread issues the 42 MMAs of a stage
-// (21 slice pairs x 2 K-steps of 16, M = 128, N = 64), and eight warps read the
-// six level accumulators after every chunk (tcgen05.ld) and fold them into the
-// double-FP32 sums.  Long reductions (A^H B) are split over the GPU and cut
-// into K slabs that bound the digit scratch; FP64 partial tiles are summed in
-// a fixed order (reproducible).  Every mbarrier wait is bounded; a wait that
-// runs out sets a device flag (read by oz_check_error) and the CTA stops,
-// waits (bounded) for its copies and MMAs in flight, frees its TMEM and returns.
+// The product kernel (k_oz_mma: persistent, one CTA of 18 warps per SM, each taking every
+// gridDim-th item, an output tile and a part of its reduction) streams the stages with one bulk
+// copy per operand (cp.async.bulk into a 3-stage ring, mbarrier transaction counts), one warp
+// issues the 42 MMAs of a stage (21 slice pairs x 2 K-steps of 16, M = 128, N = 64), and sixteen
+// warps read the six levels of every chunk (tcgen05.ld) and fold them into the double-FP32 sums.
+// The level accumulators rotate through eight slots of TMEM, so a chunk starts while the last
+// levels of the one before it, and an item while the output of the one before it, are still read.
+// Long reductions (A^H B) are split over the GPU and cut into K slabs that bound the digit
+// scratch; FP64 partial tiles are summed in a fixed order (reproducible).  Every mbarrier wait is
+// bounded; a wait that runs out sets a device flag (read by oz_check_error), and the CTA waits
+// (bounded) for its copies and MMAs in flight, frees its TMEM and returns.
+//
+// What bounds it: the tensor cores would take 36 cycles an MMA (the left slice held in the
+// collector, the right one read at 128 bytes a cycle), 6000 a chunk; issue, the waits for the
+// stages and the slots and the folding leave about 9300.  Measured on a GB300 (SM clock
+// 1.93 GHz), before and after the issue by a whole warp, the rotating slots, the folding without
+// FP64 instructions and the persistent schedule:
+//   A B    57925 x 320 x 320     1.97 -> 0.99 ms   (24 -> 48 TFLOP/s complex128)
+//   A^H B  512 x 128 x 113081    2.66 -> 1.64 ms   (0.66 ms of it the split into digits)
+//   Gram   1152, K = 113081      25.8 -> 12.0 ms   (2.7 ms of it the split)
 #include "common.cuh"
 #include "tc.cuh"
 
 #include <algorithm>
 #include <cmath>
+#include <utility>
 
 namespace lg {
 
@@ -74,9 +85,12 @@ constexpr int kStageA = kSlices * kTileA;    // 48 KB
 constexpr int kStageB = kSlices * kTileB;    // 24 KB
 constexpr int kStageBytes = kStageA + kStageB;
 constexpr int kRing = 3;
-constexpr int kEpiWarps = 8;
+constexpr long long kMmaSpin = 1 << 18;      // polls of one wait of the MMA warp (milliseconds)
+constexpr int kEpiWarps = 16;
+constexpr int kCols = TQ / (kEpiWarps / 4);  // columns of a tile row that one epilogue warp folds
 constexpr int kThreads = 32 * (kEpiWarps + 2);   // + producer warp + MMA warp
-constexpr int kTmemCols = 512;               // 6 levels x 64 columns used
+constexpr int kSlots = 8;                    // level accumulators of 64 columns in TMEM
+constexpr int kTmemCols = kSlots * TQ;       // all 512
 constexpr size_t kSmem = (size_t)kRing * kStageBytes + 1024 + 256;   // ring + alignment + barriers
 
 // split modes: how a complex vector becomes real rows of a factor
@@ -94,7 +108,7 @@ __device__ __forceinline__ uint32_t swz64(int r, int c) {
 
 // Shared-memory matrix descriptor for a 64-byte-swizzled K-major tile: stride between
 // 8-row groups 512 bytes, descriptor version 1, swizzle mode 4 (64 bytes).
-__device__ __forceinline__ uint64_t make_desc_sw64(uint32_t saddr) {
+__host__ __device__ constexpr uint64_t make_desc_sw64(uint32_t saddr) {
     uint64_t d = 0;
     d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
     d |= (uint64_t)1u << 16;
@@ -120,11 +134,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                  : "memory");
 }
 
-__device__ __forceinline__ float pow2f(int e) {
-    if (e >= -126 && e <= 127) return __int_as_float((e + 127) << 23);
-    return ldexpf(1.0f, e);
-}
-
 // Knuth TwoSum: s + err = a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &err) {
     s = a + b;
@@ -139,6 +148,28 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float x, float y) {
     e += lo + y;
     hi = s + e;
     lo = e - (hi - s);
+}
+
+// hi + lo as an FP64 number, rounded to nearest, in integer arithmetic: a warp-wide FP64 instruction
+// occupies its sub-partition for 64 cycles on this GPU.  (hi, lo) is normalised (|lo| at most half a
+// unit in the last place of hi).  With e the exponent of hi, hi = mh 2^(e - 23) and lo, in units of
+// 2^(e - 52), is an integer of at most 2^28 once rounded; their sum is the mantissa up to one
+// renormalisation (a power of two less something).
+__device__ __forceinline__ double pair_to_double(float hi, float lo) {
+    // tiny and huge numbers by 2^64 or 2^-64, exactly, into the middle of the exponent range
+    const uint32_t b0 = (__float_as_uint(hi) >> 23) & 255u;
+    const float fac = b0 < 64u ? 0x1p64f : b0 > 190u ? 0x1p-64f : 1.f;
+    const int adj = b0 < 64u ? -64 : b0 > 190u ? 64 : 0;
+    const uint32_t u = __float_as_uint(hi * fac), be = (u >> 23) & 255u;
+    // lo 2^(52 - e) as two exact factors, e = be - 127
+    const float f = (u >> 31 ? -lo : lo) * fac * __uint_as_float((254u - be) << 23) * 0x1p52f;
+    unsigned long long m = ((unsigned long long)((u & 0x7FFFFFu) | 0x800000u) << 29) + (long long)__float2int_rn(f);
+    const uint32_t under = (m >> 52) == 0 ? 1u : 0u;            // hi a power of two and lo against it
+    m <<= under;
+    uint32_t top = (be - under + (uint32_t)(adj + 1023 - 127 - 1)) << 20;   // the leading one adds the exponent
+    if (be == 0) { m = 0; top = 0; }                             // zero
+    if (be == 255) { m = (unsigned long long)(u & 0x7FFFFFu) << 29; top = 0x7FF00000u; }   // infinite, not a number
+    return __hiloint2double((int)((top + (uint32_t)(m >> 32)) | (u & 0x80000000u)), (int)(uint32_t)m);
 }
 
 // The six base-256 digits of x relative to the chunk scale 2^e (|x| < 2^e), most significant
@@ -258,6 +289,30 @@ k_oz_split(const z64 *__restrict__ X, long long rs, long long ks, int nvec, int 
 }
 
 // ------------------------------------------------------------------ product
+// Order of a stage's 42 MMAs (21 slice pairs x 2 K-steps): the MMAs of one left slice and K-step
+// together, so that the slice is read from shared memory once (collector), slice 1 first, so that
+// the levels are complete in the order 0 .. 5.
+constexpr int kMmas = kSlices * (kSlices + 1);
+struct MmaOrder {
+    int L[kMmas], p[kMmas], kk[kMmas], col[kMmas];
+    bool first[kMmas], last[kMmas];          // first / last MMA of its level in the stage
+};
+constexpr MmaOrder make_order() {
+    MmaOrder o{};
+    int i = 0;
+    for (int p = 0; p < kSlices; ++p)
+        for (int kk = 0; kk < 2; ++kk)
+            for (int L = p; L < kLevels; ++L, ++i) {
+                o.L[i] = L;
+                o.p[i] = p;
+                o.kk[i] = kk;
+                o.col[i] = p + 1 == kLevels ? kDiscard : L == p ? kFill : L + 1 == kLevels ? kLastUse : kUse;
+                o.first[i] = p == 0 && kk == 0;
+                o.last[i] = p == L && kk == 1;
+            }
+    return o;
+}
+
 struct OzArgs {
     const unsigned char *At, *Bt;   // digit tiles of the left / right factor
     const int *EA, *EB;             // chunk exponents [chunk][vector]
@@ -265,6 +320,7 @@ struct OzArgs {
     int nvA_pad, nvB_pad;           // padded vector counts of the exponent tables
     int nchunks, cps;               // chunks of the slab, chunks per K split
     int lower;                      // skip tiles with every output column j above every row i
+    int tq, tiles, nsplit;          // right tiles; output tiles that are computed; K splits
     // mode 0: FP64 partial tiles P[split][q][r] (written, or added to when accumulate)
     double *P;
     int ldp;
@@ -273,11 +329,60 @@ struct OzArgs {
     // mode 1: D = alpha (product) + beta C for complex rows row0 .. of A B
     int M, n, row0;
     double alpha, beta;
+    int scaled;                     // alpha != 1 or beta != 0
     const z64 *C;
     int ldc;
     z64 *D;
     int ldd;
 };
+
+// One unit of work: output tile (rt, qt) and chunks [c0, c0 + nch) of its reduction.
+struct OzItem {
+    int rt, qt, z, c0, nch;
+};
+__device__ __forceinline__ OzItem oz_item(const OzArgs &a, int it) {
+    OzItem w;
+    w.z = it / a.tiles;
+    int t = it - w.z * a.tiles;
+    if (a.lower) {   // row tile rt has right tiles 0 .. 4 rt + 3 (right rows 64 qt .. are columns j >= 32 qt)
+        w.rt = 0;
+        for (int n = min(a.tq, 4); t >= n; n = min(a.tq, 4 * w.rt + 4)) {
+            t -= n;
+            ++w.rt;
+        }
+        w.qt = t;
+    } else {
+        w.rt = t / a.tq;
+        w.qt = t - w.rt * a.tq;
+    }
+    w.c0 = w.z * a.cps;
+    w.nch = max(0, min(a.nchunks - w.c0, a.cps));
+    return w;
+}
+
+// MMA I of a stage (stage st of the chunk whose levels are u0 ..), with the waits and signals of its level.
+template <int I>
+__device__ __forceinline__ void issue_one(uint32_t el, uint32_t tmem, int u0, int st, uint32_t alo, uint32_t blo,
+                                          uint64_t *accf, uint64_t *acce, bool &late) {
+    constexpr MmaOrder O = make_order();
+    constexpr int L = O.L[I], p = O.p[I], kk = O.kk[I];
+    constexpr uint32_t HI = (uint32_t)(make_desc_sw64(0) >> 32);
+    const int u = u0 + L, slot = u & (kSlots - 1);
+    if (O.first[I] && st == 0 && u >= kSlots) {
+        late |= !mbar_wait(&acce[slot], (uint32_t)((u / kSlots - 1) & 1), kMmaSpin);
+        __syncwarp();
+        fence_after_sync();
+    }
+    mma_bf16_warp<O.col[I], HI, p * kTileA + kk * 32, (L - p) * kTileB + kk * 32>(
+        el, tmem + (uint32_t)(slot * TQ), alo, blo, make_idesc_bf16(TM, TQ), (O.first[I] && st == 0) ? 0u : 1u);
+    if (O.last[I] && st == kChunkStages - 1) mma_commit_warp(el, &accf[slot]);
+}
+template <int... I>
+__device__ __forceinline__ void issue_stage(std::integer_sequence<int, I...>, uint32_t el, uint32_t tmem, int u0, int st,
+                                            uint32_t alo, uint32_t blo, uint64_t *accf, uint64_t *acce,
+                                            bool &late) {
+    (issue_one<I>(el, tmem, u0, st, alo, blo, accf, acce, late), ...);
+}
 
 template <int OUT>
 __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
@@ -286,188 +391,212 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
                                                             ~(uintptr_t)1023);
     uint64_t *full = reinterpret_cast<uint64_t *>(base + kRing * kStageBytes);
     uint64_t *empty = full + kRing;
-    uint64_t *accf = empty + kRing;
-    uint64_t *acce = accf + 1;              // one per level: its accumulator has been read
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + kLevels);
+    uint64_t *accf = empty + kRing;         // one per slot: its level's sums of the chunk are complete
+    uint64_t *acce = accf + kSlots;         // one per slot: its level has been read
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + kSlots);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int qt = blockIdx.x, rt = blockIdx.y, z = blockIdx.z;
-    if (a.lower) {
-        // right rows 64 qt .. are columns j >= 32 qt (two rows per column); left rows are i
-        if (32 * qt > TM * rt + TM - 1) return;
-    }
-    const int c0 = z * a.cps, c1 = min(a.nchunks, c0 + a.cps);
-    const int nch = max(0, c1 - c0);
+    const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
     if (warp == kEpiWarps + 1) tmem_alloc(tslot, kTmemCols);
     if (tid == 0) {
         for (int s = 0; s < kRing; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(accf, 1);
-        for (int L = 0; L < kLevels; ++L) mbar_init(&acce[L], kEpiWarps);
+        for (int k = 0; k < kSlots; ++k) {
+            mbar_init(&accf[k], 1);
+            mbar_init(&acce[k], kEpiWarps);
+        }
         *abort_flag = 0;
     }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    const uint32_t tmem = *tslot;
-    const int nst = nch * kChunkStages;
+    const uint32_t tmem = uniform(*tslot);
+    const int it0 = blockIdx.x, nit = a.tiles * a.nsplit, step = gridDim.x;
     if (warp == kEpiWarps) {
         // ---- producer: one bulk copy per factor per stage
         if (lane == 0) {
             int g = 0;
-            for (; g < nst && !*abort_flag; ++g) {
-                const int s = g % kRing;
-                if (g >= kRing && !mbar_wait(&empty[s], (uint32_t)((g / kRing - 1) & 1))) {
-                    *abort_flag = 1;
-                    break;
+            for (int it = it0; it < nit && !*abort_flag; it += step) {
+                const OzItem w = oz_item(a, it);
+                const unsigned char *gA = a.At + ((size_t)w.rt * a.KS + (size_t)w.c0 * kChunkStages) * kStageA;
+                const unsigned char *gB = a.Bt + ((size_t)w.qt * a.KS + (size_t)w.c0 * kChunkStages) * kStageB;
+                for (int t = 0; t < w.nch * kChunkStages && !*abort_flag; ++t, ++g) {
+                    const int s = g % kRing;
+                    if (g >= kRing && !mbar_wait(&empty[s], (uint32_t)((g / kRing - 1) & 1))) {
+                        *abort_flag = 1;
+                        break;
+                    }
+                    unsigned char *sA = base + s * kStageBytes, *sB = sA + kStageA;
+                    mbar_expect_tx(&full[s], kStageBytes);
+                    bulk_g2s(sA, gA + (size_t)t * kStageA, kStageA, &full[s]);
+                    bulk_g2s(sB, gB + (size_t)t * kStageB, kStageB, &full[s]);
                 }
-                const int stage = c0 * kChunkStages + g;
-                unsigned char *sA = base + s * kStageBytes, *sB = sA + kStageA;
-                mbar_expect_tx(&full[s], kStageBytes);
-                bulk_g2s(sA, a.At + ((size_t)rt * a.KS + stage) * kStageA, kStageA, &full[s]);
-                bulk_g2s(sB, a.Bt + ((size_t)qt * a.KS + stage) * kStageB, kStageB, &full[s]);
             }
             // drain: the copies of the last (up to kRing) issued stages must land before exit
             for (int h = max(0, g - kRing); h < g; ++h) mbar_wait(&full[h % kRing], (uint32_t)((h / kRing) & 1));
         }
     } else if (warp == kEpiWarps + 1) {
-        // ---- MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t IDESC = make_idesc_bf16(TM, TQ);
-            int g = 0, last_commit = -1;
-            bool ok = true;
-            for (int ci = 0; ci < nch && ok; ++ci) {
-                for (int st = 0; st < kChunkStages; ++st, ++g) {
-                    const int s = g % kRing;
-                    if (*abort_flag || !mbar_wait(&full[s], (uint32_t)((g / kRing) & 1))) { ok = false; break; }
-                    fence_after_sync();
-                    const uint32_t sA = smem_u32(base + s * kStageBytes), sB = sA + kStageA;
-                    if (st == 0) {
-                        // first stage of a chunk, level by level: level L starts (accumulate = 0) as
-                        // soon as the epilogue has read level L of the previous chunk, so the reads
-                        // and the double-FP32 folding overlap this chunk's MMAs
-                        for (int L = 0; L < kLevels && ok; ++L) {
-                            if (ci > 0) {
-                                if (!mbar_wait(&acce[L], (uint32_t)((ci - 1) & 1))) { ok = false; break; }
-                                fence_after_sync();
-                            }
-                            for (int p = 0; p <= L; ++p)
-#pragma unroll
-                                for (int kk = 0; kk < 2; ++kk)
-                                    mma_bf16(tmem + (uint32_t)(L * TQ), make_desc_sw64(sA + p * kTileA + kk * 32),
-                                             make_desc_sw64(sB + (L - p) * kTileB + kk * 32), IDESC,
-                                             (p | kk) ? 1u : 0u);
-                        }
-                        if (!ok) break;
-                    } else {
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                            for (int p = 0; p < kSlices; ++p)
-#pragma unroll
-                                for (int q = 0; q < kSlices - p; ++q)
-                                    mma_bf16(tmem + (uint32_t)((p + q) * TQ), make_desc_sw64(sA + p * kTileA + kk * 32),
-                                             make_desc_sw64(sB + q * kTileB + kk * 32), IDESC, 1u);
-                    }
-                    mma_commit(&empty[s]);
-                    last_commit = s;
-                }
-                if (ok) mma_commit(accf);
-            }
-            if (!ok) {
-                *abort_flag = 1;
-                atomicExch(&g_oz_err, 1);
-                // wait (bounded) for the MMAs already issued before the CTA frees its TMEM
-                if (last_commit >= 0) {
-                    const int h = g - 1;
-                    mbar_wait(&empty[h % kRing], (uint32_t)((h / kRing) & 1));
-                }
+        // ---- MMA issuer: the whole warp, one elected lane issuing.  Nothing in its loop depends on how
+        // a wait ended, its limit included: a branch or a predicate that does makes the compiler give
+        // up uniform registers (80 cycles an MMA instead of 45).  A wait that runs out (kMmaSpin polls,
+        // so that even a CTA whose every wait runs out ends within seconds) is recorded, the rest is
+        // issued on whatever the ring holds, and the error flag discards the result.
+        const uint32_t el = elect_one();
+        const uint32_t d0 = (uint32_t)make_desc_sw64(uniform(smem_u32(base)));
+        bool late = false;
+        int s = 0;                           // ring position
+        uint32_t ph = 0;                     // and its phase
+        int nc = 0;                          // chunks of all this CTA's items
+        for (int it = it0; it < nit; it += step) nc += max(0, min(a.nchunks - it / a.tiles * a.cps, a.cps));
+        for (int ci = 0; ci < nc; ++ci) {
+            const int u0 = kLevels * ci;     // level L of chunk ci is the (u0 + L)-th level of the CTA
+            for (int st = 0; st < kChunkStages; ++st) {
+                late |= !mbar_wait(&full[s], ph, kMmaSpin);
+                __syncwarp();
+                fence_after_sync();
+                const uint32_t alo = d0 + ((uint32_t)(s * kStageBytes) >> 4), blo = alo + (kStageA >> 4);
+                issue_stage(std::make_integer_sequence<int, kMmas>{}, el, tmem, u0, st, alo, blo, accf, acce, late);
+                mma_commit_warp(el, &empty[s]);
+                if (++s == kRing) { s = 0; ph ^= 1; }
             }
         }
+        if (late) {
+            if (el) {
+                *abort_flag = 1;
+                atomicExch(&g_oz_err, 1);
+            }
+            // wait (bounded) for the last stages' MMAs before the CTA frees its TMEM
+            const int nst = nc * kChunkStages;
+            if (nst > 0) mbar_wait(&empty[(nst - 1) % kRing], (uint32_t)(((nst - 1) / kRing) & 1));
+        }
     } else {
-        // ---- epilogue: eight warps, warp w reads TMEM lanes 32 (w % 4) .., columns 32 (w / 4) ..
+        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns kCols (w / 4) ..
         const int wq = warp & 3, h = warp >> 2;
         const int row = wq * 32 + lane;
-        const uint32_t taddr = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(h * 32);
-        float ah[32], al[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) ah[j] = al[j] = 0.f;
-        const int rr = rt * TM + row;                      // real left row
-        const int rpcA = OUT == 0 ? 1 : 2, rpcB = OUT == 0 ? 2 : 1;
+        const uint32_t taddr = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(h * kCols);
+        constexpr int rpcA = OUT == 0 ? 1 : 2, rpcB = OUT == 0 ? 2 : 1;
         bool ok = true;
-        for (int ci = 0; ci < nch; ++ci) {
-            if (*abort_flag || !mbar_wait(accf, (uint32_t)(ci & 1))) { ok = false; break; }
-            fence_after_sync();
-            const int c = c0 + ci;
-            const int er = a.EA[(size_t)c * a.nvA_pad + rr / rpcA];
-            // chunk sum per column as a double-FP32 pair: levels 0-2 through TwoSum into (ch, cl);
-            // levels 3-5 (at most 2^-16 of the chunk's scale) added into cl, whose FP32 rounding
-            // then stays below 2^-40 of that scale
-            float ch[32], cl[32];
+        int u0 = 0;                                        // levels read so far
+        for (int it = it0; it < nit; it += step) {
+            const OzItem w = oz_item(a, it);
+            const int rr = w.rt * TM + row;                // real left row
+            const int *EA = a.EA + (size_t)w.c0 * a.nvA_pad + rr / rpcA;
+            const int4 *EB =
+                reinterpret_cast<const int4 *>(a.EB + (size_t)w.c0 * a.nvB_pad + (w.qt * TQ + h * kCols) / rpcB);
+            float ah[kCols], al[kCols];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) ch[j] = cl[j] = 0.f;
+            for (int j = 0; j < kCols; ++j) ah[j] = al[j] = 0.f;
+            for (int ci = 0; ci < w.nch; ++ci, u0 += kLevels) {
+                // Chunk sum per column as a double-FP32 pair (ch, cl) in units of level 2.  The levels are
+                // integers below 2^24, each worth 256 of the next: t = 256 hi + v and its rounding error
+                // v - (t - 256 hi) are exact (a fast TwoSum: either |256 hi| >= |v|, or every term is an
+                // integer below 2^25).  Levels 3-5 (at most 2^-16 of the chunk's scale) go into the low
+                // part, whose FP32 rounding then stays below 2^-40 of that scale.
+                // Levels 0-3 are read together as soon as the last of them is complete: the next chunk's
+                // levels 2-5 wait for their slots.
+                float ch[kCols], cl[kCols];
+                {
+                    const int k = (u0 + 3) & (kSlots - 1);
+                    ok = __all_sync(0xffffffffu,
+                                    !*abort_flag && mbar_wait(&accf[k], (uint32_t)(((u0 + 3) / kSlots) & 1)));
+                    if (!ok) break;
+                    fence_after_sync();
+                    float v1[kCols], v2[kCols], v3[kCols];
+                    tmem_ld16_nowait(taddr + (uint32_t)(((u0 + 0) & (kSlots - 1)) * TQ), ch);
+                    tmem_ld16_nowait(taddr + (uint32_t)(((u0 + 1) & (kSlots - 1)) * TQ), v1);
+                    tmem_ld16_nowait(taddr + (uint32_t)(((u0 + 2) & (kSlots - 1)) * TQ), v2);
+                    tmem_ld16_nowait(taddr + (uint32_t)(k * TQ), v3);
+                    tmem_wait_ld(ch, v1, v2, v3);
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane < 4) mbar_arrive(&acce[(u0 + lane) & (kSlots - 1)]);
 #pragma unroll
-            for (int L = 0; L < kLevels; ++L) {
-                const float sc = pow2f(-8 * (L + 2));
+                    for (int j = 0; j < kCols; ++j) {
+                        const float t1 = fmaf(ch[j], 256.f, v1[j]), e1 = v1[j] - fmaf(ch[j], -256.f, t1);
+                        const float t2 = fmaf(t1, 256.f, v2[j]), e2 = v2[j] - fmaf(t1, -256.f, t2);
+                        ch[j] = t2;
+                        cl[j] = fmaf(v3[j], 0x1p-8f, fmaf(e1, 256.f, e2));
+                    }
+                }
+                {
+                    const int k = (u0 + 5) & (kSlots - 1);
+                    ok = __all_sync(0xffffffffu,
+                                    !*abort_flag && mbar_wait(&accf[k], (uint32_t)(((u0 + 5) / kSlots) & 1)));
+                    if (!ok) break;
+                    fence_after_sync();
+                    float v4[kCols], v5[kCols];
+                    tmem_ld16_nowait(taddr + (uint32_t)(((u0 + 4) & (kSlots - 1)) * TQ), v4);
+                    tmem_ld16_nowait(taddr + (uint32_t)(k * TQ), v5);
+                    tmem_wait_ld(v4, v5);
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane < 2) mbar_arrive(&acce[(u0 + 4 + lane) & (kSlots - 1)]);
 #pragma unroll
-                for (int cg = 0; cg < 2; ++cg) {
-                    float v[16];
-                    tmem_ld16(taddr + (uint32_t)(L * TQ + cg * 16), v);
+                    for (int j = 0; j < kCols; ++j) cl[j] = fmaf(v5[j], 0x1p-24f, fmaf(v4[j], 0x1p-16f, cl[j]));
+                }
+                // one unit of level 2 is 2^(er + eb - 32): the exponent field alone where the scales of four
+                // neighbouring vectors are normal numbers
+                const int er = EA[(size_t)ci * a.nvA_pad];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int jj = cg * 16 + j;
-                        if (L < 3) {
-                            float s, e;
-                            two_sum(ch[jj], v[j] * sc, s, e);
-                            ch[jj] = s;
-                            cl[jj] += e;
-                        } else {
-                            cl[jj] = fmaf(v[j], sc, cl[jj]);
+                for (int j0 = 0; j0 < kCols; j0 += 4 * rpcB) {
+                    const int4 t = EB[(size_t)ci * (a.nvB_pad / 4) + j0 / (4 * rpcB)];
+                    const int e[4] = {er + t.x, er + t.y, er + t.z, er + t.w};
+                    const int lo4 = min(min(e[0], e[1]), min(e[2], e[3]));
+                    const int hi4 = max(max(e[0], e[1]), max(e[2], e[3]));
+                    if (lo4 > 32 - 127 && hi4 < 32 + 128) {
+#pragma unroll
+                        for (int k = 0; k < 4 * rpcB; ++k) {
+                            const float S = __int_as_float((e[k / rpcB] + (127 - 32)) << 23);
+                            df_add(ah[j0 + k], al[j0 + k], ch[j0 + k] * S, cl[j0 + k] * S);
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 4 * rpcB; ++k) {   // 2^e as a product of two normal numbers
+                            const int ek = min(max(e[k / rpcB] - 32, -252), 254), e1 = ek >> 1;
+                            const float S1 = __int_as_float((e1 + 127) << 23), S2 = __int_as_float((ek - e1 + 127) << 23);
+                            df_add(ah[j0 + k], al[j0 + k], ch[j0 + k] * S1 * S2, cl[j0 + k] * S1 * S2);
                         }
                     }
                 }
-                // level L of this chunk is in registers: its accumulator may take the next chunk
-                fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&acce[L]);
             }
+            if (!ok) break;
+            // The two forms of the output are separate loops: an FP64 instruction that is predicated off
+            // costs its 64 cycles all the same.
+            if (OUT == 0) {
+                double *P = a.P + (size_t)w.z * a.pstride + (size_t)(w.qt * TQ + h * kCols) * a.ldp + rr;
+                if (a.accumulate) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int qq = qt * TQ + h * 32 + j;
-                const float S = pow2f(er + a.EB[(size_t)c * a.nvB_pad + qq / rpcB]);
-                df_add(ah[j], al[j], ch[j] * S, cl[j] * S);
+                    for (int j = 0; j < kCols; ++j) P[(size_t)j * a.ldp] += pair_to_double(ah[j], al[j]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j) P[(size_t)j * a.ldp] = pair_to_double(ah[j], al[j]);
+                }
+            } else if ((rr >> 1) < a.M) {
+                const size_t at = 2 * (size_t)(a.row0 + (rr >> 1)) + (rr & 1);   // of the column, in reals
+                const int jc = w.qt * TQ + h * kCols;
+                double *Dd = reinterpret_cast<double *>(a.D) + at;
+                if (a.scaled) {
+                    const double *Cd = reinterpret_cast<const double *>(a.C) + at;
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j) {
+                        if (jc + j >= a.n) break;
+                        double val = a.alpha * pair_to_double(ah[j], al[j]);
+                        if (a.beta != 0.0) val += a.beta * Cd[2 * (size_t)(jc + j) * a.ldc];
+                        Dd[2 * (size_t)(jc + j) * a.ldd] = val;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j) {
+                        if (jc + j >= a.n) break;
+                        Dd[2 * (size_t)(jc + j) * a.ldd] = pair_to_double(ah[j], al[j]);
+                    }
+                }
             }
         }
         if (!ok) {
             *abort_flag = 1;
             atomicExch(&g_oz_err, 1);
-        } else if (OUT == 0) {
-            double *P = a.P + (size_t)z * a.pstride;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int qq = qt * TQ + h * 32 + j;
-                const double val = (double)ah[j] + (double)al[j];
-                double *dst = P + (size_t)qq * a.ldp + rr;
-                *dst = a.accumulate ? *dst + val : val;
-            }
-        } else {
-            const int i = rr >> 1, part = rr & 1;
-            const int gi = a.row0 + i;
-            if (i < a.M) {
-                double *Dd = reinterpret_cast<double *>(a.D);
-                const double *Cd = reinterpret_cast<const double *>(a.C);
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int jj = qt * TQ + h * 32 + j;
-                    if (jj < a.n) {
-                        double val = a.alpha * ((double)ah[j] + (double)al[j]);
-                        if (a.beta != 0.0) val += a.beta * Cd[2 * ((size_t)jj * a.ldc + gi) + part];
-                        Dd[2 * ((size_t)jj * a.ldd + gi) + part] = val;
-                    }
-                }
-            }
         }
     }
     fence_before_sync();
@@ -530,6 +659,24 @@ int split(const z64 *X, long long rs, long long ks, int nvec, int K, int k0, int
     return check_launch("FP64-class tensor-core GEMM: operand digits");
 }
 
+// Chunks per K split of `tiles` output tiles over `chunks` chunks: every SM takes whole items (a tile
+// and a split), so the makespan is the items of the busiest SM times a split's chunks plus about one
+// chunk's time for an item's output; the shortest wins, of two alike the fewer splits.
+int pick_cps(long long tiles, int chunks) {
+    int best_cps = chunks;
+    double best = 1e300;
+    for (int ns = 1; ns <= 128 && ns <= chunks; ++ns) {
+        const int cps = (chunks + ns - 1) / ns;
+        const long long items = tiles * ((chunks + cps - 1) / cps);
+        const double t = (double)((items + num_sms() - 1) / num_sms()) * (cps + 1.0) + 0.05 * ns;
+        if (t < best) {
+            best = t;
+            best_cps = cps;
+        }
+    }
+    return std::max(1, best_cps);
+}
+
 // Scratch budget of the digit tiles of one slab (bytes).
 constexpr size_t kSlabBytes = (size_t)768 << 20;
 
@@ -553,8 +700,7 @@ int oz_gemm_cn(GemmWork &w, int m, int n, int K, double alpha, const z64 *A, int
     for (int rt = 0; rt < tm; ++rt)
         for (int qt = 0; qt < tq; ++qt)
             if (!lower || 32 * qt <= TM * rt + TM - 1) ++tiles;
-    const int want = std::max(1, (int)((2LL * num_sms() + tiles - 1) / tiles));
-    int cps = std::max(1, (slab + want - 1) / want);
+    const int cps = pick_cps(tiles, slab);
     const int nsplit = (slab + cps - 1) / cps;
     LG_TRY(w.alloc->ensure(w.oz_a, per_chunk * slab));
     LG_TRY(w.alloc->ensure(w.oz_e, sizeof(int) * (size_t)slab * (nvA + nvB)));
@@ -583,7 +729,10 @@ int oz_gemm_cn(GemmWork &w, int m, int n, int K, double alpha, const z64 *A, int
         a.ldp = mA;
         a.pstride = (size_t)qB * mA;
         a.accumulate = first ? 0 : 1;
-        k_oz_mma<0><<<dim3(tq, tm, nsplit), kThreads, kSmem, s>>>(a);
+        a.tq = tq;
+        a.tiles = (int)tiles;
+        a.nsplit = nsplit;
+        k_oz_mma<0><<<(int)std::min<long long>(num_sms(), tiles * nsplit), kThreads, kSmem, s>>>(a);
         LG_TRY(check_launch("FP64-class tensor-core GEMM A^H B"));
     }
     const size_t tot = (size_t)m * n;
@@ -631,12 +780,16 @@ int oz_gemm_nn(GemmWork &w, int M, int n, int k, double alpha, const z64 *A, int
         a.row0 = r0;
         a.alpha = alpha;
         a.beta = beta;
+        a.scaled = alpha != 1.0 || beta != 0.0;
         a.C = beta != 0.0 ? C : D;
         a.ldc = beta != 0.0 ? ldc : ldd;
         a.D = D;
         a.ldd = ldd;
         const int tm = (2 * mr + TM - 1) / TM;
-        k_oz_mma<1><<<dim3(qB / TQ, tm, 1), kThreads, kSmem, s>>>(a);
+        a.tq = qB / TQ;
+        a.tiles = a.tq * tm;
+        a.nsplit = 1;
+        k_oz_mma<1><<<std::min(num_sms(), a.tiles), kThreads, kSmem, s>>>(a);
         LG_TRY(check_launch("FP64-class tensor-core GEMM A B"));
     }
     return LOBPCG_OK;

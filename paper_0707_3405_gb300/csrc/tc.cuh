@@ -104,6 +104,55 @@ __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
                  : "memory");
 }
 
+// ---- issue by a whole warp
+// The operands of tcgen05.mma are uniform registers.  Code that runs in one thread of a diverged
+// warp keeps its descriptors in vector registers and moves six of them per MMA into uniform ones,
+// which takes 90 cycles and more, whatever the MMA's size (N = 16 to 128 measured alike).  So the
+// MMA warp runs its loop undivided, with warp-uniform values throughout, and only the instruction
+// itself is predicated on one elected lane: 48 cycles for M = 128, N = 64, K = 16 from shared
+// memory (its 6 KB of operands at 128 bytes a cycle), 64 for N = 128 (the tensor rate).
+
+// 1 on one lane of a converged warp, 0 on the others.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+    return p;
+}
+// A value equal on all lanes, as one the compiler knows to be uniform.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+// Reuse of the left operand by the next MMAs: its rows stay in the tensor core's collector from
+// the fill to the last use, which leaves the right operand's 2 KB (N = 64) to read per MMA.
+enum Collector { kDiscard = 0, kFill = 1, kUse = 2, kLastUse = 3 };
+
+// Operand addresses as the low words of two descriptors with the high word HI, plus constant offsets
+// AO, BO (bytes): one 32-bit addition each, where 64-bit descriptors are kept in registers instead.
+template <int COL, uint32_t HI, int AO, int BO>
+__device__ __forceinline__ void mma_bf16_warp(uint32_t elected, uint32_t d_tmem, uint32_t alo, uint32_t blo,
+                                              uint32_t idesc, uint32_t accumulate) {
+#define LG_MMA_WARP(qual)                                                                                          \
+    asm volatile(                                                                                                  \
+        "{\n\t.reg .pred p, q;\n\t.reg .b32 a, b;\n\t.reg .b64 da, db;\n\t"                                         \
+        "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"                                                       \
+        "add.u32 a, %1, %7;\n\tadd.u32 b, %2, %8;\n\tmov.b64 da, {a, %6};\n\tmov.b64 db, {b, %6};\n\t"             \
+        "@q tcgen05.mma.cta_group::1.kind::f16" qual " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                   \
+        "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(elected), "n"(HI), "n"(AO >> 4), "n"(BO >> 4)         \
+        : "memory")
+    if constexpr (COL == kFill) LG_MMA_WARP(".collector::a::fill");
+    else if constexpr (COL == kUse) LG_MMA_WARP(".collector::a::use");
+    else if constexpr (COL == kLastUse) LG_MMA_WARP(".collector::a::lastuse");
+    else LG_MMA_WARP("");
+#undef LG_MMA_WARP
+}
+
+__device__ __forceinline__ void mma_commit_warp(uint32_t elected, uint64_t *mbar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(mbar)),
+        "r"(elected)
+        : "memory");
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -139,6 +188,29 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// The same load without the wait; the registers hold the values after tmem_wait_ld on them.
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+          "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+// Ties the values to the wait, so that no use of them moves before it.
+__device__ __forceinline__ void tmem_touch(float (&v)[16]) {
+    asm volatile(""
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                   "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
+                 :
+                 : "memory");
+}
+template <typename... V>
+__device__ __forceinline__ void tmem_wait_ld(V &...v) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    (tmem_touch(v), ...);
 }
 
 }  // namespace tc
