@@ -147,14 +147,14 @@ int lobpcg_k_heev(int n, const void *A, double *w, void *V, void *stream);
 int lobpcg_k_set_gemm_mode(int mode);
 
 /*
- * Poll limit of the waits inside the tensor-core GEMMs on the current device:
- * before a CTA refills a shared-memory stage it waits, at most `polls` times,
- * for the MMAs that read it.  polls < 0 restores the default (2^26 polls,
- * seconds).  A wait that runs out makes the CTA stop issuing, wait (with the
- * default limit) for the MMAs it already issued, free its tensor memory and
- * return with a device flag set, which lobpcg_k_check_timeouts and every
- * solve sweep turn into LOBPCG_ERR_TIMEOUT.  This exists so that tests can
- * drive the timeout path (polls = 0) without hanging or faulting the GPU.
+ * Poll limit of the waits inside the complex64 tensor-core GEMMs on the current
+ * device: before a warp refills a shared-memory stage it waits, at most `polls`
+ * times, for the MMAs that read it.  polls < 0 restores the default (2^26 polls,
+ * seconds).  A wait that runs out sets a device flag, which
+ * lobpcg_k_check_timeouts and every solve sweep turn into LOBPCG_ERR_TIMEOUT,
+ * and is repeated once with the default limit, so that the kernel still ends
+ * with its work drained and its tensor memory freed.  This exists so that tests
+ * can drive the timeout path (polls = 0) without hanging or faulting the GPU.
  * Errors: ERR_CUDA.
  */
 int lobpcg_k_set_spin_limit(long long polls);

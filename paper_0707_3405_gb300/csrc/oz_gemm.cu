@@ -106,25 +106,9 @@ __device__ __forceinline__ uint32_t swz64(int r, int c) {
     return (uint32_t)r * 64u + ((((uint32_t)c >> 3) ^ (((uint32_t)r >> 1) & 3u)) << 4) + (((uint32_t)c & 7u) << 1);
 }
 
-// Shared-memory matrix descriptor for a 64-byte-swizzled K-major tile: stride between
-// 8-row groups 512 bytes, descriptor version 1, swizzle mode 4 (64 bytes).
-__host__ __device__ constexpr uint64_t make_desc_sw64(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1u << 16;
-    d |= (uint64_t)(512u >> 4) << 32;
-    d |= (uint64_t)1u << 46;
-    d |= (uint64_t)4u << 61;
-    return d;
-}
-
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {

@@ -1,9 +1,8 @@
 // tcgen05 / TMEM building blocks for sm_103a (inline PTX).
 //
-// Shared-memory operand layout: K-major, 128-byte swizzle.  A tile of R rows x
-// 64 bf16 (128 bytes of K per row) is stored row after row; rows are grouped
-// by 8 into 1024-byte atoms (tile base 1024-byte aligned) and inside an atom
-// the 16-byte chunk c of row r sits at chunk position c ^ (r % 8).
+// Shared-memory operand layout: K-major, 64-byte swizzle.  A tile of R rows x 64 bytes of K is
+// stored row after row; rows are grouped by 8 into 512-byte atoms (tile base 512-byte aligned),
+// and the 16-byte chunk c of row r sits at chunk position c ^ ((r / 2) % 4).
 //
 // Every wait in here is bounded: a wait that runs out sets *err and returns.
 #pragma once
@@ -15,27 +14,20 @@ namespace lg {
 namespace tc {
 
 constexpr long long kSpinLimit = 1LL << 26;   // ~ seconds of polling at most
-constexpr int kTileRowsK = 64;                 // bf16 elements of K per smem row (128 bytes)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Byte offset of element (r, k) (k < 64) of a swizzled K-major tile.
-__device__ __forceinline__ uint32_t swz_offset(int r, int k) {
-    const uint32_t chunk = (uint32_t)(k >> 3);            // 8 bf16 = 16 bytes
-    return (uint32_t)r * 128u + (((chunk ^ (uint32_t)(r & 7)) << 4) | (uint32_t)((k & 7) << 1));
-}
-
-// Shared-memory matrix descriptor (tcgen05): start address, leading / stride byte
-// offsets (in 16-byte units), descriptor version 1, 128-byte swizzle.
-__device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr) {
+// Shared-memory matrix descriptor for a 64-byte-swizzled K-major tile: stride between
+// 8-row groups 512 bytes, descriptor version 1, swizzle mode 4 (64 bytes).
+__host__ __device__ constexpr uint64_t make_desc_sw64(uint32_t saddr) {
     uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);          // bits 0-13   start address
-    d |= (uint64_t)(1u) << 16;                        // bits 16-29  leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024u >> 4) << 32;                // bits 32-45  stride byte offset: 8 rows x 128 B
-    d |= (uint64_t)1u << 46;                          // bits 46-47  descriptor version
-    d |= (uint64_t)2u << 61;                          // bits 61-63  swizzle: 128 B
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)1u << 16;
+    d |= (uint64_t)(512u >> 4) << 32;
+    d |= (uint64_t)1u << 46;
+    d |= (uint64_t)4u << 61;
     return d;
 }
 
@@ -79,31 +71,6 @@ __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fenc
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t *mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar))
-                 : "memory");
-}
-
 // ---- issue by a whole warp
 // The operands of tcgen05.mma are uniform registers.  Code that runs in one thread of a diverged
 // warp keeps its descriptors in vector registers and moves six of them per MMA into uniform ones,
@@ -127,23 +94,31 @@ enum Collector { kDiscard = 0, kFill = 1, kUse = 2, kLastUse = 3 };
 
 // Operand addresses as the low words of two descriptors with the high word HI, plus constant offsets
 // AO, BO (bytes): one 32-bit addition each, where 64-bit descriptors are kept in registers instead.
-template <int COL, uint32_t HI, int AO, int BO>
-__device__ __forceinline__ void mma_bf16_warp(uint32_t elected, uint32_t d_tmem, uint32_t alo, uint32_t blo,
-                                              uint32_t idesc, uint32_t accumulate) {
-#define LG_MMA_WARP(qual)                                                                                          \
+#define LG_MMA_WARP(kind, qual)                                                                                    \
     asm volatile(                                                                                                  \
         "{\n\t.reg .pred p, q;\n\t.reg .b32 a, b;\n\t.reg .b64 da, db;\n\t"                                         \
         "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"                                                       \
         "add.u32 a, %1, %7;\n\tadd.u32 b, %2, %8;\n\tmov.b64 da, {a, %6};\n\tmov.b64 db, {b, %6};\n\t"             \
-        "@q tcgen05.mma.cta_group::1.kind::f16" qual " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                   \
+        "@q tcgen05.mma.cta_group::1.kind::" kind qual " [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),                 \
         "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "r"(elected), "n"(HI), "n"(AO >> 4), "n"(BO >> 4)         \
         : "memory")
-    if constexpr (COL == kFill) LG_MMA_WARP(".collector::a::fill");
-    else if constexpr (COL == kUse) LG_MMA_WARP(".collector::a::use");
-    else if constexpr (COL == kLastUse) LG_MMA_WARP(".collector::a::lastuse");
-    else LG_MMA_WARP("");
-#undef LG_MMA_WARP
+template <int COL, uint32_t HI, int AO, int BO>
+__device__ __forceinline__ void mma_bf16_warp(uint32_t elected, uint32_t d_tmem, uint32_t alo, uint32_t blo,
+                                              uint32_t idesc, uint32_t accumulate) {
+    if constexpr (COL == kFill) LG_MMA_WARP("f16", ".collector::a::fill");
+    else if constexpr (COL == kUse) LG_MMA_WARP("f16", ".collector::a::use");
+    else if constexpr (COL == kLastUse) LG_MMA_WARP("f16", ".collector::a::lastuse");
+    else LG_MMA_WARP("f16", "");
 }
+template <int COL, uint32_t HI, int AO, int BO>
+__device__ __forceinline__ void mma_tf32_warp(uint32_t elected, uint32_t d_tmem, uint32_t alo, uint32_t blo,
+                                              uint32_t idesc, uint32_t accumulate) {
+    if constexpr (COL == kFill) LG_MMA_WARP("tf32", ".collector::a::fill");
+    else if constexpr (COL == kUse) LG_MMA_WARP("tf32", ".collector::a::use");
+    else if constexpr (COL == kLastUse) LG_MMA_WARP("tf32", ".collector::a::lastuse");
+    else LG_MMA_WARP("tf32", "");
+}
+#undef LG_MMA_WARP
 
 __device__ __forceinline__ void mma_commit_warp(uint32_t elected, uint64_t *mbar) {
     asm volatile(
@@ -156,6 +131,10 @@ __device__ __forceinline__ void mma_commit_warp(uint32_t elected, uint64_t *mbar
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // Wait for phase `parity` of the mbarrier to complete; at most `limit` polls.  Returns false
@@ -176,21 +155,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, long 
     return false;
 }
 
-// 32 lanes x 16 consecutive 32-bit columns of TMEM into registers (one warp).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// The same load without the wait; the registers hold the values after tmem_wait_ld on them.
+// 32 lanes x 16 consecutive 32-bit columns of TMEM into registers (one warp), which hold the values
+// after tmem_wait_ld on them.
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"

@@ -8,28 +8,38 @@
 // (the lo*lo term is below FP32 resolution), accumulated in FP32 by the tensor
 // core.  The relative error per product is about 2^-21, i.e. FP32 class.
 //
-// Complex arithmetic as one real GEMM per tile (interleaved re/im along K):
-//   C = A^H B:  Re C = A'.B', Im C = A'.B'' where A' is a column of A read as
-//               [re, im, re, im, ...], B' likewise and B'' = [im, -re, ...].
-//               The MMA runs with N = 2 NT: B' rows and B'' rows side by side.
-//   D = A B:    D read as a real (2M x n) matrix equals Ahat Bhat with
-//               Ahat rows 2g = [re, -im, ...], 2g+1 = [im, re, ...] (along K
-//               pairs) and Bhat = B read as real; the producer expands A.
+// Complex arithmetic as one real GEMM per tile, re / im interleaved along K.  The left factor's
+// vectors (columns of A, or rows of A) are the 128 MMA rows [re, im, re, im, ...]; each of the NT
+// columns of the right factor is two MMA columns, j (the real part) and NT + j (the imaginary one):
+//   C = A^H B:  [re, im, ...] and [im, -re, ...] of B's column;
+//   D = A B:    [re, -im, ...] and [im, re, ...] of B's column.
 //
-// Data path per CTA (256 threads, one tile): the threads load FP32 from HBM
-// (coalesced) one stage ahead into registers, split, and store hi / lo into
-// 128-byte-swizzled K-major shared tiles (the layout tcgen05 descriptors
-// address); thread 0 issues the MMAs of a stage and commits them to that
-// stage's mbarrier; the stage is refilled once the barrier shows the MMAs
-// done (2-3 stage ring).  The accumulator tile is read back from TMEM by the
-// eight warps (warp w reads lane quarter w % 4, column half w / 4).
-// Long reductions (A^H B over the plane-wave count) are split over grid.z;
-// FP64 partial tiles are summed afterwards in a fixed order (reproducible).
+// One persistent CTA per SM takes every gridDim-th item (an output tile, and for A^H B a part of
+// the reduction, which is split over the GPU).  Eight warps load FP32 from HBM two stages ahead
+// into registers, split it and store hi / lo into 64-byte-swizzled K-major shared tiles of a
+// 4-stage ring (8 complex K a stage); one warp issues a stage's six MMAs of M = 128, N = 2 NT and
+// commits them to the stage's mbarrier; four warps read the accumulator of the finished item from
+// TMEM, which holds two, and write it out while the next item runs.  FP32 partial tiles of a split
+// reduction are summed afterwards in a fixed order (reproducible).
 //
-// Every mbarrier wait is bounded; a wait that runs out raises a device flag
-// (read by tc_check_error) and the CTA stops issuing work, waits (bounded) for
-// the MMAs it has in flight, frees its TMEM and returns.
+// What bounds it (NT = 128): a stage's MMAs take 768 cycles of the tensor pipe and, with the left
+// rows kept in the collector, 64 KB of shared-memory reads beside the loaders' 48 KB of stores, 896
+// cycles of shared-memory bandwidth.  Measured on a GB300 (tensor rate: 3 x 8 m n K flops), before
+// (256 threads loading, splitting and storing in lockstep, one of them issuing) and after:
+//   A B    113081 x 128 x 256    330 -> 131 us  (269 -> 680 TFLOP/s of about 960 for TF32)
+//          113081 x 128 x 1024  1070 -> 420 us;  57925 x 64 x 128  50 -> 33 us
+//   A^H B  432 x 128 x 113081    333 -> 259 us;  384 x 256 x 113081  468 -> 375 us
+//          64 x 64 x 57925        65 -> 40 us
+// All loaders filling one stage together (8 or 16 warps, 2 to 4 stages ahead in registers) took 179 to
+// 197 us for the first: each stage then costs one group's whole chain of wait, stores, fence and
+// signal, which the slot groups overlap.
+//
+// Every mbarrier wait is bounded.  A loader's wait that runs out raises a device flag (read by
+// tc_check_error), is repeated with the full limit, and the CTA carries on, so that it always ends
+// with its copies and MMAs done and its TMEM freed; the MMA warp's and the readers' waits raise the
+// flag and go on without what they waited for.
 #include "common.cuh"
+#include "df64.cuh"
 #include "tc.cuh"
 
 #include <algorithm>
@@ -40,297 +50,302 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 256;  // 8 warps: all load / split / store; thread 0 issues the MMAs
-constexpr int KBC = 16;     // complex K per stage: 32 floats = one 128-byte shared row
-constexpr int ROWB = 128;   // bytes per shared row
+constexpr int kLoaders = 16, kReaders = 4;                   // warps
+constexpr int kThreads = 32 * (kLoaders + 1 + kReaders);     // + the MMA warp
+constexpr int KST = 8;       // complex K per stage: 16 floats = one 64-byte shared row
+constexpr int ROWB = 64;     // bytes per shared row
+constexpr int kRing = 4;
+constexpr int kRows = 128;   // vectors of the left factor per tile (MMA M)
+constexpr long long kPipeSpin = 1 << 18;   // polls of one wait of the MMA and reader warps (milliseconds)
 
 __device__ int g_tc_err = 0;
-// Poll limit of the ring waits (a stage's MMAs done before its refill); the drain wait for the
-// MMAs a CTA has issued always takes the full kSpinLimit, so a CTA that gave up never frees
-// TMEM or returns while its own MMAs may still run.  Lowered only by tests of the timeout path.
+// Poll limit of the loaders' first wait for a stage (lowered only by tests of the timeout path).
 __device__ long long g_tc_spin = kSpinLimit;
-
-// Byte offset of complex element kc (0..15) of row r in a 128-byte-swizzled K-major tile.
-__device__ __forceinline__ uint32_t swz(int r, int kc) {
-    return (uint32_t)r * 128u + ((((uint32_t)kc >> 1) ^ ((uint32_t)r & 7u)) << 4) + (((uint32_t)kc & 1u) << 3);
-}
-
-__device__ __forceinline__ void put_split(unsigned char *hi, unsigned char *lo, uint32_t off, float a, float b) {
-    const float ah = to_tf32(a), bh = to_tf32(b);
-    *reinterpret_cast<float2 *>(hi + off) = make_float2(ah, bh);
-    *reinterpret_cast<float2 *>(lo + off) = make_float2(to_tf32(a - ah), to_tf32(b - bh));
-}
 
 __device__ __forceinline__ unsigned char *align1k(unsigned char *p) {
     return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
 }
 
-// Ring depth: NSF if given, else 3 stages when they fit in 200 KB, else 2.
-template <int STAGE, int NSF = 0>
-constexpr int n_stages() { return NSF ? NSF : (3 * STAGE <= 200 * 1024 ? 3 : 2); }
+constexpr int stage_bytes(int NT) { return 2 * kRows * ROWB + 2 * 2 * NT * ROWB; }
+constexpr size_t smem_bytes(int NT) { return (size_t)kRing * stage_bytes(NT) + 1024 + 256; }
 
-template <int STAGE, int NSF = 0>
-constexpr size_t smem_bytes() { return (size_t)n_stages<STAGE, NSF>() * STAGE + 1024 + 64; }
-
-// A B with 64 columns: a 2-stage ring (97 KB) lets two CTAs share an SM; the products of the
-// block iterations are tall and short (K = 64 .. 192), so a deeper ring never fills anyway.
-template <int NN>
-constexpr int nn_ring() { return NN == 64 ? 2 : 0; }
-template <int NN>
-constexpr int nn_ctas_per_sm() { return NN == 64 ? 2 : 1; }
-
-// Issue the 3xTF32 MMAs of one stage (4 K-steps of 8) and commit them to `bar`.
-__device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t a_h, uint32_t a_l, uint32_t b_h, uint32_t b_l,
-                                            uint32_t idesc, bool first, uint64_t *bar) {
-    fence_after_sync();
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t o = 32u * kk;
-        mma_tf32(tmem, make_desc_sw128(a_h + o), make_desc_sw128(b_h + o), idesc, (first && kk == 0) ? 0u : 1u);
-        mma_tf32(tmem, make_desc_sw128(a_h + o), make_desc_sw128(b_l + o), idesc, 1u);
-        mma_tf32(tmem, make_desc_sw128(a_l + o), make_desc_sw128(b_h + o), idesc, 1u);
-    }
-    mma_commit(bar);
+// Byte offset of complex element k (0 .. 7) of row r in a 64-byte-swizzled tile.
+__device__ __forceinline__ uint32_t elem_at(int r, int k) {
+    return (uint32_t)r * (uint32_t)ROWB + ((uint32_t)((k >> 1) ^ ((r >> 1) & 3)) << 4) + (uint32_t)((k & 1) << 3);
 }
 
-// ------------------------------------------------------------------ C = A^H B
-// CTA tile: 128 columns of A (rows i of C) x NT columns of B; K range
-// [blockIdx.z * kchunk, +kchunk).  Writes the FP64 partial tile of its split.
+// hi and lo parts of a complex number to the same place of a hi and a lo tile.
+__device__ __forceinline__ void put2(unsigned char *hi, unsigned char *lo, uint32_t off, float x, float y) {
+    const float2 h = make_float2(to_tf32(x), to_tf32(y));
+    *reinterpret_cast<float2 *>(hi + off) = h;
+    *reinterpret_cast<float2 *>(lo + off) = make_float2(to_tf32(x - h.x), to_tf32(y - h.y));
+}
+
+// hi and lo parts of four floats to the same place of a hi and a lo tile.
+__device__ __forceinline__ void put4(unsigned char *hi, unsigned char *lo, uint32_t off, float4 v) {
+    const float4 h = make_float4(to_tf32(v.x), to_tf32(v.y), to_tf32(v.z), to_tf32(v.w));
+    *reinterpret_cast<float4 *>(hi + off) = h;
+    *reinterpret_cast<float4 *>(lo + off) =
+        make_float4(to_tf32(v.x - h.x), to_tf32(v.y - h.y), to_tf32(v.z - h.z), to_tf32(v.w - h.w));
+}
+
+struct TcArgs {
+    int m, n, K;                 // left vectors, right columns, reduction
+    const c32 *A, *B;
+    int lda, ldb;
+    int tm, tn, nsplit, kchunk;  // tiles, splits of the reduction and their length (a multiple of KST)
+    float alpha, beta;           // A B
+    const c32 *C;
+    c32 *D;
+    int ldc, ldd;
+    c32 *part;                   // A^H B: FP32 partial tiles [split][j][i]
+};
+
+struct TcItem {
+    int i0, j0, z, kbeg, kend, nst;   // first left vector and right column, split, reduction range, stages
+};
 template <int NT>
-__global__ void __launch_bounds__(kThreads, 1)
-k_tc_cn(int m, int n, int K, int kchunk, const c32 *__restrict__ A, int lda, const c32 *__restrict__ B, int ldb,
-        z64 *__restrict__ part) {
-    constexpr int NR = 2 * NT;  // B' rows then B'' rows
-    constexpr int A_BYTES = 128 * ROWB, B_BYTES = NR * ROWB;
-    constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
-    constexpr int NS = n_stages<STAGE>();
-    constexpr uint32_t IDESC = make_idesc_tf32(128, NR);
+__device__ __forceinline__ TcItem tc_item(const TcArgs &a, int it) {
+    TcItem w;
+    const int tiles = a.tm * a.tn;
+    w.z = it / tiles;
+    const int t = it - w.z * tiles, ti = t / a.tn;
+    w.i0 = ti * kRows;
+    w.j0 = (t - ti * a.tn) * NT;
+    w.kbeg = w.z * a.kchunk;
+    w.kend = min(a.K, w.kbeg + a.kchunk);
+    w.nst = (w.kend - w.kbeg + KST - 1) / KST;
+    return w;
+}
+
+// CN: C = A^H B (partial tiles), else D = alpha A B + beta C.
+template <bool CN, int NT>
+__device__ __forceinline__ void tc_body(const TcArgs &a) {
+    constexpr int A_BYTES = kRows * ROWB, B_BYTES = 2 * NT * ROWB, STAGE = stage_bytes(NT);
+    constexpr int ACC = 2 * NT, TCOLS = 2 * ACC;           // TMEM columns of an accumulator, of both
     extern __shared__ unsigned char smraw[];
     unsigned char *base = align1k(smraw);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(base + NS * STAGE);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + NS);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int i0 = blockIdx.x * 128, j0 = blockIdx.y * NT;
-    const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
-    const int nkb = kend > kbeg ? (kend - kbeg + KBC - 1) / KBC : 0;
-    if (warp == 0) tmem_alloc(tslot, NR);
-    if (tid == 0)
-        for (int s = 0; s < NS; ++s) mbar_init(&bar[s], 1);
+    uint64_t *full = reinterpret_cast<uint64_t *>(base + kRing * STAGE);
+    uint64_t *empty = full + kRing, *accf = empty + kRing, *acce = accf + 2;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + 2);
+    const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
+    if (warp == kLoaders) tmem_alloc(tslot, TCOLS);
+    if (tid == 0) {
+        for (int s = 0; s < kRing; ++s) {
+            mbar_init(&full[s], kLoaders / kRing);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&accf[b], 1);
+            mbar_init(&acce[b], kReaders);
+        }
+    }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    const uint32_t tmem = *tslot;
-    // Each thread owns NA elements of the A tile and NB of the B tile per stage; the loads of
-    // stage kb + 1 are issued before stage kb is split and stored, so they overlap the MMAs.
-    constexpr int NA = 128 * KBC / kThreads, NB = NT * KBC / kThreads;
-    float2 ra[NA], rb[NB];
-    auto load = [&](int kb) {
-        const int k0 = kbeg + kb * KBC;
+    const uint32_t tmem = uniform(*tslot);
+    const int nit = a.tm * a.tn * a.nsplit, it0 = blockIdx.x, step = gridDim.x;
+    if (warp < kLoaders) {
+        // ---- loaders: group w / 4 fills ring slot w / 4, that is every kRing-th stage, so that one
+        // group's wait, stores and proxy fence overlap the others'.  Operands that are contiguous along
+        // K: eight threads take a vector's eight numbers (64 bytes), or, for the right factor of A B,
+        // which is small and stays in L2, four threads take two numbers each (fewer, 16-byte stores).
+        // The left factor of A B is contiguous along its vectors: a warp takes 256 bytes of two columns,
+        // a thread one vector's two consecutive K.
+        constexpr int TH = 32 * kLoaders / kRing, EA = kRows * KST / TH, EB = NT * KST / TH;
+        static_assert(EA * TH == kRows * KST && EB * TH == NT * KST, "whole elements per thread");
+        const int t = tid % TH, s = warp / (kLoaders / kRing), tk = t & 7, tv = t >> 3;
+        constexpr int VS = TH / KST;                       // vectors between a thread's elements
+        float2 ra[EA], rb[EB];
+        int li = it0, lk = s;                              // load cursor: item, stage
+        TcItem lw{};
+        auto settle = [&]() {                              // carry the cursor into the next items
+            while (li < nit) {
+                lw = tc_item<NT>(a, li);
+                if (lk < lw.nst) return true;
+                lk -= lw.nst;
+                li += step;
+            }
+            return false;
+        };
+        bool more = settle();
+        const float2 zero = make_float2(0.f, 0.f);
+        auto load = [&]() {
+            const int k0 = lw.kbeg + lk * KST;
 #pragma unroll
-        for (int q = 0; q < NA; ++q) {
-            const int idx = tid + kThreads * q, r = idx >> 4, kc = idx & 15;
-            const int i = i0 + r, k = k0 + kc;
-            ra[q] = (i < m && k < kend) ? __ldg(reinterpret_cast<const float2 *>(A + (size_t)i * lda + k))
-                                        : make_float2(0.f, 0.f);
-        }
+            for (int q = 0; q < EA; ++q) {
+                const int i = lw.i0 + (CN ? tv + VS * q : t % kRows);
+                const int k = k0 + (CN ? tk : 2 * (t / kRows + TH / kRows * (q >> 1)) + (q & 1));
+                const c32 *src = CN ? a.A + (size_t)i * a.lda + k : a.A + (size_t)k * a.lda + i;
+                ra[q] = (i < a.m && k < lw.kend) ? __ldg(reinterpret_cast<const float2 *>(src)) : zero;
+            }
 #pragma unroll
-        for (int q = 0; q < NB; ++q) {
-            const int idx = tid + kThreads * q, j = idx >> 4, kc = idx & 15;
-            const int k = k0 + kc;
-            rb[q] = (j0 + j < n && k < kend) ? __ldg(reinterpret_cast<const float2 *>(B + (size_t)(j0 + j) * ldb + k))
-                                             : make_float2(0.f, 0.f);
-        }
-    };
-    int bad = 0, issued = 0;
-    if (nkb > 0) load(0);
-    for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % NS;
-        if (kb >= NS && !mbar_wait(&bar[s], (uint32_t)((kb / NS - 1) & 1), g_tc_spin)) bad = 1;
+            for (int q = 0; q < EB; ++q) {
+                const int j = lw.j0 + (CN ? tv + VS * q : (t >> 2) + 2 * VS * (q >> 1));
+                const int k = k0 + (CN ? tk : 2 * (t & 3) + (q & 1));
+                rb[q] = (j < a.n && k < lw.kend) ? __ldg(reinterpret_cast<const float2 *>(a.B + (size_t)j * a.ldb + k)) : zero;
+            }
+        };
+        const long long spin = g_tc_spin;
         unsigned char *sAh = base + s * STAGE, *sAl = sAh + A_BYTES, *sBh = sAl + A_BYTES, *sBl = sBh + B_BYTES;
+        if (more) load();
+        for (uint32_t n = 0; more; ++n) {                  // n-th filling of the slot
+            if (n > 0 && !mbar_wait(&empty[s], (n - 1) & 1u, spin)) {
+                atomicExch(&g_tc_err, 1);
+                mbar_wait(&empty[s], (n - 1) & 1u);
+            }
+            if (CN) {
 #pragma unroll
-        for (int q = 0; q < NA; ++q) {
-            const int idx = tid + kThreads * q;
-            put_split(sAh, sAl, swz(idx >> 4, idx & 15), ra[q].x, ra[q].y);
-        }
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-            const int idx = tid + kThreads * q, j = idx >> 4, kc = idx & 15;
-            put_split(sBh, sBl, swz(j, kc), rb[q].x, rb[q].y);
-            put_split(sBh, sBl, swz(NT + j, kc), rb[q].y, -rb[q].x);
-        }
-        if (kb + 1 < nkb) load(kb + 1);
-        fence_proxy_async();
-        if (__syncthreads_or(bad)) break;
-        if (tid == 0)
-            issue_stage(tmem, smem_u32(sAh), smem_u32(sAl), smem_u32(sBh), smem_u32(sBl), IDESC, kb == 0, &bar[s]);
-        ++issued;
-    }
-    if (issued > 0) {
-        const int kl = issued - 1;
-        if (!mbar_wait(&bar[kl % NS], (uint32_t)((kl / NS) & 1))) bad = 1;
-    }
-    fence_after_sync();
-    bad = __syncthreads_or(bad);
-    z64 *P = part + (size_t)blockIdx.z * m * n;
-    const int quarter = warp & 3, half = warp >> 2;
-    const int i = i0 + quarter * 32 + lane;
-    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (!bad) {
-#pragma unroll 1
-        for (int c0 = half * (NT / 2); c0 < (half + 1) * (NT / 2); c0 += 16) {
-            float re[16], im[16];
-            if (issued > 0) {
-                tmem_ld16(trow + (uint32_t)c0, re);
-                tmem_ld16(trow + (uint32_t)(NT + c0), im);
+                for (int q = 0; q < EA; ++q) put2(sAh, sAl, elem_at(tv + VS * q, tk), ra[q].x, ra[q].y);
             } else {
 #pragma unroll
-                for (int jj = 0; jj < 16; ++jj) re[jj] = im[jj] = 0.f;
+                for (int q = 0; q < EA; q += 2)
+                    put4(sAh, sAl, elem_at(t % kRows, 2 * (t / kRows + TH / kRows * (q >> 1))),
+                         make_float4(ra[q].x, ra[q].y, ra[q + 1].x, ra[q + 1].y));
             }
-            if (i < m) {
+            if (CN) {
 #pragma unroll
-                for (int jj = 0; jj < 16; ++jj) {
-                    const int j = j0 + c0 + jj;
-                    if (j < n) P[(size_t)j * m + i] = mkc((double)re[jj], (double)im[jj]);
+                for (int q = 0; q < EB; ++q) {
+                    const float x = rb[q].x, y = rb[q].y;
+                    put2(sBh, sBl, elem_at(tv + VS * q, tk), x, y);
+                    put2(sBh, sBl, elem_at(NT + tv + VS * q, tk), y, -x);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < EB; q += 2) {
+                    const int j = (t >> 2) + 2 * VS * (q >> 1), k = 2 * (t & 3);
+                    const float2 x = rb[q], y = rb[q + 1];
+                    put4(sBh, sBl, elem_at(j, k), make_float4(x.x, -x.y, y.x, -y.y));
+                    put4(sBh, sBl, elem_at(NT + j, k), make_float4(x.y, x.x, y.y, y.x));
                 }
             }
+            lk += kRing;
+            more = settle();
+            if (more) load();                              // in flight during the fence and the next wait
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[s]);
         }
-    } else if (tid == 0) {
-        atomicExch(&g_tc_err, 1);
+    } else if (warp == kLoaders) {
+        // ---- MMA issuer: the whole warp, one elected lane issuing; nothing in the loop depends on how a
+        // wait ended (see tc.cuh)
+        const uint32_t el = elect_one();
+        constexpr uint32_t HI = (uint32_t)(make_desc_sw64(0) >> 32), IDESC = make_idesc_tf32(kRows, ACC);
+        const uint32_t d0 = (uint32_t)make_desc_sw64(uniform(smem_u32(base)));
+        bool late = false;
+        int s = 0, g = 0;
+        uint32_t ph = 0;
+        int q = 0;                                         // items so far
+        for (int it = it0; it < nit; it += step, ++q) {
+            const int z = it / (a.tm * a.tn), kbeg = z * a.kchunk;
+            const int nst = (min(a.K, kbeg + a.kchunk) - kbeg + KST - 1) / KST;
+            const int b = q & 1;
+            const uint32_t dt = tmem + (uint32_t)(b * ACC);
+            if (q >= 2) late |= !mbar_wait(&acce[b], (uint32_t)((q / 2 - 1) & 1), kPipeSpin);
+            for (int t = 0; t < nst; ++t, ++g) {
+                late |= !mbar_wait(&full[s], ph, kPipeSpin);
+                __syncwarp();
+                fence_after_sync();
+                const uint32_t ah = d0 + ((uint32_t)(s * STAGE) >> 4), bh = ah + ((2 * A_BYTES) >> 4);
+                const uint32_t first = t == 0 ? 0u : 1u;
+                mma_tf32_warp<kFill, HI, 0, 0>(el, dt, ah, bh, IDESC, first);
+                mma_tf32_warp<kLastUse, HI, 0, B_BYTES>(el, dt, ah, bh, IDESC, 1u);
+                mma_tf32_warp<kDiscard, HI, A_BYTES, 0>(el, dt, ah, bh, IDESC, 1u);
+                mma_tf32_warp<kFill, HI, 32, 32>(el, dt, ah, bh, IDESC, 1u);
+                mma_tf32_warp<kLastUse, HI, 32, B_BYTES + 32>(el, dt, ah, bh, IDESC, 1u);
+                mma_tf32_warp<kDiscard, HI, A_BYTES + 32, 32>(el, dt, ah, bh, IDESC, 1u);
+                mma_commit_warp(el, &empty[s]);
+                if (++s == kRing) { s = 0; ph ^= 1; }
+            }
+            mma_commit_warp(el, &accf[b]);
+        }
+        if (late && el) atomicExch(&g_tc_err, 1);
+        // every MMA is done before the CTA frees its TMEM
+        if (g > 0) mbar_wait(&empty[(g - 1) % kRing], (uint32_t)(((g - 1) / kRing) & 1));
+    } else {
+        // ---- readers: warp w reads TMEM lanes 32 (w % 4) .. (the left vectors), 16 columns at a time
+        const int quarter = warp & 3, r = quarter * 32 + lane;
+        int q = 0;
+        bool late = false;
+        for (int it = it0; it < nit; it += step, ++q) {
+            const TcItem w = tc_item<NT>(a, it);
+            const int b = q & 1, i = w.i0 + r, nj = min(NT, a.n - w.j0);
+            const bool row_ok = i < a.m;
+            late |= !mbar_wait(&accf[b], (uint32_t)((q / 2) & 1), kPipeSpin);
+            __syncwarp();
+            fence_after_sync();
+            const uint32_t t0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * ACC);
+#pragma unroll 1
+            for (int c0 = 0; c0 < nj; c0 += 16) {
+                float re[16], im[16];
+                tmem_ld16_nowait(t0 + (uint32_t)c0, re);
+                tmem_ld16_nowait(t0 + (uint32_t)(NT + c0), im);
+                if (CN) {
+                    tmem_wait_ld(re, im);
+                    c32 *P = a.part + ((size_t)w.z * a.n + w.j0 + c0) * a.m + i;
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj)
+                        if (row_ok && c0 + jj < nj) P[(size_t)jj * a.m] = mkc(re[jj], im[jj]);
+                } else {
+                    // C may be D (in-place accumulate): the 16 loads of the step come before its stores
+                    float2 cv[16];
+                    const c32 *Cp = a.C + (size_t)(w.j0 + c0) * a.ldc + i;
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj)
+                        cv[jj] = (row_ok && c0 + jj < nj && a.beta != 0.f)
+                                     ? *reinterpret_cast<const float2 *>(Cp + (size_t)jj * a.ldc)
+                                     : make_float2(0.f, 0.f);
+                    tmem_wait_ld(re, im);
+                    c32 *Dp = a.D + (size_t)(w.j0 + c0) * a.ldd + i;
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj)
+                        if (row_ok && c0 + jj < nj)
+                            Dp[(size_t)jj * a.ldd] =
+                                mkc(fmaf(a.beta, cv[jj].x, a.alpha * re[jj]), fmaf(a.beta, cv[jj].y, a.alpha * im[jj]));
+                }
+            }
+            fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[b]);
+        }
+        if (late && lane == 0) atomicExch(&g_tc_err, 1);
     }
     fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, NR);
+    if (warp == kLoaders) tmem_dealloc(tmem, TCOLS);
 }
 
-__global__ void k_tc_reduce(int m, int n, int nsplit, float alpha, const z64 *__restrict__ part, float beta,
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 1) k_tc_cn(TcArgs a) { tc_body<true, NT>(a); }
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 1) k_tc_nn(TcArgs a) { tc_body<false, NT>(a); }
+
+// C = alpha (sum of the partial tiles, in split order) + beta C.  The sum is a double-FP32 pair (TwoSum):
+// FP64 additions would cost 64 cycles a warp each.
+__global__ void k_tc_reduce(int m, int n, int nsplit, float alpha, const c32 *__restrict__ part, float beta,
                             c32 *C, int ldc) {
     const size_t tot = (size_t)m * n;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
         const int i = (int)(e % m), j = (int)(e / m);
-        z64 acc = part[e];
-        for (int z = 1; z < nsplit; ++z) acc = acc + part[(size_t)z * tot + e];
-        z64 v = (double)alpha * acc;
-        if (beta != 0.f) v = v + (double)beta * cvt<double, float>(C[(size_t)j * ldc + i]);
-        C[(size_t)j * ldc + i] = cvt<float, double>(v);
+        float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+        auto add = [](float &h, float &l, float x) {
+            float err;
+            df64::two_sum(h, x, h, err);
+            l = __fadd_rn(l, err);
+        };
+#pragma unroll 8
+        for (int z = 0; z < nsplit; ++z) {
+            const c32 v = part[(size_t)z * tot + e];
+            add(rh, rl, v.x);
+            add(ih, il, v.y);
+        }
+        c32 v = mkc(fmaf(alpha, rh, alpha * rl), fmaf(alpha, ih, alpha * il));
+        if (beta != 0.f) {
+            const c32 c = C[(size_t)j * ldc + i];
+            v = mkc(fmaf(beta, c.x, v.x), fmaf(beta, c.y, v.y));
+        }
+        C[(size_t)j * ldc + i] = v;
     }
-}
-
-// ------------------------------------------------------------------ D = alpha A B + beta C
-// CTA tile: 64 complex rows of A / D (128 real rows) x NN columns of B / D, full K.
-template <int NN>
-__global__ void __launch_bounds__(kThreads, nn_ctas_per_sm<NN>())
-k_tc_nn(int M, int n, int k, float alpha, const c32 *__restrict__ A, int lda, const c32 *__restrict__ B, int ldb,
-        float beta, const c32 *C, int ldc, c32 *D, int ldd) {
-    constexpr int A_BYTES = 128 * ROWB, B_BYTES = NN * ROWB;
-    constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
-    constexpr int NS = n_stages<STAGE, nn_ring<NN>()>();
-    constexpr uint32_t IDESC = make_idesc_tf32(128, NN);
-    extern __shared__ unsigned char smraw[];
-    unsigned char *base = align1k(smraw);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(base + NS * STAGE);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + NS);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g0 = blockIdx.x * 64, jt0 = blockIdx.y * NN;
-    const int nkb = (k + KBC - 1) / KBC;
-    if (warp == 0) tmem_alloc(tslot, NN);
-    if (tid == 0)
-        for (int s = 0; s < NS; ++s) mbar_init(&bar[s], 1);
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    const uint32_t tmem = *tslot;
-    // producer map for A: each warp step covers 8 consecutive rows g x 4 consecutive K (l);
-    // lane bits -> (g low 3, l low 2), warp -> l high 2 of the 16, q -> g high 3 (of 64)
-    // with 8 warps: warp & 3 -> l high bits, warp >> 2 -> g offset 32
-    const int gl = lane & 7, ll = (lane >> 3) + 4 * (warp & 3), gq = (warp >> 2) * 32;
-    constexpr int NA = 4, NB = NN * KBC / kThreads;
-    float2 ra[NA], rb[NB];
-    auto load = [&](int kb) {
-        const int l0 = kb * KBC;
-        const int l = l0 + ll;
-#pragma unroll
-        for (int q = 0; q < NA; ++q) {
-            const int g = gq + 8 * q + gl;
-            ra[q] = (g0 + g < M && l < k) ? __ldg(reinterpret_cast<const float2 *>(A + (size_t)l * lda + g0 + g))
-                                          : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-            const int idx = tid + kThreads * q, j = idx >> 4, kc = idx & 15;
-            const int lk = l0 + kc;
-            rb[q] = (jt0 + j < n && lk < k) ? __ldg(reinterpret_cast<const float2 *>(B + (size_t)(jt0 + j) * ldb + lk))
-                                            : make_float2(0.f, 0.f);
-        }
-    };
-    int bad = 0, issued = 0;
-    if (nkb > 0) load(0);
-    for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % NS;
-        if (kb >= NS && !mbar_wait(&bar[s], (uint32_t)((kb / NS - 1) & 1), g_tc_spin)) bad = 1;
-        unsigned char *sAh = base + s * STAGE, *sAl = sAh + A_BYTES, *sBh = sAl + A_BYTES, *sBl = sBh + B_BYTES;
-#pragma unroll
-        for (int q = 0; q < NA; ++q) {
-            const int g = gq + 8 * q + gl;
-            const float rh = to_tf32(ra[q].x), ih = to_tf32(ra[q].y);
-            const float rl = to_tf32(ra[q].x - rh), il = to_tf32(ra[q].y - ih);
-            const uint32_t o0 = swz(2 * g, ll), o1 = swz(2 * g + 1, ll);
-            *reinterpret_cast<float2 *>(sAh + o0) = make_float2(rh, -ih);
-            *reinterpret_cast<float2 *>(sAl + o0) = make_float2(rl, -il);
-            *reinterpret_cast<float2 *>(sAh + o1) = make_float2(ih, rh);
-            *reinterpret_cast<float2 *>(sAl + o1) = make_float2(il, rl);
-        }
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-            const int idx = tid + kThreads * q;
-            put_split(sBh, sBl, swz(idx >> 4, idx & 15), rb[q].x, rb[q].y);
-        }
-        if (kb + 1 < nkb) load(kb + 1);
-        fence_proxy_async();
-        if (__syncthreads_or(bad)) break;
-        if (tid == 0)
-            issue_stage(tmem, smem_u32(sAh), smem_u32(sAl), smem_u32(sBh), smem_u32(sBl), IDESC, kb == 0, &bar[s]);
-        ++issued;
-    }
-    if (issued > 0) {
-        const int kl = issued - 1;
-        if (!mbar_wait(&bar[kl % NS], (uint32_t)((kl / NS) & 1))) bad = 1;
-    }
-    fence_after_sync();
-    bad = __syncthreads_or(bad);
-    const int quarter = warp & 3, half = warp >> 2;
-    const int rho = quarter * 32 + lane;  // real row of the tile: complex row g0 + rho/2, part rho & 1
-    const bool row_ok = g0 + (rho >> 1) < M;
-    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    float *Df = reinterpret_cast<float *>(D);
-    const float *Cf = reinterpret_cast<const float *>(C);
-    if (!bad) {
-#pragma unroll 1
-        for (int c0 = half * (NN / 2); c0 < (half + 1) * (NN / 2); c0 += 16) {
-            // C may be D (in-place accumulate): all 16 loads of the chunk are issued before its stores
-            float cv[16], acc[16];
-#pragma unroll
-            for (int jj = 0; jj < 16; ++jj) {
-                const int j = jt0 + c0 + jj;
-                cv[jj] = (row_ok && j < n && beta != 0.f) ? Cf[2 * ((size_t)j * ldc + g0) + rho] : 0.f;
-            }
-            if (issued > 0) {
-                tmem_ld16(trow + (uint32_t)c0, acc);
-            } else {
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) acc[jj] = 0.f;
-            }
-#pragma unroll
-            for (int jj = 0; jj < 16; ++jj) {
-                const int j = jt0 + c0 + jj;
-                if (row_ok && j < n) Df[2 * ((size_t)j * ldd + g0) + rho] = fmaf(beta, cv[jj], alpha * acc[jj]);
-            }
-        }
-    } else if (tid == 0) {
-        atomicExch(&g_tc_err, 1);
-    }
-    fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, NN);
 }
 
 template <typename Kern>
@@ -354,56 +369,64 @@ int num_sms_tc() {
     return v;
 }
 
+// Cycles of a stage (MMAs and shared-memory traffic) by NT.
+constexpr int stage_cycles(int NT) { return NT == 128 ? 900 : NT == 64 ? 600 : 450; }
+
+// NT of the cheapest tiling of n columns.
+int pick_nt(int n) {
+    int best = 128;
+    for (int nt : {64, 32})
+        if ((long long)((n + nt - 1) / nt) * stage_cycles(nt) < (long long)((n + best - 1) / best) * stage_cycles(best))
+            best = nt;
+    return best;
+}
+
 template <int NT>
-int launch_cn(GemmWork &w, int m, int n, int K, float alpha, const c32 *A, int lda, const c32 *B, int ldb,
-              float beta, c32 *C, int ldc, cudaStream_t s) {
-    constexpr int STAGE = 2 * 128 * ROWB + 2 * 2 * NT * ROWB;
-    constexpr size_t SMEM = smem_bytes<STAGE>();
+int launch_cn(GemmWork &w, TcArgs &a, float beta, c32 *C, int ldc, cudaStream_t s) {
     static std::atomic<bool> attr{false};
-    LG_TRY(ensure_smem(k_tc_cn<NT>, SMEM, attr));
-    const int tm = (m + 127) / 128, tn = (n + NT - 1) / NT;
-    const int tiles = tm * tn;
-    // one CTA per SM (shared memory): split K over the GPU.  Cost model in units of one 16-term
-    // stage of a CTA (about a microsecond): whole waves x stages per CTA, plus the FP64 partial
-    // tiles written and summed (about 7 MB per stage-time of HBM traffic); the cheapest split
-    // with chunks of 256 to 8192 terms wins.
+    LG_TRY(ensure_smem(k_tc_cn<NT>, smem_bytes(NT), attr));
+    a.tm = (a.m + kRows - 1) / kRows;
+    a.tn = (a.n + NT - 1) / NT;
+    // Split of the reduction: the busiest SM's items x (stages + about four stages' time of pipeline
+    // fill), plus the partial tiles written and summed (in units of a stage, half a microsecond, at
+    // 5 TB/s); chunks of 64 to 4096 terms, so that no FP32 accumulation is longer than that.
     const int sms = num_sms_tc();
-    int kchunk = std::max(KBC, ((K + KBC - 1) / KBC) * KBC);
+    const long long tiles = (long long)a.tm * a.tn;
     double best = 1e300;
     for (int ns = 1; ns <= 4 * sms; ++ns) {
-        const int kc = ((K + ns - 1) / ns + KBC - 1) / KBC * KBC;
-        if (kc > 8192) continue;
-        if (kc < 256 && ns > 1) break;
-        const int nsp = (K + kc - 1) / kc;
-        const long long ctas = (long long)tiles * nsp;
-        const long long waves = (ctas + sms - 1) / sms;
-        const double cost = (double)waves * (kc / KBC) + (double)nsp * 32.0 * m * (double)n / 7.2e6;
+        const int kc = ((a.K + ns - 1) / ns + KST - 1) / KST * KST;
+        if (kc > 4096) continue;
+        if (kc < 64 && ns > 1) break;
+        const int nsp = (a.K + kc - 1) / kc;
+        const long long items = tiles * nsp;
+        const double cost = (double)((items + sms - 1) / sms) * ((kc / KST + 4) * (double)stage_cycles(NT) / 900.0) +
+                            (double)nsp * 16.0 * a.m * (double)a.n / 2.3e6;
         if (cost < best) {
             best = cost;
-            kchunk = kc;
+            a.kchunk = kc;
         }
     }
-    kchunk = std::max(kchunk, KBC);
-    const int nsplit = (K + kchunk - 1) / kchunk;
-    LG_TRY(w.alloc->ensure(w.part, sizeof(z64) * (size_t)nsplit * m * n));
-    z64 *part = reinterpret_cast<z64 *>(w.part.p);
-    k_tc_cn<NT><<<dim3(tm, tn, nsplit), kThreads, SMEM, s>>>(m, n, K, kchunk, A, lda, B, ldb, part);
+    a.nsplit = (a.K + a.kchunk - 1) / a.kchunk;
+    LG_TRY(w.alloc->ensure(w.part, sizeof(c32) * (size_t)a.nsplit * a.m * a.n));
+    a.part = reinterpret_cast<c32 *>(w.part.p);
+    const int grid = (int)std::min<long long>(sms, tiles * a.nsplit);
+    k_tc_cn<NT><<<grid, kThreads, smem_bytes(NT), s>>>(a);
     LG_TRY(check_launch("tensor-core gemm A^H B"));
-    const size_t tot = (size_t)m * n;
-    const int blocks = (int)std::min<size_t>((tot + 255) / 256, 4096);
-    k_tc_reduce<<<blocks, 256, 0, s>>>(m, n, nsplit, alpha, part, beta, C, ldc);
+    const size_t tot = (size_t)a.m * a.n;
+    const int blocks = (int)std::min<size_t>((tot + 127) / 128, 4096);
+    k_tc_reduce<<<blocks, 128, 0, s>>>(a.m, a.n, a.nsplit, a.alpha, a.part, beta, C, ldc);
     return check_launch("tensor-core gemm reduce");
 }
 
-template <int NN>
-int launch_nn(int M, int n, int k, float alpha, const c32 *A, int lda, const c32 *B, int ldb, float beta,
-              const c32 *C, int ldc, c32 *D, int ldd, cudaStream_t s) {
-    constexpr int STAGE = 2 * 128 * ROWB + 2 * NN * ROWB;
-    constexpr size_t SMEM = smem_bytes<STAGE, nn_ring<NN>()>();
+template <int NT>
+int launch_nn(TcArgs &a, cudaStream_t s) {
     static std::atomic<bool> attr{false};
-    LG_TRY(ensure_smem(k_tc_nn<NN>, SMEM, attr));
-    const dim3 grid((M + 63) / 64, (n + NN - 1) / NN);
-    k_tc_nn<NN><<<grid, kThreads, SMEM, s>>>(M, n, k, alpha, A, lda, B, ldb, beta, beta != 0.f ? C : D, ldc, D, ldd);
+    LG_TRY(ensure_smem(k_tc_nn<NT>, smem_bytes(NT), attr));
+    a.tm = (a.m + kRows - 1) / kRows;
+    a.tn = (a.n + NT - 1) / NT;
+    a.nsplit = 1;
+    a.kchunk = (a.K + KST - 1) / KST * KST;
+    k_tc_nn<NT><<<(int)std::min<long long>(num_sms_tc(), (long long)a.tm * a.tn), kThreads, smem_bytes(NT), s>>>(a);
     return check_launch("tensor-core gemm A B");
 }
 
@@ -412,16 +435,42 @@ int launch_nn(int M, int n, int k, float alpha, const c32 *A, int lda, const c32
 int tc_gemm_cn(GemmWork &w, int m, int n, int K, float alpha, const c32 *A, int lda, const c32 *B, int ldb,
                float beta, c32 *C, int ldc, cudaStream_t s) {
     if (m <= 0 || n <= 0) return LOBPCG_OK;
-    if (n > 64) return launch_cn<128>(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
-    return launch_cn<64>(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, s);
+    TcArgs a{};
+    a.m = m;
+    a.n = n;
+    a.K = K;
+    a.A = A;
+    a.B = B;
+    a.lda = lda;
+    a.ldb = ldb;
+    a.alpha = alpha;
+    const int nt = pick_nt(n);
+    if (nt == 128) return launch_cn<128>(w, a, beta, C, ldc, s);
+    if (nt == 64) return launch_cn<64>(w, a, beta, C, ldc, s);
+    return launch_cn<32>(w, a, beta, C, ldc, s);
 }
 
 int tc_gemm_nn(int M, int n, int k, float alpha, const c32 *A, int lda, const c32 *B, int ldb, float beta,
                const c32 *C, int ldc, c32 *D, int ldd, cudaStream_t s) {
     if (M <= 0 || n <= 0) return LOBPCG_OK;
-    if (n > 128) return launch_nn<256>(M, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s);
-    if (n > 64) return launch_nn<128>(M, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s);
-    return launch_nn<64>(M, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s);
+    TcArgs a{};
+    a.m = M;
+    a.n = n;
+    a.K = k;
+    a.A = A;
+    a.B = B;
+    a.lda = lda;
+    a.ldb = ldb;
+    a.alpha = alpha;
+    a.beta = beta;
+    a.C = beta != 0.f ? C : D;
+    a.ldc = beta != 0.f ? ldc : ldd;
+    a.D = D;
+    a.ldd = ldd;
+    const int nt = pick_nt(n);
+    if (nt == 128) return launch_nn<128>(a, s);
+    if (nt == 64) return launch_nn<64>(a, s);
+    return launch_nn<32>(a, s);
 }
 
 int *device_wait_flag() {
