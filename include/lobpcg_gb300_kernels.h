@@ -126,7 +126,7 @@ int lobpcg_k_rayleigh_ritz32(int n, int m, const void *S, const void *A, double 
  *   A   (device, n x n complex128, ld n; lower triangle used, not modified),
  *   w   (device, n doubles), V (device, n x n complex128, ld n).
  * Householder tridiagonalisation (in one thread-block cluster's shared memory
- * up to n = 416, else one cooperative grid), multisection and inverse iteration
+ * up to n = 128, else one cooperative grid), multisection and inverse iteration
  * on the tridiagonal matrix, compact-WY back-transformation.
  */
 int lobpcg_k_heev(int n, const void *A, double *w, void *V, void *stream);

@@ -582,172 +582,6 @@ k_tri_coop(int n, cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv, cx<R
     if (blockIdx.x == 0 && tid == 0) dg[n - 1] = ldcg_cx(A + (size_t)(n - 1) * lda + n - 1).x;
 }
 
-// Fused single-launch tridiagonalisation: one grid barrier per column.
-// Block g owns the TS x TS tiles t = g, g + G, ... of the matrix (row-major tile index) and keeps
-// them in shared memory for the whole factorisation.  Invariant at the top of column i (after a
-// barrier): ypart[i & 1] holds, per tile column, the partial products A^(i)[J,J] v_i
-// (J = i+1..n-1, A^(i) = the matrix after reflectors 0..i-1), and colbuf[i & 1] holds column
-// i+1 of A^(i) from row i+1 down.  Column i then runs:
-//   (a) y_i = sum of the partials (fixed order), w_i = tau y_i - |tau|^2/2 (v_i^H y_i) v_i;
-//   (b) column i+1 of A^(i+1) = colbuf - w_i v_i^H - v_i w_i^H restricted to it, its diagonal
-//       (-> d[i+1]) and reflector i+1 (every block, redundantly, same arithmetic);
-//   (c) each owned tile: A -= w_i v_i^H + v_i w_i^H on J x J and, in the same pass, the partial
-//       product with v_{i+1} on J' x J' (J' = i+2..n-1) -> ypart[(i+1) & 1];
-//   (d) owners of column i+2 publish it (rows i+2..) -> colbuf[(i+1) & 1];  barrier.
-// Same formulas as k_tri_step1 / k_tri_step2.  Small tiles spread the FP64 work of a column
-// over more SMs (this GPU has few FP64 units per SM).  256 threads: TS rows x (256 / TS)
-// column groups of CPT = TS*TS/256 columns.  Dynamic shared memory: the owned tiles, then
-// v_i, w_i, v_{i+1} and the working column (n complex each).
-template <typename RT, int TS, typename CT = RT>
-__global__ void __launch_bounds__(256)
-k_tri_fused(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv, cx<RT> *__restrict__ taus,
-            RT *__restrict__ dg, RT *__restrict__ eg, cx<RT> *__restrict__ ypart_st, cx<RT> *__restrict__ colbuf_st,
-            unsigned int *bar, int *err) {
-    static_assert(sizeof(cx<CT>) == sizeof(cx<RT>), "the compute type keeps the storage size");
-    cx<CT> *ypart = reinterpret_cast<cx<CT> *>(ypart_st);   // scratch kept in the compute type
-    cx<CT> *colbuf = reinterpret_cast<cx<CT> *>(colbuf_st);
-    constexpr int TT = TS * TS, NG = 256 / TS, CPT = TT / 256;
-    extern __shared__ __align__(16) unsigned char dsm[];
-    const int T = (n + TS - 1) / TS, G = gridDim.x, g = blockIdx.x, tid = threadIdx.x;
-    const int nown = (T * T - g + G - 1) / G;  // tiles g, g+G, ... below T*T
-    cx<CT> *tiles = reinterpret_cast<cx<CT> *>(dsm);  // nown x [TS cols][TS rows]
-    cx<CT> *v = tiles + (size_t)nown * TT;             // v_i on [0, n)
-    cx<CT> *w = v + n;                                  // w_i
-    cx<CT> *vn = w + n;                                 // v_{i+1}
-    cx<CT> *x = vn + n;                                 // working column
-    __shared__ CT sh[32];
-    __shared__ cx<CT> acc[NG][TS + 1];
-    const int rl = tid % TS, cg = tid / TS;
-    const cx<CT> zero = mkc<CT>(0.0, 0.0);
-    unsigned int arrivals = 0;
-    // load the owned tiles (entries outside the matrix are zero)
-    for (int q = 0; q < nown; ++q) {
-        const int t = g + q * G, TR = t / T, TC = t % T;
-        for (int e = tid; e < TT; e += blockDim.x) {
-            const int r = TR * TS + (e % TS), c = TC * TS + (e / TS);
-            tiles[(size_t)q * TT + e] = (r < n && c < n) ? ld_as<CT>(A + (size_t)c * lda + r) : zero;
-        }
-    }
-    // reflector 0 from column 0 (read from A, unmodified), d[0]
-    Refl<CT> R = make_reflector<CT, false, RT>(A + 1, n - 1, sh);
-    for (int r = tid; r < n; r += blockDim.x)
-        v[r] = (r < 1) ? zero : (r == 1 ? mkc<CT>(1.0, 0.0) : ld_as<CT>(A + r) * R.scal);
-    if (g == 0 && tid == 0) dg[0] = A[0].x;
-    __syncthreads();
-    // partial products A^(0)[J,J] v_0 and column 1 of A^(0)
-    for (int q = 0; q < nown; ++q) {
-        const int t = g + q * G, TR = t / T, TC = t % T;
-        const cx<CT> *tl = tiles + (size_t)q * TT;
-        const int r = TR * TS + rl;
-        cx<CT> sacc = zero;
-#pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            const int cl = cg * CPT + k, c = TC * TS + cl;
-            if (r >= 1 && r < n && c >= 1 && c < n) sacc = sacc + tl[cl * TS + rl] * v[c];
-        }
-        acc[cg][rl] = sacc;
-        __syncthreads();
-        if (tid < TS) {
-            cx<CT> u = acc[0][tid];
-            for (int k = 1; k < NG; ++k) u = u + acc[k][tid];
-            const int rr = TR * TS + tid;
-            if (rr < n) ypart[(size_t)TC * n + rr] = u;
-            if (n > 1 && TC == 1 / TS && rr >= 1 && rr < n) colbuf[rr] = tl[(1 % TS) * TS + tid];
-        }
-        __syncthreads();
-    }
-    arrivals += G;
-    if (!grid_barrier(bar, arrivals, err)) return;
-
-    for (int i = 0; i + 1 < n; ++i) {
-        const int par = i & 1;
-        const cx<CT> *yp = ypart + (size_t)par * T * n;
-        const cx<CT> *cb = colbuf + (size_t)par * n;
-        // (a) y_i and w_i on J = [i+1, n); loads issued in groups of 8 before they are summed
-        CT dre = 0.0;
-        for (int r = i + 1 + tid; r < n; r += blockDim.x) {
-            cx<CT> y = zero;
-            for (int c = 0; c < T; c += 8) {
-                cx<CT> t8[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) t8[k] = (c + k < T) ? ldcg_cx(yp + (size_t)(c + k) * n + r) : zero;
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (c + k < T) y = y + t8[k];
-            }
-            dre += v[r].x * y.x + v[r].y * y.y;
-            w[r] = y;
-        }
-        dre = block_sum(dre, sh);
-        const CT t2 = (CT)0.5 * abs2(R.tau) * dre;
-        for (int r = i + 1 + tid; r < n; r += blockDim.x) w[r] = R.tau * w[r] - t2 * v[r];
-        __syncthreads();
-        // (b) column i+1 of A^(i+1) from row i+1; d[i+1]; reflector i+1
-        const cx<CT> vi1 = v[i + 1], wi1 = w[i + 1];
-        for (int r = i + 1 + tid; r < n; r += blockDim.x)
-            x[r] = ldcg_cx(cb + r) - mul_conj(w[r], vi1) - mul_conj(v[r], wi1);
-        __syncthreads();
-        if (g == 0) {  // reflectors kept in the compute type (read by the back-transformation)
-            cx<CT> *HvC = reinterpret_cast<cx<CT> *>(Hv);
-            for (int r = i + 1 + tid; r < n; r += blockDim.x) HvC[(size_t)i * n + r] = v[r];
-            if (tid == 0) {
-                reinterpret_cast<cx<CT> *>(taus)[i] = R.tau;
-                eg[i] = (RT)R.beta;
-                dg[i + 1] = (RT)x[i + 1].x;
-            }
-        }
-        if (i + 2 >= n) break;  // last column: nothing left to transform
-        const Refl<CT> Rn = make_reflector<CT>(x + i + 2, n - i - 2, sh);
-        for (int r = tid; r < n; r += blockDim.x)
-            vn[r] = (r < i + 2) ? zero : (r == i + 2 ? mkc<CT>(1.0, 0.0) : x[r] * Rn.scal);
-        __syncthreads();
-        // (c) update the owned tiles with (w_i, v_i) and multiply by v_{i+1}; (d) publish column i+2
-        cx<CT> *ypn = ypart + (size_t)(1 - par) * T * n;
-        cx<CT> *cbn = colbuf + (size_t)(1 - par) * n;
-        const int c2 = i + 2;
-        for (int q = 0; q < nown; ++q) {
-            const int t = g + q * G, TR = t / T, TC = t % T;
-            cx<CT> *tl = tiles + (size_t)q * TT;
-            if (TR * TS + TS - 1 < i + 1 || TC * TS + TS - 1 < i + 1) {
-                // tile outside J x J: its share of y_{i+1} is zero (uniform branch)
-                if (tid < TS) {
-                    const int rr = TR * TS + tid;
-                    if (rr < n) ypn[(size_t)TC * n + rr] = zero;
-                }
-                continue;
-            }
-            const int r = TR * TS + rl;
-            const bool rin = r >= i + 1 && r < n;
-            const cx<CT> wr = rin ? w[r] : zero, vr = rin ? v[r] : zero;
-            cx<CT> sacc = zero;
-#pragma unroll
-            for (int k = 0; k < CPT; ++k) {
-                const int cl = cg * CPT + k, c = TC * TS + cl;
-                if (rin && c >= i + 1 && c < n) {
-                    cx<CT> a = tl[cl * TS + rl];
-                    a = a - mul_conj(wr, v[c]) - mul_conj(vr, w[c]);
-                    tl[cl * TS + rl] = a;
-                    if (r >= c2 && c >= c2) sacc = sacc + a * vn[c];
-                }
-            }
-            acc[cg][rl] = sacc;
-            __syncthreads();
-            if (tid < TS) {
-                cx<CT> u = acc[0][tid];
-                for (int k = 1; k < NG; ++k) u = u + acc[k][tid];
-                const int rr = TR * TS + tid;
-                if (rr < n) ypn[(size_t)TC * n + rr] = u;
-                if (TC == c2 / TS && rr >= c2 && rr < n) cbn[rr] = tl[(c2 % TS) * TS + tid];
-            }
-            __syncthreads();
-        }
-        R = Rn;
-        for (int r = tid; r < n; r += blockDim.x) v[r] = vn[r];
-        arrivals += G;
-        if (!grid_barrier(bar, arrivals, err)) return;
-    }
-}
-
 // a - w_r conj(v_c) - v_r conj(w_c), each real part through fused multiply-adds
 template <typename CT>
 __device__ __forceinline__ cx<CT> rank2_entry(cx<CT> a, cx<CT> wr, cx<CT> vr, cx<CT> vc, cx<CT> wc) {
@@ -771,8 +605,8 @@ __device__ __forceinline__ cx<CT> cmac(cx<CT> acc, cx<CT> a, cx<CT> b) {
     return mkc<CT>(re, im);
 }
 
-// The same reduction held in the shared memory of one thread-block cluster of CS CTAs, for
-// matrices small enough to fit there (n up to about 416 with 16 CTAs).  CTA q keeps the rows
+// The reduction held in the shared memory of one thread-block cluster of CS CTAs, for small
+// matrices (see kTriClusterMaxN).  CTA q keeps the rows
 // r = q + CS j of the full Hermitian matrix, row-major, so that y = A v needs no reduction
 // across CTAs.  Per column i, after one cluster barrier every CTA holds y_i = A^(i) v_i and
 // column i+1 of A^(i), both gathered through distributed shared memory, and forms w_i, the
@@ -781,8 +615,8 @@ __device__ __forceinline__ cx<CT> cmac(cx<CT> acc, cx<CT> a, cx<CT> b) {
 // its rows of the trailing block and, in the same pass, multiplies them by v_{i+1} (one warp
 // per row), and sends its entries of y_{i+1} and of column i+2 to every CTA.  The gathered
 // vectors alternate between two buffers, so that one barrier per column orders every write
-// after the reads of the buffer it overwrites.  Outputs as k_tri_fused (Hv, taus in the
-// compute type; d, e).  Dynamic shared memory: nr x n matrix entries (nr = ceil(n / CS)) and
+// after the reads of the buffer it overwrites.  Outputs: Hv, taus in the
+// compute type; d, e.  Dynamic shared memory: nr x n matrix entries (nr = ceil(n / CS)) and
 // 7 n vector entries.
 template <typename RT, typename CT>
 __global__ void __launch_bounds__(1024, 1)
@@ -883,6 +717,234 @@ k_tri_cluster(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__
         }
         R = Rn;
         cl.sync();
+    }
+}
+
+// ---- light sums, for the few steps of a shuffle tree: double-FP32 pairs whose low part is renormalised
+// only at the end.  Each step keeps the exact error of the high parts' sum; the low part, a few units
+// of 2^-24 of the high one, rounds at 2^-48 of it.  Plain arithmetic for other types.
+template <typename CT>
+__device__ __forceinline__ CT light_add(CT a, CT b) { return a + b; }
+template <>
+__device__ __forceinline__ df64 light_add<df64>(df64 a, df64 b) {
+    df64 r;
+    df64::two_sum(a.hi, b.hi, r.hi, r.lo);
+    r.lo = __fadd_rn(r.lo, __fadd_rn(a.lo, b.lo));
+    return r;
+}
+template <typename CT>
+__device__ __forceinline__ CT light_norm(CT a) { return a; }
+template <>
+__device__ __forceinline__ df64 light_norm<df64>(df64 a) { return df64::norm(a.hi, a.lo); }
+
+template <typename CT>
+__device__ __forceinline__ CT light_warp_sum(CT v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v = light_add<CT>(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// The warps' partial sums into sh (one entry per warp, not reused before another barrier), and, in one
+// warp after the barrier, their sum.
+template <typename CT>
+__device__ __forceinline__ void light_partial(CT v, CT *sh) {
+    v = light_warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+}
+template <typename CT>
+__device__ __forceinline__ CT light_total(const CT *sh) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    return light_norm(light_warp_sum(lane < nw ? sh[lane] : CT(0.0)));
+}
+
+// Reflector from alpha = x[0] and s = sum_{r>=1} |x[r]|^2 (as reflector_from), by a whole warp: lanes 0-3
+// each take one of the four divisions.
+template <typename CT>
+__device__ __forceinline__ Refl<CT> reflector_warp(cx<CT> alpha, CT s) {
+    Refl<CT> R;
+    if (s == CT(0.0) && alpha.y == CT(0.0)) {
+        R.tau = mkc<CT>(0.0, 0.0);
+        R.beta = alpha.x;
+        R.scal = mkc<CT>(0.0, 0.0);
+        return R;
+    }
+    const int lane = threadIdx.x & 31;
+    const CT beta = -copysign(sqrt(abs2(alpha) + s), alpha.x);
+    const cx<CT> den = mkc<CT>(alpha.x - beta, alpha.y);
+    const CT num = (lane & 3) == 0 ? beta - alpha.x : (lane & 3) == 2 ? den.x : (lane & 3) == 1 ? -alpha.y : -den.y;
+    const CT quo = num / ((lane & 2) ? abs2(den) : beta);
+    R.beta = beta;
+    R.tau = mkc<CT>(__shfl_sync(0xffffffffu, quo, 0), __shfl_sync(0xffffffffu, quo, 1));
+    R.scal = mkc<CT>(__shfl_sync(0xffffffffu, quo, 2), __shfl_sync(0xffffffffu, quo, 3));
+    return R;
+}
+
+// Grid barrier of co-resident blocks: one counter, arrival by a releasing reduction, one polling thread
+// per block with acquiring loads.  2250 cycles on 152 blocks (fences around a plain atomic: 2850;
+// a flag per block, polled by a warp or by every thread: 7000 to 9000, the polls delay the stores).
+// Bounded like grid_barrier.
+__device__ __forceinline__ bool release_barrier(unsigned int *count, unsigned int target, int *err) {
+    __syncthreads();
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        ok = false;
+        for (long long it = 0; it < (1LL << 22); ++it) {
+            unsigned int c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
+            if (c >= target) { ok = true; break; }
+            if ((it & 255) == 255 && *reinterpret_cast<volatile int *>(err)) break;
+        }
+        if (!ok) atomicExch(err, 1);
+    }
+    return __syncthreads_and(ok) != 0;
+}
+
+// Householder tridiagonalisation with the rows of the full Hermitian matrix dealt cyclically to the
+// blocks of one cooperative grid (row r to block r mod G), in shared memory, so that y = A v needs
+// no reduction across blocks.  Per column i, after one grid barrier every block reads y_i = A^(i) v_i and
+// column i+1 of A^(i) (2 n entries through L2) and forms w_i, the next column, d, e and reflector i+1
+// itself: the same operations on the same values in the same order, so the same bits in every
+// block.  Then each block updates its rows of the trailing block and in the same pass multiplies
+// them by v_{i+1} (WPR warps per row), and publishes its entries of y_{i+1} and of column i+2 in the other of
+// two buffers.  v_i[i+1] = 1, so column i+1 needs only each thread's own w and the scalar w[i+1].
+// What bounds it: the chain of a column (grid barrier, the L2 reads, two block sums, square root and
+// divisions), about 4 us, and above n = 800 the double-FP32 updates of the rows.  Cycles of a column at
+// n = 384 / 1152: grid barrier 2250, L2 reads 900 / 1500, sums and scalars 2500, vectors 1500 / 3000, rows
+// 1500 / 7000.  Measured (Rayleigh-Ritz step, m = n / 3, double-FP32 / FP64, ms), the cluster kernel
+// (n = 384) or the tile kernel (n = 1152), whose blocks each summed 36 partial products per row, before:
+//   n = 192  2.50 -> 2.26 / 5.45 -> 4.51;  384  5.96 -> 5.05 / 13.8 -> 10.1;  1152  62 -> 34 / 140 -> 84
+// Dynamic shared memory: nr x n matrix entries (nr = ceil(n / G)), 3 n vector entries.
+template <typename RT, typename CT>
+__global__ void __launch_bounds__(512)
+k_tri_rows(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv, cx<RT> *__restrict__ taus,
+           RT *__restrict__ dg, RT *__restrict__ eg, cx<RT> *__restrict__ xch_st, unsigned int *count, int *err) {
+    static_assert(sizeof(cx<CT>) == sizeof(cx<RT>), "the compute type keeps the storage size");
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ CT sh[2][16], dots;
+    __shared__ cx<CT> part[512 / 32], al;
+    __shared__ Refl<CT> rs;
+    const int G = gridDim.x, q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, nw = blockDim.x >> 5;
+    const int nr = (n + G - 1) / G;
+    const int WPR = max(1, nw / nr), rstep = nw / WPR;   // warps per row, rows at a time
+    cx<CT> *M = reinterpret_cast<cx<CT> *>(dsm);          // local row j = global row q + G j
+    cx<CT> *v = M + (size_t)nr * n, *w = v + n, *x = w + n;
+    cx<CT> *xch = reinterpret_cast<cx<CT> *>(xch_st);     // [parity][y, column][n]
+    cx<CT> *HvC = reinterpret_cast<cx<CT> *>(Hv);
+    const cx<CT> zero = mkc<CT>(0.0, 0.0);
+    for (size_t e = tid; e < (size_t)nr * n; e += blockDim.x) {
+        const int r = q + G * (int)(e % nr), c = (int)(e / nr);   // neighbouring threads on neighbouring owned rows
+        M[(size_t)(e % nr) * n + c] = r < n ? ld_as<CT>(A + (size_t)c * lda + r) : zero;
+    }
+    // reflector 0 from column 0 of A, d[0]
+    CT sq = 0.0;
+    for (int r = 2 + tid; r < n; r += blockDim.x) sq = light_add<CT>(sq, abs2(ld_as<CT>(A + r)));
+    light_partial(sq, sh[0]);
+    Refl<CT> R = reflector_warp<CT>(ld_as<CT>(A + 1), light_total(sh[0]));
+    for (int r = tid; r < n; r += blockDim.x) v[r] = (r < 1) ? zero : (r == 1 ? mkc<CT>(1.0, 0.0) : ld_as<CT>(A + r) * R.scal);
+    if (q == 0 && tid == 0) dg[0] = A[0].x;
+    __syncthreads();
+    for (int i = -1; i + 1 < n; ++i) {
+        // i = -1: only the products A^(0) v_0 and column 1 of A^(0)
+        const int c2 = i + 2;
+        cx<CT> *vn = v;
+        if (i >= 0) {
+            const cx<CT> *yv = xch + (size_t)(i & 1) * 2 * n, *cv = yv + n;
+            const cx<CT> y1 = ldcg_cx(yv + i + 1);
+            CT dre = 0.0;
+            for (int r = i + 1 + tid; r < n; r += blockDim.x) {
+                const cx<CT> y = ldcg_cx(yv + r), vr = v[r];
+                x[r] = ldcg_cx(cv + r);
+                w[r] = y;
+                dre = fma(vr.x, y.x, fma(vr.y, y.y, dre));
+            }
+            light_partial(dre, sh[1]);
+            if (wp == 0) {
+                const CT t = light_total(sh[1]);
+                if (lane == 0) dots = (CT)0.5 * abs2(R.tau) * t;
+            }
+            __syncthreads();
+            // w = tau y - |tau|^2 / 2 (v^H y) v, column i+1 of A^(i+1) = c - w - conj(w[i+1]) v on J = [i+1, n)
+            const CT t2 = dots;
+            cx<CT> w1 = R.tau * y1;
+            w1.x = w1.x - t2;
+            CT s = 0.0;
+            for (int r = i + 1 + tid; r < n; r += blockDim.x) {
+                const cx<CT> vr = v[r], y = w[r], c = x[r];
+                cx<CT> wr, xr;
+                wr.x = fma(R.tau.x, y.x, fma(-R.tau.y, y.y, -(t2 * vr.x)));
+                wr.y = fma(R.tau.x, y.y, fma(R.tau.y, y.x, -(t2 * vr.y)));
+                xr.x = fma(-vr.x, w1.x, fma(-vr.y, w1.y, c.x - wr.x));
+                xr.y = fma(-vr.y, w1.x, fma(vr.x, w1.y, c.y - wr.y));
+                w[r] = wr;
+                x[r] = xr;
+                if (r == c2) al = xr;
+                if (r > c2) s = fma(xr.x, xr.x, fma(xr.y, xr.y, s));
+                if (q == i % G) HvC[(size_t)i * n + r] = vr;
+                if (r == i + 1 && q == 0) {
+                    reinterpret_cast<cx<CT> *>(taus)[i] = R.tau;
+                    eg[i] = (RT)R.beta;
+                    dg[i + 1] = (RT)xr.x;
+                }
+            }
+            if (c2 >= n) break;   // last column: nothing left to transform
+            light_partial(s, sh[0]);
+            if (wp == 0) {        // one warp: every warp at once would share the FP64 units' and divisions' time
+                const Refl<CT> t = reflector_warp<CT>(al, light_total(sh[0]));
+                if (lane == 0) rs = t;
+            }
+            __syncthreads();
+            R = rs;
+            for (int r = c2 + tid; r < n; r += blockDim.x) x[r] = r == c2 ? mkc<CT>(1.0, 0.0) : x[r] * R.scal;
+            vn = x;
+            __syncthreads();
+        }
+        // rank-2 update of the owned rows of [c2, n)^2 (columns and rows from 1 on at i = -1), times vn
+        cx<CT> *yo = xch + (size_t)((i + 1) & 1) * 2 * n, *co = yo + n;
+        for (int j0 = 0; j0 < nr; j0 += rstep) {
+            const int j = j0 + wp / WPR, sub = wp % WPR, r = q + G * j;
+            const bool on = wp < rstep * WPR && j < nr && r >= c2 && r < n;
+            if (on) {
+                cx<CT> *Mr = M + (size_t)j * n;
+                cx<CT> acc = zero;
+                const cx<CT> wr = i >= 0 ? w[r] : zero, vr = i >= 0 ? v[r] : zero;
+                for (int c = c2 + lane + 32 * sub; c < n; c += 32 * WPR) {
+                    cx<CT> a = Mr[c];
+                    if (i >= 0) {
+                        const cx<CT> vc = v[c], wc = w[c];
+                        // pairs: accurate sums here (a third more instructions of this line); the chain of
+                        // multiply-adds leaves a tenth to a quarter more error in the eigenvectors at n = 640
+                        if constexpr (std::is_same<CT, df64>::value) a = a - mul_conj(wr, vc) - mul_conj(vr, wc);
+                        else a = rank2_entry(a, wr, vr, vc, wc);
+                        Mr[c] = a;
+                    }
+                    acc = cmac(acc, a, vn[c]);
+                }
+                // both parts in one tree: after the first step the lower half warp has re, the upper im
+                const bool up = lane >= 16;
+                const CT mine = up ? acc.y : acc.x, other = __shfl_xor_sync(0xffffffffu, up ? acc.x : acc.y, 16);
+                CT t = light_add<CT>(mine, other);
+#pragma unroll
+                for (int o = 8; o; o >>= 1) t = light_add<CT>(t, __shfl_xor_sync(0xffffffffu, t, o));
+                const CT im = __shfl_sync(0xffffffffu, t, 16);
+                if (lane == 0) part[wp] = mkc<CT>(t, im);
+            }
+            __syncthreads();
+            if (on && sub == 0 && lane == 0) {
+                cx<CT> t = part[wp];
+                for (int k = 1; k < WPR; ++k) t = mkc<CT>(light_add<CT>(t.x, part[wp + k].x), light_add<CT>(t.y, part[wp + k].y));
+                yo[r] = mkc<CT>(light_norm(t.x), light_norm(t.y));
+                co[r] = M[(size_t)j * n + c2];
+            }
+            if (j0 + rstep < nr) __syncthreads();
+        }
+        if (i >= 0) {
+            cx<CT> *t = v;
+            v = x;
+            x = t;
+        }
+        if (!release_barrier(count, (unsigned int)(i + 2) * (unsigned int)G, err)) return;
     }
 }
 
@@ -1437,14 +1499,13 @@ int allow_max_dyn_smem(const void *fn) {
     return LOBPCG_OK;
 }
 
-// The cluster-resident tridiagonalisation when the matrix fits one cluster's shared memory
-// (16 CTAs above n = 192, else 8) and the device can place such a cluster; done = false
-// leaves the reduction to the grid-wide kernels.
+// The cluster-resident tridiagonalisation (8 CTAs) when the device can place such a cluster;
+// done = false leaves the reduction to the grid-wide kernels.
 template <typename RT, typename CT>
 int launch_tri_cluster(int n, const cx<RT> *A, int lda, cx<RT> *Hv, cx<RT> *taus, RT *dg, RT *eg, cudaStream_t s,
                        bool &done) {
     done = false;
-    const int CS = n > 192 ? 16 : 8;
+    const int CS = 8;
     const int nr = (n + CS - 1) / CS;
     const size_t dsm = sizeof(cx<CT>) * ((size_t)nr * n + 7 * (size_t)n);
     int dev = 0, smem_max = 0, cl_ok = 0;
@@ -1458,7 +1519,6 @@ int launch_tri_cluster(int n, const cx<RT> *A, int lda, cx<RT> *Hv, cx<RT> *taus
     // the same (largest) limit from every caller: concurrent lanes launch this kernel with
     // different sizes, and a per-call limit set by one would invalidate another's launch
     LG_TRY(allow_max_dyn_smem(fn));
-    if (CS > 8) LG_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CS);
     cfg.blockDim = dim3(std::min(1024, 32 * nr));  // one warp per owned row
@@ -1481,7 +1541,51 @@ int launch_tri_cluster(int n, const cx<RT> *A, int lda, cx<RT> *Hv, cx<RT> *taus
     done = true;
     return LOBPCG_OK;
 }
-constexpr int kTriClusterMaxN = 416;
+// The row-cyclic cooperative tridiagonalisation, when the rows of a block and three vectors fit its
+// shared memory; done = false leaves the reduction to the other kernels.  With concurrent streams
+// each grid takes its share of the SMs (so that all of them are resident together).
+template <typename RT, typename CT>
+int launch_tri_rows(EigWork &w, int n, const cx<RT> *A, int lda, cx<RT> *Hv, cx<RT> *taus, RT *dg, RT *eg, cx<RT> *xch,
+                    unsigned int *count, cudaStream_t s, bool &done) {
+    done = false;
+    int dev = 0, sms = 0, coop = 0, smem_max = 0;
+    LG_CUDA_TRY(cudaGetDevice(&dev));
+    LG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    LG_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    LG_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    int *err = device_wait_flag();
+    const int share = std::max(1, w.coop_share);
+    int G = std::max(1, std::min(n, sms / share));
+    const int nr = (n + G - 1) / G;
+    G = (n + nr - 1) / nr;   // as few blocks as give the same rows per block
+    const size_t dsm = sizeof(cx<CT>) * ((size_t)nr * n + 3 * (size_t)n);
+    const void *fn = (const void *)k_tri_rows<RT, CT>;
+    cudaFuncAttributes fa;
+    LG_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
+    if (!coop || !err || dsm + fa.sharedSizeBytes > (size_t)smem_max) return LOBPCG_OK;
+    LG_TRY(allow_max_dyn_smem(fn));
+    int per_sm = 0;
+    LG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 512, dsm));
+    if (per_sm < 1 || (size_t)G * share > (size_t)sms * per_sm) return LOBPCG_OK;
+    void *args[] = {(void *)&n, (void *)&A, (void *)&lda, (void *)&Hv, (void *)&taus, (void *)&dg,
+                    (void *)&eg, (void *)&xch, (void *)&count, (void *)&err};
+    if (w.gate && share == 1) {
+        // one cooperative grid at a time across concurrent streams
+        std::lock_guard<std::mutex> lk(w.gate->mu);
+        if (w.gate->used) LG_CUDA_TRY(cudaStreamWaitEvent(s, w.gate->ev, 0));
+        LG_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(512), args, dsm, s));
+        LG_CUDA_TRY(cudaEventRecord(w.gate->ev, s));
+        w.gate->used = true;
+    } else {
+        LG_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(512), args, dsm, s));
+    }
+    LG_TRY(check_launch("tridiagonalisation (rows)"));
+    done = true;
+    return LOBPCG_OK;
+}
+// One cluster's barrier is cheaper than the grid's, its 8 or 16 SMs' arithmetic dearer: 1.48 against
+// 1.52 ms at n = 128 (double-FP32 step, m = n / 3), 2.50 against 2.26 at n = 192; FP64 3.10 / 3.03, 5.45 / 4.51.
+constexpr int kTriClusterMaxN = 128;
 constexpr int kWyChunks = 8;   // row chunks of the back-transformation's Gram partials
 
 // T factors, then the blocked application; NV eigenvectors per CTA, as many as keep about
@@ -1520,8 +1624,8 @@ int heev_lowest_t(EigWork &w, int n, int m, cx<RT> *A, int lda, RT *theta, cx<RT
     const size_t o_tau = take(sizeof(cx<RT>) * n);
     const size_t o_d = take(sizeof(RT) * n);
     const size_t o_e = take(sizeof(RT) * n);
-    const size_t o_yp = take(sizeof(cx<RT>) * 2 * (size_t)((n + 15) / 16) * n);
-    const size_t o_wv = take(sizeof(cx<RT>) * 2 * (size_t)n);
+    const size_t o_yp = take(sizeof(cx<RT>) * (size_t)((n + 31) / 32) * n);
+    const size_t o_wv = take(sizeof(cx<RT>) * 4 * (size_t)n);
     const size_t o_z = take(sizeof(RT) * (size_t)n * m);
     const size_t o_cnt = take(sizeof(unsigned int) * n);
     const size_t o_tf = take(sizeof(cx<RT>) * (size_t)kWy * kWy * ((n + kWy - 1) / kWy));
@@ -1552,56 +1656,14 @@ int heev_lowest_t(EigWork &w, int n, int m, cx<RT> *A, int lda, RT *theta, cx<RT
         hv_df = done && df;
     }
     if (!coop_done && n >= 2) {
-        // fused version: tiles resident in shared memory, one grid barrier per column; 16 x 16
-        // tiles for small matrices (more SMs share a column's FP64 work), else 32 x 32
-        int dev = 0, sms = 0, coop = 0, smem_max = 0;
-        LG_CUDA_TRY(cudaGetDevice(&dev));
-        LG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        LG_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        LG_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        const bool small_tiles = n <= 256;
-        const int TS = small_tiles ? 16 : 32;
-        const int T = (n + TS - 1) / TS;
-        // with concurrent streams each cooperative grid gets its share of the SMs, so that all of
-        // them fit at once (no gate needed then)
-        const int share = std::max(1, w.coop_share);
-        const int G = std::max(1, std::min(T * T, sms / share));
-        const int nown = (T * T + G - 1) / G;
-        const size_t dsm = sizeof(cx<RT>) * ((size_t)nown * TS * TS + 4 * (size_t)n);
-        const size_t static_sm = sizeof(RT) * 32 + sizeof(cx<RT>) * 16 * 33 + 64;
-        int *err = device_wait_flag();
-        const void *fn = small_tiles ? (const void *)k_tri_fused<RT, 16> : (const void *)k_tri_fused<RT, 32>;
-        bool fn_df = false;
+        bool done = false, df = false;
         if constexpr (std::is_same<RT, double>::value) {
-            if (w.df) {  // the column's vector work in double-FP32 (this GPU has few FP64 units per SM)
-                fn = small_tiles ? (const void *)k_tri_fused<RT, 16, df64> : (const void *)k_tri_fused<RT, 32, df64>;
-                fn_df = true;
-            }
+            df = w.df;
+            if (df) LG_TRY((launch_tri_rows<RT, df64>(w, n, A, lda, Hv, taus, dg, eg, wv, cnt, s, done)));
         }
-        if (coop && err && dsm + static_sm <= (size_t)smem_max) {
-            LG_TRY(allow_max_dyn_smem(fn));
-            int per_sm = 0;
-            LG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, dsm));
-            if (per_sm >= 1 && (size_t)G * share <= (size_t)sms * per_sm) {
-                unsigned int *bar = cnt;
-                const cx<RT> *Ac = A;
-                void *args[] = {(void *)&n, (void *)&Ac, (void *)&lda, (void *)&Hv, (void *)&taus, (void *)&dg,
-                                (void *)&eg, (void *)&yp, (void *)&wv, (void *)&bar, (void *)&err};
-                if (w.gate && share == 1) {
-                    // one cooperative grid at a time across concurrent streams
-                    std::lock_guard<std::mutex> lk(w.gate->mu);
-                    if (w.gate->used) LG_CUDA_TRY(cudaStreamWaitEvent(s, w.gate->ev, 0));
-                    LG_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(256), args, dsm, s));
-                    LG_CUDA_TRY(cudaEventRecord(w.gate->ev, s));
-                    w.gate->used = true;
-                } else {
-                    LG_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(256), args, dsm, s));
-                }
-                LG_TRY(check_launch("tridiagonalisation (fused cooperative)"));
-                coop_done = true;
-                hv_df = fn_df;  // reflectors stored as pairs
-            }
-        }
+        if (!df) LG_TRY((launch_tri_rows<RT, RT>(w, n, A, lda, Hv, taus, dg, eg, wv, cnt, s, done)));
+        coop_done = done;
+        hv_df = done && df;
     }
     if (!coop_done && n >= 2 && n <= 1024) {
         // one cooperative launch; falls back to two launches per column if it cannot run
