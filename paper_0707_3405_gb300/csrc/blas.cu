@@ -12,6 +12,7 @@
 // split over grid.z; the partial tiles are summed afterwards in a fixed
 // order, so results are bitwise reproducible.
 #include "common.cuh"
+#include "df64.cuh"
 
 #include <algorithm>
 #include <type_traits>
@@ -28,11 +29,23 @@ constexpr int BK = 16, TH = 256;
 // about 1e-6 relative accuracy; split partial sums are FP64.
 constexpr int KFLUSH = 256;
 
+// The part of [kbeg, kend) where a tile's operands are not known to be zero (see kTriA, kTriB): A lower
+// triangular has k <= i as it is and k >= i conjugate-transposed (kbeg stays a multiple of BK), B lower
+// triangular and conjugate-transposed has k <= j.
+template <bool CA, int BM, int BN>
+__device__ __forceinline__ void tri_range(int form, int i0, int j0, int &kbeg, int &kend) {
+    if (form & kTriA) {
+        if (CA) kbeg = max(kbeg, i0);
+        else kend = min(kend, i0 + BM);
+    }
+    if (form & kTriB) kend = min(kend, j0 + BN);
+}
+
 template <typename R, bool CA, bool CB, int T>
 __global__ void __launch_bounds__(TH)
 k_gemm(int m, int n, int K, int kchunk, R alpha, const cx<R> *__restrict__ A, int lda,
        const cx<R> *__restrict__ B, int ldb, R beta, const cx<R> *C, int ldc, cx<R> *D, int ldd,
-       z64 *__restrict__ part, int lower) {
+       z64 *__restrict__ part, int form, GemmBatch bt) {
     constexpr int BM = 16 * T, BN = 16 * T;
     __shared__ cx<R> As[BK][BM + 1];
     __shared__ cx<R> Bs[BK][BN + 1];
@@ -40,9 +53,23 @@ k_gemm(int m, int n, int K, int kchunk, R alpha, const cx<R> *__restrict__ A, in
     const int tx = tid & 15, ty = tid >> 4;
     const int i0 = blockIdx.x * BM, j0 = blockIdx.y * BN;
     // lower-triangle output: a tile strictly above the diagonal is neither computed nor written
-    if (lower && blockIdx.x < blockIdx.y) return;
-    const int kbeg = blockIdx.z * kchunk;
-    const int kend = min(K, kbeg + kchunk);
+    if ((form & kLowerOut) && blockIdx.x < blockIdx.y) return;
+    int kbeg = blockIdx.z * kchunk;
+    if (bt.count) {   // one product per blockIdx.z, the last one smaller
+        const int z = blockIdx.z;
+        A += z * bt.a;
+        B += z * bt.b;
+        C += z * bt.c;
+        D += z * bt.c;
+        if (z == bt.count - 1) {
+            m = bt.mlast;
+            K = bt.klast;
+        }
+        kbeg = 0;
+        if (i0 >= m) return;
+    }
+    int kend = min(K, kbeg + kchunk);
+    tri_range<CA, BM, BN>(form, i0, j0, kbeg, kend);
     const cx<R> zero = mkc<R>(0, 0);
     constexpr bool F32 = sizeof(R) == 4;
     cx<R> acc[T][T];
@@ -144,9 +171,8 @@ struct dfc {
 };
 
 __device__ __forceinline__ dfc to_dfc(z64 v, bool conj) {
-    const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
-    const float rl = __double2float_rn(v.x - (double)rh), il = __double2float_rn(v.y - (double)ih);
-    return conj ? dfc{rh, rl, -ih, -il} : dfc{rh, rl, ih, il};
+    const df64 r(v.x), i(v.y);
+    return conj ? dfc{r.hi, r.lo, -i.hi, -i.lo} : dfc{r.hi, r.lo, i.hi, i.lo};
 }
 
 // (sh, sl) += (xh + xl)(yh + yl); the intrinsics keep the compiler from contracting the steps.
@@ -172,16 +198,30 @@ template <bool CA, bool CB, int T>
 __global__ void __launch_bounds__(TH, 2)
 k_gemm_df(int m, int n, int K, int kchunk, double alpha, const z64 *__restrict__ A, int lda,
           const z64 *__restrict__ B, int ldb, double beta, const z64 *C, int ldc, z64 *D, int ldd,
-          z64 *__restrict__ part, int lower) {
+          z64 *__restrict__ part, int form, GemmBatch bt) {
     constexpr int BM = 16 * T, BN = 16 * T;
     __shared__ dfc As[BK][BM + 1];
     __shared__ dfc Bs[BK][BN + 1];
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
     const int i0 = blockIdx.x * BM, j0 = blockIdx.y * BN;
-    if (lower && blockIdx.x < blockIdx.y) return;
-    const int kbeg = blockIdx.z * kchunk;
-    const int kend = min(K, kbeg + kchunk);
+    if ((form & kLowerOut) && blockIdx.x < blockIdx.y) return;
+    int kbeg = blockIdx.z * kchunk;
+    if (bt.count) {   // as in k_gemm
+        const int z = blockIdx.z;
+        A += z * bt.a;
+        B += z * bt.b;
+        C += z * bt.c;
+        D += z * bt.c;
+        if (z == bt.count - 1) {
+            m = bt.mlast;
+            K = bt.klast;
+        }
+        kbeg = 0;
+        if (i0 >= m) return;
+    }
+    int kend = min(K, kbeg + kchunk);
+    tri_range<CA, BM, BN>(form, i0, j0, kbeg, kend);
     dfc acc[T][T];
 #pragma unroll
     for (int i = 0; i < T; ++i)
@@ -237,24 +277,33 @@ k_gemm_df(int m, int n, int K, int kchunk, double alpha, const z64 *__restrict__
                 df_norm(acc[i][j].ih, acc[i][j].il);
             }
     }
+    // two loops: an FP64 instruction that is predicated off costs its 64 cycles all the same
+    auto out = [&](auto put) {
 #pragma unroll
-    for (int j = 0; j < T; ++j) {
-        const int gj = j0 + ty + 16 * j;
-        if (gj >= n) continue;
+        for (int j = 0; j < T; ++j) {
+            const int gj = j0 + ty + 16 * j;
+            if (gj >= n) continue;
 #pragma unroll
-        for (int i = 0; i < T; ++i) {
-            const int gi = i0 + tx + 16 * i;
-            if (gi >= m) continue;
-            const dfc &c = acc[i][j];
-            const z64 t = mkc((double)c.rh + (double)c.rl, (double)c.ih + (double)c.il);
-            if (part) {
-                part[((size_t)blockIdx.z * n + gj) * m + gi] = t;
-            } else {
-                z64 v = alpha * t;
-                if (beta != 0.0) v = v + beta * C[(size_t)gj * ldc + gi];
-                D[(size_t)gj * ldd + gi] = v;
+            for (int i = 0; i < T; ++i) {
+                const int gi = i0 + tx + 16 * i;
+                if (gi >= m) continue;
+                const dfc &c = acc[i][j];
+                put(gi, gj, mkc((double)df64(c.rh, c.rl), (double)df64(c.ih, c.il)));
             }
         }
+    };
+    if (part) {
+        out([&](int gi, int gj, z64 t) { part[((size_t)blockIdx.z * n + gj) * m + gi] = t; });
+    } else if (alpha == 1.0 && beta == 0.0) {
+        out([&](int gi, int gj, z64 t) { D[(size_t)gj * ldd + gi] = t; });
+    } else if (alpha == -1.0 && beta == 0.0) {
+        out([&](int gi, int gj, z64 t) { D[(size_t)gj * ldd + gi] = mkc(-t.x, -t.y); });
+    } else {
+        out([&](int gi, int gj, z64 t) {
+            z64 v = alpha * t;
+            if (beta != 0.0) v = v + beta * C[(size_t)gj * ldc + gi];
+            D[(size_t)gj * ldd + gi] = v;
+        });
     }
 }
 
@@ -290,12 +339,12 @@ int num_sms() {
 template <typename R, bool CA, bool CB, int T, bool DF = false>
 int launch_gemm_t(GemmWork *w, int m, int n, int K, R alpha, const cx<R> *A, int lda, const cx<R> *B, int ldb,
                   R beta, const cx<R> *C, int ldc, cx<R> *D, int ldd, cudaStream_t s, bool allow_split,
-                  int min_chunk, bool lower) {
+                  int min_chunk, int form) {
     constexpr int BM = 16 * T, BN = 16 * T;
     if (m <= 0 || n <= 0) return LOBPCG_OK;
     const int tm = (m + BM - 1) / BM, tn = (n + BN - 1) / BN;
     int tiles = tm * tn;
-    if (lower) {  // tiles on or below the diagonal
+    if (form & kLowerOut) {  // tiles on or below the diagonal
         tiles = 0;
         for (int tj = 0; tj < tn; ++tj) tiles += std::max(0, tm - tj);
     }
@@ -313,10 +362,10 @@ int launch_gemm_t(GemmWork *w, int m, int n, int K, R alpha, const cx<R> *A, int
     auto kern = [&](dim3 grid, z64 *part) {
         if constexpr (DF)
             k_gemm_df<CA, CB, T><<<grid, TH, 0, s>>>(m, n, K, kchunk, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd,
-                                                     part, lower ? 1 : 0);
+                                                     part, form, GemmBatch{});
         else
             k_gemm<R, CA, CB, T><<<grid, TH, 0, s>>>(m, n, K, kchunk, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd,
-                                                     part, lower ? 1 : 0);
+                                                     part, form, GemmBatch{});
     };
     if (nsplit == 1) {
         kern(dim3(tm, tn, 1), nullptr);
@@ -329,29 +378,29 @@ int launch_gemm_t(GemmWork *w, int m, int n, int K, R alpha, const cx<R> *A, int
     LG_TRY(check_launch("gemm split"));
     const size_t tot = (size_t)m * n;
     const int blocks = (int)std::min<size_t>((tot + 255) / 256, 4096);
-    k_reduce_parts<R><<<blocks, 256, 0, s>>>(m, n, nsplit, alpha, part, beta, C, ldc, D, ldd, lower ? BM : 0);
+    k_reduce_parts<R><<<blocks, 256, 0, s>>>(m, n, nsplit, alpha, part, beta, C, ldc, D, ldd, (form & kLowerOut) ? BM : 0);
     return check_launch("gemm reduce");
 }
 
 template <typename R, bool CA, bool CB>
 int launch_gemm(GemmWork *w, int m, int n, int K, R alpha, const cx<R> *A, int lda, const cx<R> *B, int ldb,
                 R beta, const cx<R> *C, int ldc, cx<R> *D, int ldd, cudaStream_t s, bool allow_split,
-                bool lower = false) {
+                int form = 0) {
     if constexpr (std::is_same<R, double>::value) {
         if (w && w->df) {  // double-FP32 arithmetic, same tiles and split
             if ((long long)m * n <= 512LL * 512LL && K <= 8192)
                 return launch_gemm_t<R, CA, CB, 2, true>(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s,
-                                                         allow_split, 2 * BK, lower);
+                                                         allow_split, 2 * BK, form);
             return launch_gemm_t<R, CA, CB, 4, true>(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s,
-                                                     allow_split, 4 * BK, lower);
+                                                     allow_split, 4 * BK, form);
         }
     }
     // tall-skinny and large products: 64 x 64 tiles; small dense ones: 32 x 32 tiles + fine split
     if ((long long)m * n <= 512LL * 512LL && K <= 8192)
         return launch_gemm_t<R, CA, CB, 2>(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s, allow_split,
-                                           2 * BK, lower);
+                                           2 * BK, form);
     return launch_gemm_t<R, CA, CB, 4>(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s, allow_split,
-                                       4 * BK, lower);
+                                       4 * BK, form);
 }
 
 }  // namespace
@@ -381,8 +430,8 @@ int zgemm_cn_lower(GemmWork &w, int n, int K, const z64 *A, int lda, const z64 *
     if (df && w.oz) return oz_gemm_cn(w, n, n, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, s, true);
     if (df)
         return launch_gemm_t<double, true, false, 4, true>(&w, n, n, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, C, ldc, s,
-                                                          true, 4 * BK, true);
-    return launch_gemm<double, true, false>(&w, n, n, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, C, ldc, s, true, true);
+                                                          true, 4 * BK, kLowerOut);
+    return launch_gemm<double, true, false>(&w, n, n, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, C, ldc, s, true, kLowerOut);
 }
 
 int zgemm_cn_df(GemmWork &w, int m, int n, int K, double alpha, const z64 *A, int lda, const z64 *B, int ldb,
@@ -390,7 +439,7 @@ int zgemm_cn_df(GemmWork &w, int m, int n, int K, double alpha, const z64 *A, in
     if (m <= 0 || n <= 0) return LOBPCG_OK;
     if (w.oz) return oz_gemm_cn(w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, s, false);
     return launch_gemm_t<double, true, false, 4, true>(&w, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, C, ldc, s,
-                                                      true, 4 * BK, false);
+                                                      true, 4 * BK, 0);
 }
 
 int zgemm_nn_df(GemmWork *w, int M, int n, int k, double alpha, const z64 *A, int lda, const z64 *B, int ldb,
@@ -398,7 +447,7 @@ int zgemm_nn_df(GemmWork *w, int M, int n, int k, double alpha, const z64 *A, in
     if (M <= 0 || n <= 0) return LOBPCG_OK;
     if (w && w->oz && k > 0) return oz_gemm_nn(*w, M, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s);
     return launch_gemm_t<double, false, false, 4, true>(nullptr, M, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D,
-                                                       ldd, s, false, 4 * BK, false);
+                                                       ldd, s, false, 4 * BK, 0);
 }
 
 template <typename R>
@@ -411,21 +460,43 @@ int gemm_nn(int M, int n, int k, R alpha, const cx<R> *A, int lda, const cx<R> *
     return launch_gemm<R, false, false>(nullptr, M, n, k, alpha, A, lda, B, ldb, beta, C, ldc, D, ldd, s, false);
 }
 
+// D = alpha A B for every product of the batch (32 x 32 tiles, no split).
+template <typename R>
+int gemm_batch(GemmWork &w, int m, int n, int k, double alpha, const cx<R> *A, int lda, const cx<R> *B, int ldb,
+               cx<R> *D, int ldd, const GemmBatch &b, cudaStream_t s) {
+    const dim3 grid((m + 31) / 32, (n + 31) / 32, b.count);
+    const int kchunk = (k + BK - 1) / BK * BK;
+    if constexpr (std::is_same<R, double>::value) {
+        if (w.df) {
+            k_gemm_df<false, false, 2><<<grid, TH, 0, s>>>(m, n, k, kchunk, alpha, A, lda, B, ldb, 0.0, D, ldd, D, ldd,
+                                                           nullptr, 0, b);
+            return check_launch("gemm batch");
+        }
+    }
+    k_gemm<R, false, false, 2><<<grid, TH, 0, s>>>(m, n, k, kchunk, (R)alpha, A, lda, B, ldb, (R)0, D, ldd, D, ldd, nullptr,
+                                                   0, b);
+    return check_launch("gemm batch");
+}
+template int gemm_batch<double>(GemmWork &, int, int, int, double, const z64 *, int, const z64 *, int, z64 *, int,
+                                const GemmBatch &, cudaStream_t);
+template int gemm_batch<float>(GemmWork &, int, int, int, double, const c32 *, int, const c32 *, int, c32 *, int,
+                               const GemmBatch &, cudaStream_t);
+
 template <typename R>
 int gemm_small(GemmWork *w, char opA, char opB, int m, int n, int k, double alpha, const cx<R> *A, int lda,
-               const cx<R> *B, int ldb, double beta, cx<R> *C, int ldc, cudaStream_t s) {
+               const cx<R> *B, int ldb, double beta, cx<R> *C, int ldc, cudaStream_t s, int form) {
     const bool ca = (opA == 'C'), cb = (opB == 'C');
     const bool sp = w != nullptr;
     const R al = (R)alpha, be = (R)beta;
-    if (!ca && !cb) return launch_gemm<R, false, false>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp);
-    if (ca && !cb) return launch_gemm<R, true, false>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp);
-    if (!ca && cb) return launch_gemm<R, false, true>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp);
-    return launch_gemm<R, true, true>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp);
+    if (!ca && !cb) return launch_gemm<R, false, false>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp, form);
+    if (ca && !cb) return launch_gemm<R, true, false>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp, form);
+    if (!ca && cb) return launch_gemm<R, false, true>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp, form);
+    return launch_gemm<R, true, true>(w, m, n, k, al, A, lda, B, ldb, be, C, ldc, C, ldc, s, sp, form);
 }
 template int gemm_small<double>(GemmWork *, char, char, int, int, int, double, const z64 *, int, const z64 *, int,
-                                double, z64 *, int, cudaStream_t);
+                                double, z64 *, int, cudaStream_t, int);
 template int gemm_small<float>(GemmWork *, char, char, int, int, int, double, const c32 *, int, const c32 *, int,
-                               double, c32 *, int, cudaStream_t);
+                               double, c32 *, int, cudaStream_t, int);
 
 int zgemm_small(GemmWork *w, char opA, char opB, int m, int n, int k, double alpha, const z64 *A, int lda,
                 const z64 *B, int ldb, double beta, z64 *C, int ldc, cudaStream_t s) {

@@ -290,10 +290,23 @@ template <typename R>
 int gemm_nn(int M, int n, int k, R alpha, const cx<R> *A, int lda, const cx<R> *B, int ldb, R beta,
             const cx<R> *C, int ldc, cx<R> *D, int ldd, cudaStream_t s);
 // Small general complex128 product: C = alpha op(A) op(B) + beta C, op in {'N','C'}.
-// Small general complex product in precision R; w (nullable) enables a split of the reduction dimension.
+// Small general complex product in precision R; w (nullable) enables a split of the reduction dimension;
+// form: what the operands and the output are known to be (the sum skips zeros tile by tile).
+constexpr int kLowerOut = 1;   // output tiles strictly above the diagonal are left as they are
+constexpr int kTriA = 2;       // the stored A is lower triangular
+constexpr int kTriB = 4;       // the stored B is lower triangular, op(B) = B^H
 template <typename R>
 int gemm_small(GemmWork *w, char opA, char opB, int m, int n, int k, double alpha, const cx<R> *A, int lda,
-               const cx<R> *B, int ldb, double beta, cx<R> *C, int ldc, cudaStream_t s);
+               const cx<R> *B, int ldb, double beta, cx<R> *C, int ldc, cudaStream_t s, int form = 0);
+// Products of one shape in one launch: element strides between them, and the rows and the
+// reduction of the last one (count = 0: a single product).
+struct GemmBatch {
+    long long a = 0, b = 0, c = 0;
+    int count = 0, mlast = 0, klast = 0;
+};
+template <typename R>
+int gemm_batch(GemmWork &w, int m, int n, int k, double alpha, const cx<R> *A, int lda, const cx<R> *B, int ldb,
+               cx<R> *D, int ldd, const GemmBatch &b, cudaStream_t s);
 // w (nullable) enables a split of the reduction dimension.
 int zgemm_small(GemmWork *w, char opA, char opB, int m, int n, int k, double alpha, const z64 *A, int lda,
                 const z64 *B, int ldb, double beta, z64 *C, int ldc, cudaStream_t s);

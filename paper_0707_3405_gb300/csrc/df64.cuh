@@ -21,7 +21,54 @@
 
 #include <cuda_runtime.h>
 
+#include <cstdint>
+
 namespace lg {
+
+// hi + lo as an FP64 number, rounded to nearest, in integer arithmetic: a warp-wide FP64 instruction
+// occupies its sub-partition for 64 cycles on this GPU.  (hi, lo) is normalised (|lo| at most half a
+// unit in the last place of hi).  With e the exponent of hi, hi = mh 2^(e - 23) and lo, in units of
+// 2^(e - 52), is an integer of at most 2^28 once rounded; their sum is the mantissa up to one
+// renormalisation (a power of two less something).
+__device__ __forceinline__ double pair_to_double(float hi, float lo) {
+    // tiny and huge numbers by 2^64 or 2^-64, exactly, into the middle of the exponent range
+    const uint32_t b0 = (__float_as_uint(hi) >> 23) & 255u;
+    const float fac = b0 < 64u ? 0x1p64f : b0 > 190u ? 0x1p-64f : 1.f;
+    const int adj = b0 < 64u ? -64 : b0 > 190u ? 64 : 0;
+    const uint32_t u = __float_as_uint(hi * fac), be = (u >> 23) & 255u;
+    // lo 2^(52 - e) as two exact factors, e = be - 127
+    const float f = (u >> 31 ? -lo : lo) * fac * __uint_as_float((254u - be) << 23) * 0x1p52f;
+    unsigned long long m = ((unsigned long long)((u & 0x7FFFFFu) | 0x800000u) << 29) + (long long)__float2int_rn(f);
+    const uint32_t under = (m >> 52) == 0 ? 1u : 0u;            // hi a power of two and lo against it
+    m <<= under;
+    uint32_t top = (be - under + (uint32_t)(adj + 1023 - 127 - 1)) << 20;   // the leading one adds the exponent
+    if (be == 0) { m = 0; top = 0; }                             // zero
+    if (be == 255) { m = (unsigned long long)(u & 0x7FFFFFu) << 29; top = 0x7FF00000u; }   // infinite, not a number
+    return __hiloint2double((int)((top + (uint32_t)(m >> 32)) | (u & 0x80000000u)), (int)(uint32_t)m);
+}
+
+// The pair of an FP64 number, hi = x rounded to nearest and lo = x - hi likewise, in integer arithmetic
+// for the same reason (and with no FP64 instruction in a rare branch: predicated off it costs the
+// same): the 53-bit mantissa is cut into 24 bits, rounded, and the signed rest.  Numbers whose low
+// part would leave the FP32 range are brought into it by 2^64 or 2^-64; below 2^-138 they are zero.
+__device__ __forceinline__ void double_to_pair(double x, float &hi, float &lo) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);   // (folds for constants)
+    const uint32_t top = (uint32_t)(b >> 32), sign = top & 0x80000000u;
+    const int e0 = (int)((top >> 20) & 0x7FFu) - 1023;
+    const int e = e0 < -74 ? e0 + 64 : e0 > 126 ? e0 - 64 : e0;
+    const float fac = e0 < -74 ? 0x1p-64f : e0 > 126 ? 0x1p64f : 1.f;
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
+    const uint32_t mh = (uint32_t)((m + (1ULL << 28)) >> 29);                       // in [2^23, 2^24]
+    const int ml = (int)(uint32_t)((uint32_t)m - (mh << 29));                       // in [-2^28, 2^28], mod 2^32
+    hi = __uint_as_float((((uint32_t)(e + 126) << 23) + mh) | sign) * fac;           // the leading one adds the exponent
+    lo = (float)ml * __uint_as_float(((uint32_t)(e - 52 + 127) << 23) | sign) * fac;
+    if (e < -74) hi = lo = 0.f;
+    if (e > 126) {   // beyond FP32's range, infinite or not a number
+        const bool nan = e0 == 1024 && (b & 0xFFFFFFFFFFFFFULL) != 0;
+        hi = __uint_as_float((nan ? 0x7FC00000u : 0x7F800000u) | sign);
+        lo = 0.f;
+    }
+}
 
 struct alignas(8) df64 {
     float hi, lo;
@@ -32,10 +79,20 @@ struct alignas(8) df64 {
     __host__ __device__ __forceinline__ df64(int i) : df64((double)i) {}
     __host__ __device__ __forceinline__ df64(unsigned int i) : df64((double)i) {}
     __host__ __device__ __forceinline__ df64(double d) {
+#ifdef __CUDA_ARCH__
+        double_to_pair(d, hi, lo);
+#else
         hi = (float)d;
         lo = (float)(d - (double)hi);
+#endif
     }
-    __host__ __device__ __forceinline__ explicit operator double() const { return (double)hi + (double)lo; }
+    __host__ __device__ __forceinline__ explicit operator double() const {
+#ifdef __CUDA_ARCH__
+        return pair_to_double(hi, lo);
+#else
+        return (double)hi + (double)lo;
+#endif
+    }
 
     // ---- error-free transformations
     static __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -159,10 +216,20 @@ struct alignas(8) df64f {
     __host__ __device__ __forceinline__ df64f(float f) : hi(f), lo(0.f) {}
     __host__ __device__ __forceinline__ df64f(int i) : df64f((double)i) {}
     __host__ __device__ __forceinline__ df64f(double d) {
+#ifdef __CUDA_ARCH__
+        double_to_pair(d, hi, lo);
+#else
         hi = (float)d;
         lo = (float)(d - (double)hi);
+#endif
     }
-    __host__ __device__ __forceinline__ explicit operator double() const { return (double)hi + (double)lo; }
+    __host__ __device__ __forceinline__ explicit operator double() const {
+#ifdef __CUDA_ARCH__
+        return pair_to_double(hi, lo);
+#else
+        return (double)hi + (double)lo;
+#endif
+    }
 
     friend __device__ __forceinline__ df64f operator-(df64f a) { return df64f(-a.hi, -a.lo); }
     friend __device__ __forceinline__ df64f operator+(df64f a, df64f b) {

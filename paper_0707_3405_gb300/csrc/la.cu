@@ -96,6 +96,16 @@ __device__ RT block_sum(RT v, RT *sh) {
     return t;
 }
 
+// acc + a b
+template <typename CT>
+__device__ __forceinline__ cx<CT> cmac(cx<CT> acc, cx<CT> a, cx<CT> b) {
+    CT re = fma(a.x, b.x, acc.x);
+    re = fma(-a.y, b.y, re);
+    CT im = fma(a.x, b.y, acc.y);
+    im = fma(a.y, b.x, im);
+    return mkc<CT>(re, im);
+}
+
 // ------------------------------------------------------------------ scaling
 template <typename RT>
 __global__ void k_scale_gram(int n, const cx<RT> *__restrict__ S, int lds, const cx<RT> *__restrict__ A, int lda,
@@ -123,35 +133,35 @@ __global__ void k_scale_gram(int n, const cx<RT> *__restrict__ S, int lds, const
 // ------------------------------------------------------------------ Cholesky with dropping
 // Factor the kb x kb diagonal block at k0 (already updated by earlier panels),
 // write L_kk over it and its inverse into Linv.
-// CT: compute type (double-FP32 where one SM's FP64 units would be the limit).
-template <typename RT, typename CT = RT>
+// (FP64 and FP32 arithmetic.  The FP64 schedule's steps on nearly dependent bases follow the exact
+// roundings of this form; the elimination form below gained nothing there, the FP64 units bounding both.)
+template <typename RT>
 __global__ void __launch_bounds__(256)
-k_chol_diag(int n, int k0, int kb, cx<RT> *__restrict__ L, cx<RT> *__restrict__ Linv, RT drop_tol_in,
+k_chol_diag(int n, int k0, int kb, cx<RT> *__restrict__ L, cx<RT> *__restrict__ Linv, RT drop_tol,
             int *__restrict__ dropped, int *__restrict__ ndrop) {
-    __shared__ cx<CT> T[NBK][NBK + 1];
-    __shared__ cx<CT> I[NBK][NBK + 1];
+    __shared__ cx<RT> T[NBK][NBK + 1];
+    __shared__ cx<RT> I[NBK][NBK + 1];
     __shared__ int dflag[NBK];
-    const CT drop_tol = (CT)drop_tol_in;
     const int tid = threadIdx.x;
     for (int e = tid; e < NBK * NBK; e += blockDim.x) {
         const int r = e % NBK, c = e / NBK;
-        cx<CT> v = mkc<CT>(0.0, 0.0);
-        if (r < kb && c < kb && r >= c) v = ld_as<CT>(L + (size_t)(k0 + c) * n + k0 + r);
+        cx<RT> v = mkc<RT>(0.0, 0.0);
+        if (r < kb && c < kb && r >= c) v = L[(size_t)(k0 + c) * n + k0 + r];
         T[r][c] = v;
-        I[r][c] = mkc<CT>(0.0, 0.0);
+        I[r][c] = mkc<RT>(0.0, 0.0);
     }
     __syncthreads();
     for (int j = 0; j < kb; ++j) {
-        const CT p = T[j][j].x;
+        const RT p = T[j][j].x;
         const bool drop = !(p > drop_tol);
         __syncthreads();
         if (drop) {
-            for (int r = j + 1 + tid; r < kb; r += blockDim.x) T[r][j] = mkc<CT>(0.0, 0.0);
-            if (tid == 0) { T[j][j] = mkc<CT>(1.0, 0.0); dflag[j] = 1; }
+            for (int r = j + 1 + tid; r < kb; r += blockDim.x) T[r][j] = mkc<RT>(0.0, 0.0);
+            if (tid == 0) { T[j][j] = mkc<RT>(1.0, 0.0); dflag[j] = 1; }
         } else {
-            const CT rt = sqrt(p), inv = (CT)1.0 / rt;
+            const RT rt = sqrt(p), inv = (RT)1.0 / rt;
             for (int r = j + 1 + tid; r < kb; r += blockDim.x) T[r][j] = inv * T[r][j];
-            if (tid == 0) { T[j][j] = mkc<CT>(rt, 0.0); dflag[j] = 0; }
+            if (tid == 0) { T[j][j] = mkc<RT>(rt, 0.0); dflag[j] = 0; }
         }
         __syncthreads();
         if (!drop) {
@@ -166,20 +176,20 @@ k_chol_diag(int n, int k0, int kb, cx<RT> *__restrict__ L, cx<RT> *__restrict__ 
     // clear the rows of dropped columns inside the block
     for (int e = tid; e < kb * kb; e += blockDim.x) {
         const int r = e % kb, c = e / kb;
-        if (c < r && dflag[r]) T[r][c] = mkc<CT>(0.0, 0.0);
+        if (c < r && dflag[r]) T[r][c] = mkc<RT>(0.0, 0.0);
     }
     __syncthreads();
     // inverse of the lower-triangular block (real positive diagonal) by forward substitution,
     // column c on the 8 lanes of one warp segment: I[r][c] = -(1 / T[r][r]) sum_{l=c}^{r-1} T[r][l] I[l][c],
     // each lane taking every 8th l, the segment adding its partial sums by shuffles (fixed order)
-    __shared__ CT rdiag[NBK];
-    if (tid < kb) rdiag[tid] = (CT)1.0 / T[tid][tid].x;
+    __shared__ RT rdiag[NBK];
+    if (tid < kb) rdiag[tid] = (RT)1.0 / T[tid][tid].x;
     __syncthreads();
     {
         const int c = tid >> 3, sub = tid & 7;
         const bool on = c < kb;
         for (int r = 0; r < kb; ++r) {
-            cx<CT> sacc = mkc<CT>(0.0, 0.0);
+            cx<RT> sacc = mkc<RT>(0.0, 0.0);
             if (on && c < r)
                 for (int l = c + sub; l < r; l += 8) sacc = sacc + T[r][l] * I[l][c];
 #pragma unroll
@@ -189,7 +199,7 @@ k_chol_diag(int n, int k0, int kb, cx<RT> *__restrict__ L, cx<RT> *__restrict__ 
             }
             if (on && sub == 0) {
                 if (c < r) I[r][c] = (-rdiag[r]) * sacc;
-                else if (c == r) I[r][r] = mkc<CT>(rdiag[r], 0.0);
+                else if (c == r) I[r][r] = mkc<RT>(rdiag[r], 0.0);
             }
             __syncwarp();
         }
@@ -197,8 +207,8 @@ k_chol_diag(int n, int k0, int kb, cx<RT> *__restrict__ L, cx<RT> *__restrict__ 
     __syncthreads();
     for (int e = tid; e < kb * kb; e += blockDim.x) {
         const int r = e % kb, c = e / kb;
-        L[(size_t)(k0 + c) * n + k0 + r] = (r >= c) ? as_store<RT>(T[r][c]) : mkc<RT>(0.0, 0.0);
-        Linv[(size_t)(k0 + c) * n + k0 + r] = (r >= c) ? as_store<RT>(I[r][c]) : mkc<RT>(0.0, 0.0);
+        L[(size_t)(k0 + c) * n + k0 + r] = (r >= c) ? T[r][c] : mkc<RT>(0.0, 0.0);
+        Linv[(size_t)(k0 + c) * n + k0 + r] = (r >= c) ? I[r][c] : mkc<RT>(0.0, 0.0);
     }
     if (tid < kb) {
         dropped[k0 + tid] = dflag[tid];
@@ -206,20 +216,90 @@ k_chol_diag(int n, int k0, int kb, cx<RT> *__restrict__ L, cx<RT> *__restrict__ 
     }
 }
 
-// Panel: L21 = S21 Linv_kk^H for rows k0+kb..n-1 (8 rows per block, 32 columns).
-template <typename RT>
+// The same in double-FP32 (one SM's FP64 units would be the limit).  Elimination in the form Lu D Lu^H with the identity beside it: column j's pivot p, m_r = T[r][j] / p, then
+// T[r][c] -= m_r conj(T[c][j]) for j < c <= r and I[r][c] -= m_r I[j][c] for c <= j, so that the
+// inverse of Lu grows in the same step.  A step is one division, one multiply-add and one block
+// barrier; the square roots come once at the end, for all columns together (L = Lu D^1/2).  A chain
+// of 32 steps is what bounds it: double-FP32 52 -> 31 us per block, against
+// square root, column scaling, update and a separate forward substitution.
 __global__ void __launch_bounds__(256)
+k_chol_diag_df(int n, int k0, int kb, z64 *__restrict__ L, z64 *__restrict__ Linv, double drop_tol_in,
+               int *__restrict__ dropped, int *__restrict__ ndrop) {
+    using CT = df64;
+    __shared__ cx<CT> T[NBK][NBK + 1];
+    __shared__ cx<CT> I[NBK][NBK + 1];
+    __shared__ CT rs[NBK];     // 1 / sqrt(pivot)
+    __shared__ int dflag[NBK];
+    const CT drop_tol = (CT)drop_tol_in;
+    const int tid = threadIdx.x, r = tid & (NBK - 1), w = tid / NBK;   // a thread has row r, columns w, w + 8, ...
+    const cx<CT> zero = mkc<CT>(0.0, 0.0);
+#pragma unroll
+    for (int k = 0; k < NBK / 8; ++k) {
+        const int c = w + 8 * k;
+        T[r][c] = (r < kb && r >= c) ? ld_as<CT>(L + (size_t)(k0 + c) * n + k0 + r) : zero;
+        I[r][c] = mkc<CT>(r == c ? 1.0 : 0.0, 0.0);
+    }
+    __syncthreads();
+    for (int j = 0; j < kb; ++j) {
+        const CT p = T[j][j].x;
+        const bool drop = !(p > drop_tol);
+        if (tid == 0) dflag[j] = drop;
+        if (drop) {            // row and column j become those of the identity
+            if (r == j)
+                for (int c = w; c < j; c += 8) I[j][c] = zero;
+        } else if (r > j && r < kb) {
+            const cx<CT> mm = ((CT)-1.0 / p) * T[r][j];
+#pragma unroll
+            for (int k = 0; k < NBK / 8; ++k) {
+                const int c = w + 8 * k;
+                if (c > r) continue;
+                cx<CT> *e = c > j ? &T[r][c] : &I[r][c];
+                *e = cmac(*e, mm, c > j ? conjc(T[c][j]) : I[j][c]);
+            }
+        }
+        __syncthreads();
+    }
+    if (tid < kb) {
+        const CT p = T[tid][tid].x;
+        rs[tid] = dflag[tid] ? CT(1.0) : (CT)1.0 / sqrt(p);
+        dropped[k0 + tid] = dflag[tid];
+        if (dflag[tid]) atomicAdd(ndrop, 1);
+    }
+    __syncthreads();
+    if (r < kb)
+#pragma unroll
+        for (int k = 0; k < NBK / 8; ++k) {
+            const int c = w + 8 * k;
+            if (c >= kb) continue;
+            cx<CT> l = zero, li = zero;
+            if (r == c) {
+                l = mkc<CT>(dflag[c] ? CT(1.0) : rs[c] * T[c][c].x, 0.0);
+                li = mkc<CT>(rs[c], 0.0);
+            } else if (r > c) {
+                if (!dflag[r] && !dflag[c]) l = rs[c] * T[r][c];
+                li = rs[r] * I[r][c];
+            }
+            L[(size_t)(k0 + c) * n + k0 + r] = as_store<double>(l);
+            Linv[(size_t)(k0 + c) * n + k0 + r] = as_store<double>(li);
+        }
+}
+
+// Panel: L21 = S21 Linv_kk^H for rows k0+kb..n-1 (kPanelRows rows per block, 32 columns).  FP64 throughput
+// bounds it: four rows rather than eight per block spread it over twice the SMs (n = 384: 21 -> 13 us).
+constexpr int kPanelRows = 4;
+template <typename RT>
+__global__ void __launch_bounds__(32 * kPanelRows)
 k_chol_panel(int n, int k0, int kb, cx<RT> *__restrict__ L, const cx<RT> *__restrict__ Linv,
              const int *__restrict__ dropped) {
     __shared__ cx<RT> Di[NBK][NBK + 1];
-    __shared__ cx<RT> Srow[8][NBK + 1];
+    __shared__ cx<RT> Srow[kPanelRows][NBK + 1];
     const int tid = threadIdx.x;
     for (int e = tid; e < NBK * NBK; e += blockDim.x) {
         const int r = e % NBK, c = e / NBK;
         Di[r][c] = (r < kb && c < kb) ? Linv[(size_t)(k0 + c) * n + k0 + r] : mkc<RT>(0.0, 0.0);
     }
     const int rl = tid / NBK, c = tid % NBK;
-    const int row = k0 + kb + blockIdx.x * 8 + rl;
+    const int row = k0 + kb + blockIdx.x * kPanelRows + rl;
     if (row < n && c < kb) Srow[rl][c] = L[(size_t)(k0 + c) * n + row];
     __syncthreads();
     if (row < n && c < kb) {
@@ -595,16 +675,6 @@ __device__ __forceinline__ cx<CT> rank2_entry(cx<CT> a, cx<CT> wr, cx<CT> vr, cx
     im = fma(vr.x, wc.y, im);
     return mkc<CT>(re, im);
 }
-// acc + a b
-template <typename CT>
-__device__ __forceinline__ cx<CT> cmac(cx<CT> acc, cx<CT> a, cx<CT> b) {
-    CT re = fma(a.x, b.x, acc.x);
-    re = fma(-a.y, b.y, re);
-    CT im = fma(a.x, b.y, acc.y);
-    im = fma(a.y, b.x, im);
-    return mkc<CT>(re, im);
-}
-
 // The reduction held in the shared memory of one thread-block cluster of CS CTAs, for small
 // matrices (see kTriClusterMaxN).  CTA q keeps the rows
 // r = q + CS j of the full Hermitian matrix, row-major, so that y = A v needs no reduction
@@ -1794,7 +1864,7 @@ int rayleigh_ritz_t(EigWork &w, int n, int m, const cx<RT> *S, int lds, const cx
         bool chol_done = false;
         if constexpr (std::is_same<RT, double>::value) {
             if (w.df) {  // one block: double-FP32 instead of that SM's FP64 units
-                k_chol_diag<RT, df64><<<1, 256, 0, s>>>(n, k0, kb, Ss, Li, (RT)drop_tol, dr, nd);
+                k_chol_diag_df<<<1, 256, 0, s>>>(n, k0, kb, Ss, Li, drop_tol, dr, nd);
                 chol_done = true;
             }
         }
@@ -1802,33 +1872,38 @@ int rayleigh_ritz_t(EigWork &w, int n, int m, const cx<RT> *S, int lds, const cx
         LG_TRY(check_launch("cholesky diag"));
         const int rem = n - k0 - kb;
         if (rem > 0) {
-            k_chol_panel<RT><<<(rem + 7) / 8, 256, 0, s>>>(n, k0, kb, Ss, Li, dr);
+            k_chol_panel<RT><<<(rem + kPanelRows - 1) / kPanelRows, 32 * kPanelRows, 0, s>>>(n, k0, kb, Ss, Li, dr);
             LG_TRY(check_launch("cholesky panel"));
             const cx<RT> *L21 = Ss + (size_t)k0 * n + k0 + kb;
             cx<RT> *S22 = Ss + (size_t)(k0 + kb) * n + k0 + kb;
-            LG_TRY(gemm_small<RT>(&w.gw, 'N', 'C', rem, rem, kb, -1.0, L21, n, L21, n, 1.0, S22, n, s));
+            LG_TRY(gemm_small<RT>(&w.gw, 'N', 'C', rem, rem, kb, -1.0, L21, n, L21, n, 1.0, S22, n, s, kLowerOut));
         }
     }
     k_zero_dropped_rows<RT><<<n, 128, 0, s>>>(n, Ss, dr);
     LG_TRY(check_launch("zero dropped rows"));
-    // off-diagonal blocks of L^-1, block row by block row
-    for (int r0 = NBK; r0 < n; r0 += NBK) {
-        const int kb = std::min(NBK, n - r0);
-        // Tm(kb x r0) = L[r0:r0+kb, 0:r0] * Li[0:r0, 0:r0]
-        LG_TRY(gemm_small<RT>(&w.gw, 'N', 'N', kb, r0, r0, 1.0, Ss + r0, n, Li, n, 0.0, Tm, n, s));
-        // Li[r0:r0+kb, 0:r0] = -Li_rr * Tm
-        LG_TRY(gemm_small<RT>(&w.gw, 'N', 'N', kb, r0, kb, -1.0, Li + (size_t)r0 * n + r0, n, Tm, n, 0.0, Li + r0, n, s));
+    // off-diagonal blocks of L^-1 by doubling: with the inverses of two adjacent diagonal blocks of
+    // width h known, the block below the first is -L22^-1 (L21 L11^-1); all pairs of a width in one launch
+    // per product (log2(n / 32) levels instead of n / 32 block rows)
+    for (int h = NBK; h < n; h *= 2) {
+        const int pairs = (n + h - 1) / (2 * h);                       // pairs with a second block
+        const int last = std::min(h, n - (2 * (pairs - 1) + 1) * h);   // its width in the last pair
+        const long long st = 2LL * h * (n + 1);
+        GemmBatch b1{st, st, st, pairs, last, h};
+        LG_TRY(gemm_batch<RT>(w.gw, h, h, h, 1.0, Ss + h, n, Li, n, Tm + h, n, b1, s));
+        GemmBatch b2{st, st, st, pairs, last, last};
+        LG_TRY(gemm_batch<RT>(w.gw, h, h, h, -1.0, Li + (size_t)h * (n + 1), n, Tm + h, n, Li + h, n, b2, s));
     }
-    // Ahat = Li As Li^H
-    LG_TRY(gemm_small<RT>(&w.gw, 'N', 'N', n, n, n, 1.0, Li, n, As, n, 0.0, Tm, n, s));
-    LG_TRY(gemm_small<RT>(&w.gw, 'N', 'C', n, n, n, 1.0, Tm, n, Li, n, 0.0, As, n, s));
+    // Ahat = Li As Li^H (its lower triangle).  Li is lower triangular: the products skip its zeros, and
+    // are a half, a sixth and (below) a half of full ones
+    LG_TRY(gemm_small<RT>(&w.gw, 'N', 'N', n, n, n, 1.0, Li, n, As, n, 0.0, Tm, n, s, kTriA));
+    LG_TRY(gemm_small<RT>(&w.gw, 'N', 'C', n, n, n, 1.0, Tm, n, Li, n, 0.0, As, n, s, kTriB | kLowerOut));
     k_hermitize_rowsum<RT><<<n, 128, 0, s>>>(n, As, dr, rs);
     LG_TRY(check_launch("hermitize"));
     k_set_dropped_diag<RT><<<1, 1024, 0, s>>>(n, As, dr, nd, rs);
     LG_TRY(check_launch("dropped diag"));
     LG_TRY(heev_lowest_t<RT>(w, n, m, As, n, theta, Q, n, s));
     // C = D Li^H Q
-    LG_TRY(gemm_small<RT>(&w.gw, 'C', 'N', n, m, n, 1.0, Li, n, Q, n, 0.0, Tm, n, s));
+    LG_TRY(gemm_small<RT>(&w.gw, 'C', 'N', n, m, n, 1.0, Li, n, Q, n, 0.0, Tm, n, s, kTriA));
     k_scale_rows_copy<RT><<<dim3((n + 127) / 128, m), 128, 0, s>>>(n, m, d, Tm, n, C, ldc);
     LG_TRY(check_launch("scale C"));
     if (ndropped) {

@@ -60,6 +60,7 @@
 //   A^H B  512 x 128 x 113081    2.66 -> 1.64 ms   (0.66 ms of it the split into digits)
 //   Gram   1152, K = 113081      25.8 -> 12.0 ms   (2.7 ms of it the split)
 #include "common.cuh"
+#include "df64.cuh"
 #include "tc.cuh"
 
 #include <algorithm>
@@ -132,28 +133,6 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float x, float y) {
     e += lo + y;
     hi = s + e;
     lo = e - (hi - s);
-}
-
-// hi + lo as an FP64 number, rounded to nearest, in integer arithmetic: a warp-wide FP64 instruction
-// occupies its sub-partition for 64 cycles on this GPU.  (hi, lo) is normalised (|lo| at most half a
-// unit in the last place of hi).  With e the exponent of hi, hi = mh 2^(e - 23) and lo, in units of
-// 2^(e - 52), is an integer of at most 2^28 once rounded; their sum is the mantissa up to one
-// renormalisation (a power of two less something).
-__device__ __forceinline__ double pair_to_double(float hi, float lo) {
-    // tiny and huge numbers by 2^64 or 2^-64, exactly, into the middle of the exponent range
-    const uint32_t b0 = (__float_as_uint(hi) >> 23) & 255u;
-    const float fac = b0 < 64u ? 0x1p64f : b0 > 190u ? 0x1p-64f : 1.f;
-    const int adj = b0 < 64u ? -64 : b0 > 190u ? 64 : 0;
-    const uint32_t u = __float_as_uint(hi * fac), be = (u >> 23) & 255u;
-    // lo 2^(52 - e) as two exact factors, e = be - 127
-    const float f = (u >> 31 ? -lo : lo) * fac * __uint_as_float((254u - be) << 23) * 0x1p52f;
-    unsigned long long m = ((unsigned long long)((u & 0x7FFFFFu) | 0x800000u) << 29) + (long long)__float2int_rn(f);
-    const uint32_t under = (m >> 52) == 0 ? 1u : 0u;            // hi a power of two and lo against it
-    m <<= under;
-    uint32_t top = (be - under + (uint32_t)(adj + 1023 - 127 - 1)) << 20;   // the leading one adds the exponent
-    if (be == 0) { m = 0; top = 0; }                             // zero
-    if (be == 255) { m = (unsigned long long)(u & 0x7FFFFFu) << 29; top = 0x7FF00000u; }   // infinite, not a number
-    return __hiloint2double((int)((top + (uint32_t)(m >> 32)) | (u & 0x80000000u)), (int)(uint32_t)m);
 }
 
 // The six base-256 digits of x relative to the chunk scale 2^e (|x| < 2^e), most significant
