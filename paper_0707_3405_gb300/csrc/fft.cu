@@ -28,6 +28,12 @@
 
 namespace lg {
 
+#define LG_FFT_DF(n)                                                                                              \
+    int fft_df_apply_##n(const FFTGeom &g, const z64 *X, int ldx, z64 *Y, int ldy, int nb, const double *kin,     \
+                         const df64f *vt, const z64 *tw, cx<df64f> *T2, int nbatch, int smem_max, cudaStream_t s);
+LG_FFT_DF(1) LG_FFT_DF(2) LG_FFT_DF(3) LG_FFT_DF(4)
+#undef LG_FFT_DF
+
 bool make_fft_plan(int N, FFTPlan &p, bool allow8) {
     p.N = N;
     p.nstage = 0;
@@ -133,14 +139,10 @@ struct DFT<R, 8> {
 
 // One Stockham stage over `nlines` lines (all butterflies held in registers
 // between the two barriers, so the stage can run in place).
-// NC > 0: the line length and the stage's Ns are the compile-time NC and NSC (constant index
-// arithmetic); NC = 0: the runtime N and Ns.
-template <typename R, int RDX, int VPT, int NC = 0, int NSC = 1>
-__device__ __forceinline__ void fft_stage(cx<R> *buf, int nlines, int ls, int es, int N_, int Ns_,
+template <typename R, int RDX, int VPT>
+__device__ __forceinline__ void fft_stage(cx<R> *buf, int nlines, int ls, int es, int N, int Ns,
                                           const cx<R> *tw, int sg) {
     constexpr int NB = (VPT + RDX - 1) / RDX;
-    const int N = NC ? NC : N_;
-    const int Ns = NC ? NSC : Ns_;
     const int bpl = N / RDX;
     const int total = nlines * bpl;
     const int tstride = N / (Ns * RDX);
@@ -196,46 +198,12 @@ constexpr bool radix8() { return vpt<CT>() == 8; }
 template <typename CT>
 constexpr int plane_threads() { return vpt<CT>() == 4 ? 512 : kThreads; }
 
-// Radix of stage s of the plan make_fft_plan builds for N (0 past the last stage).
-constexpr int plan_radix(int N, bool allow8, int s) {
-    const int pref[5] = {8, 4, 2, 5, 3};
-    int r = N, k = 0;
-    for (int i = 0; i < 5; ++i) {
-        const int f = pref[i];
-        if (f == 8 && !allow8) continue;
-        while (r % f == 0) {
-            if (k == s) return f;
-            r /= f;
-            ++k;
-        }
-    }
-    return 0;
-}
-
-// The stages of a compile-time plan for line length NC, from stage S on (Ns = NS).
-template <typename R, int NC, int S = 0, int NS = 1>
-__device__ __forceinline__ void fft_stages_c(cx<R> *b, int nl, int ls, int es, const cx<R> *tw, int sg) {
-    constexpr int RDX = plan_radix(NC, radix8<R>(), S);
-    if constexpr (RDX != 0) {
-        fft_stage<R, RDX, vpt<R>(), NC, NS>(b, nl, ls, es, NC, NS, tw, sg);
-        fft_stages_c<R, NC, S + 1, NS * RDX>(b, nl, ls, es, tw, sg);
-    }
-}
-
 // In-place FFT of `nlines` lines (line stride ls, element stride es) by the whole block.
-// sg = -1: forward (e^{-i...}); sg = +1: inverse without 1/N.  NC > 0: the plan of a line of
-// NC points unrolled at compile time (plan.N must equal NC); NC = 0: the runtime plan.
-template <typename R, int NC = 0>
+// sg = -1: forward (e^{-i...}); sg = +1: inverse without 1/N.
+template <typename R>
 __device__ void fft_lines(cx<R> *buf, int nlines, int ls, int es, const FFTPlan &plan, const cx<R> *tw, int sg) {
     constexpr int kVPT = vpt<R>();
-    const int N = NC ? NC : plan.N;
-    if constexpr (NC > 0) {
-        int lpg = (int)(blockDim.x * kVPT) / N;
-        if (lpg < 1) lpg = 1;
-        for (int l0 = 0; l0 < nlines; l0 += lpg)
-            fft_stages_c<R, NC>(buf + l0 * ls, min(lpg, nlines - l0), ls, es, tw, sg);
-        return;
-    }
+    const int N = plan.N;
     int lpg = (int)(blockDim.x * kVPT) / N;
     if (lpg < 1) lpg = 1;
     for (int l0 = 0; l0 < nlines; l0 += lpg) {
@@ -266,13 +234,13 @@ __device__ __forceinline__ cx<CT> to_ct(cx<R> v) {
     else return mkc<CT>((CT)v.x, (CT)v.y);
 }
 
-template <typename R, typename CT = R, int NC = 0>
+template <typename R, typename CT = R>
 __global__ void __launch_bounds__(plane_threads<CT>())
 k_pass_a(const cx<R> *__restrict__ X, int ldx, cx<CT> *__restrict__ T2, FFTPlan plan, int Px, int Py, int ny0m,
          const int *__restrict__ plane_begin, const int2 *__restrict__ yrange, const int *__restrict__ gmap,
          const cx<R> *__restrict__ twg, int zc_max) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = NC ? NC : plan.N;
+    const int N = plan.N;
     cx<CT> *tw = reinterpret_cast<cx<CT> *>(smem_raw);
     cx<CT> *A = tw + N;
     cx<CT> *L = A + Py * N;
@@ -287,7 +255,7 @@ k_pass_a(const cx<R> *__restrict__ X, int ldx, cx<CT> *__restrict__ T2, FFTPlan 
     for (int g = g0 + threadIdx.x; g < g1; g += blockDim.x) A[gmap[g]] = to_ct<CT>(Xb[g]);
     __syncthreads();
     const int2 yr = yrange[px];
-    fft_lines<CT, NC>(A + yr.x * N, yr.y - yr.x + 1, N, 1, plan, tw, 1);
+    fft_lines<CT>(A + yr.x * N, yr.y - yr.x + 1, N, 1, plan, tw, 1);
     cx<CT> *out = T2 + ((size_t)b * Px + px) * (size_t)N * N;  // [z][y]
     for (int z0 = 0; z0 < N; z0 += zc_max) {
         const int nz = min(zc_max, N - z0);
@@ -298,7 +266,7 @@ k_pass_a(const cx<R> *__restrict__ X, int ldx, cx<CT> *__restrict__ T2, FFTPlan 
             L[zc * lsL + iy] = (py < Py) ? A[py * N + z0 + zc] : zero;
         }
         __syncthreads();
-        fft_lines<CT, NC>(L, nz, lsL, 1, plan, tw, 1);
+        fft_lines<CT>(L, nz, lsL, 1, plan, tw, 1);
         for (int i = threadIdx.x; i < nz * N; i += blockDim.x) {
             const int zc = i / N, iy = i - zc * N;
             out[(size_t)(z0 + zc) * N + iy] = L[zc * lsL + iy];
@@ -307,12 +275,12 @@ k_pass_a(const cx<R> *__restrict__ X, int ldx, cx<CT> *__restrict__ T2, FFTPlan 
     }
 }
 
-template <typename R, typename CT = R, int NC = 0>
+template <typename R, typename CT = R>
 __global__ void __launch_bounds__(plane_threads<CT>())
 k_pass_b(cx<CT> *__restrict__ T2, FFTPlan plan, int Px, int nx0m, const R *__restrict__ vt,
          const CT *__restrict__ vtc, const cx<R> *__restrict__ twg, int yc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = NC ? NC : plan.N;
+    const int N = plan.N;
     cx<CT> *tw = reinterpret_cast<cx<CT> *>(smem_raw);
     cx<CT> *L = tw + N;
     const int lsL = N + 1;
@@ -331,7 +299,7 @@ k_pass_b(cx<CT> *__restrict__ T2, FFTPlan plan, int Px, int nx0m, const R *__res
         L[yy * lsL + ix] = base[(size_t)px * NN + yy];
     }
     __syncthreads();
-    fft_lines<CT, NC>(L, ny, lsL, 1, plan, tw, 1);
+    fft_lines<CT>(L, ny, lsL, 1, plan, tw, 1);
     // V in the compute type: from vtc when given (no conversion), else converted here
     const R *vz = vt + (size_t)z * NN + y0;
     const CT *vcz = vtc ? vtc + (size_t)z * NN + y0 : nullptr;
@@ -341,7 +309,7 @@ k_pass_b(cx<CT> *__restrict__ T2, FFTPlan plan, int Px, int nx0m, const R *__res
         L[yy * lsL + ix] = vv * L[yy * lsL + ix];
     }
     __syncthreads();
-    fft_lines<CT, NC>(L, ny, lsL, 1, plan, tw, -1);
+    fft_lines<CT>(L, ny, lsL, 1, plan, tw, -1);
     for (int i = threadIdx.x; i < Px * ny; i += blockDim.x) {
         const int px = i / ny, yy = i - px * ny;
         int ix = nx0m + px;
@@ -350,14 +318,14 @@ k_pass_b(cx<CT> *__restrict__ T2, FFTPlan plan, int Px, int nx0m, const R *__res
     }
 }
 
-template <typename R, typename CT = R, int NC = 0>
+template <typename R, typename CT = R>
 __global__ void __launch_bounds__(plane_threads<CT>())
 k_pass_c(const cx<CT> *__restrict__ T2, cx<R> *__restrict__ Y, int ldy, const cx<R> *__restrict__ X, int ldx,
          const R *__restrict__ kin, FFTPlan plan, int Px, int Py, int ny0m, const int *__restrict__ plane_begin,
          const int2 *__restrict__ yrange, const int *__restrict__ gmap, const cx<R> *__restrict__ twg,
          int zc_max) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = NC ? NC : plan.N;
+    const int N = plan.N;
     cx<CT> *tw = reinterpret_cast<cx<CT> *>(smem_raw);
     cx<CT> *A = tw + N;
     cx<CT> *L = A + Py * N;
@@ -373,7 +341,7 @@ k_pass_c(const cx<CT> *__restrict__ T2, cx<R> *__restrict__ Y, int ldy, const cx
             L[zc * lsL + iy] = in[(size_t)(z0 + zc) * N + iy];
         }
         __syncthreads();
-        fft_lines<CT, NC>(L, nz, lsL, 1, plan, tw, -1);
+        fft_lines<CT>(L, nz, lsL, 1, plan, tw, -1);
         for (int i = threadIdx.x; i < nz * Py; i += blockDim.x) {
             const int zc = i % nz, py = i / nz;
             int iy = py + ny0m;
@@ -383,7 +351,7 @@ k_pass_c(const cx<CT> *__restrict__ T2, cx<R> *__restrict__ Y, int ldy, const cx
         __syncthreads();
     }
     const int2 yr = yrange[px];
-    fft_lines<CT, NC>(A + yr.x * N, yr.y - yr.x + 1, N, 1, plan, tw, -1);
+    fft_lines<CT>(A + yr.x * N, yr.y - yr.x + 1, N, 1, plan, tw, -1);
     const int g0 = plane_begin[px], g1 = plane_begin[px + 1];
     cx<R> *Yb = Y + (size_t)b * ldy;
     const cx<R> *Xb = X + (size_t)b * ldx;
@@ -491,10 +459,9 @@ size_t fft_smem_need(const FFTGeom &g) {
 
 namespace {
 
-// The three passes over batches of bands; CT is the compute type (see k_pass_a); NC > 0: the
-// kernels compiled for that grid edge.
-template <typename R, typename CT, int NC>
-int fft_passes_n(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx, cx<R> *Y, int ldy, int nb,
+// The three passes over batches of bands; CT is the compute type (see k_pass_a).
+template <typename R, typename CT>
+int fft_passes(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx, cx<R> *Y, int ldy, int nb,
                  const R *kin, const R *vt, const CT *vtc, const cx<R> *tw, cx<CT> *T2, int nbatch, cudaStream_t s) {
     const int N = g.N;
     const int zc = pick_zc<R>(g);
@@ -505,9 +472,9 @@ int fft_passes_n(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx,
     static std::atomic<bool> attr_set{false};
     if (!attr_set.load()) {
         const int lim = max_dyn_smem();
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_a<R, CT, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_b<R, CT, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_c<R, CT, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_a<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_b<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_c<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
         attr_set.store(true);
     }
     const int ny0m = ((g.ny0 % N) + N) % N;
@@ -516,32 +483,16 @@ int fft_passes_n(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx,
         const int nbb = std::min(nbatch, nb - b0);
         const cx<R> *Xb = X + (size_t)b0 * ldx;
         cx<R> *Yb = Y + (size_t)b0 * ldy;
-        k_pass_a<R, CT, NC><<<dim3(g.Px, nbb), plane_threads<CT>(), sm_ac, s>>>(Xb, ldx, T2, plan, g.Px, g.Py, ny0m, g.plane_begin,
+        k_pass_a<R, CT><<<dim3(g.Px, nbb), plane_threads<CT>(), sm_ac, s>>>(Xb, ldx, T2, plan, g.Px, g.Py, ny0m, g.plane_begin,
                                                              g.plane_yrange, g.gmap, tw, zc);
         LG_TRY(check_launch("fft pass A"));
-        k_pass_b<R, CT, NC><<<dim3((N + yc - 1) / yc, N, nbb), plane_threads<CT>(), sm_b, s>>>(T2, plan, g.Px, nx0m, vt, vtc, tw, yc);
+        k_pass_b<R, CT><<<dim3((N + yc - 1) / yc, N, nbb), plane_threads<CT>(), sm_b, s>>>(T2, plan, g.Px, nx0m, vt, vtc, tw, yc);
         LG_TRY(check_launch("fft pass B"));
-        k_pass_c<R, CT, NC><<<dim3(g.Px, nbb), plane_threads<CT>(), sm_ac, s>>>(T2, Yb, ldy, Xb, ldx, kin, plan, g.Px, g.Py, ny0m,
+        k_pass_c<R, CT><<<dim3(g.Px, nbb), plane_threads<CT>(), sm_ac, s>>>(T2, Yb, ldy, Xb, ldx, kin, plan, g.Px, g.Py, ny0m,
                                                              g.plane_begin, g.plane_yrange, g.gmap, tw, zc);
         LG_TRY(check_launch("fft pass C"));
     }
     return LOBPCG_OK;
-}
-
-// Grid edges of the benchmark cells get their own double-FP32 kernels (compile-time plan).
-template <typename R, typename CT>
-int fft_passes(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx, cx<R> *Y, int ldy, int nb,
-               const R *kin, const R *vt, const CT *vtc, const cx<R> *tw, cx<CT> *T2, int nbatch, cudaStream_t s) {
-    if constexpr (std::is_same<CT, df64f>::value) {
-        switch (g.N) {
-            case 72: return fft_passes_n<R, CT, 72>(g, plan, X, ldx, Y, ldy, nb, kin, vt, vtc, tw, T2, nbatch, s);
-            case 96: return fft_passes_n<R, CT, 96>(g, plan, X, ldx, Y, ldy, nb, kin, vt, vtc, tw, T2, nbatch, s);
-            case 120: return fft_passes_n<R, CT, 120>(g, plan, X, ldx, Y, ldy, nb, kin, vt, vtc, tw, T2, nbatch, s);
-            case 160: return fft_passes_n<R, CT, 160>(g, plan, X, ldx, Y, ldy, nb, kin, vt, vtc, tw, T2, nbatch, s);
-            default: break;
-        }
-    }
-    return fft_passes_n<R, CT, 0>(g, plan, X, ldx, Y, ldy, nb, kin, vt, vtc, tw, T2, nbatch, s);
 }
 
 // rho += scale sum_b f_b |psi_b|^2 over batches of bands: pass A then the density pass.
@@ -611,6 +562,14 @@ int fft_vloc_apply(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ld
         if (fft_reg_supported(g.N)) return fft_reg_apply(g, X, ldx, Y, ldy, nb, kin, vt, T2, nbatch, s);
     } else {
         if (df) {  // FP64 data transformed in double-FP32 (the half box holds pairs of floats)
+            if (vt_pair) {  // grid edges with their own kernels (fft_df.cuh): 1 where they do not apply
+                const df64f *vp = reinterpret_cast<const df64f *>(vt_pair);
+                cx<df64f> *t2 = reinterpret_cast<cx<df64f> *>(T2);
+                for (auto f : {fft_df_apply_1, fft_df_apply_2, fft_df_apply_3, fft_df_apply_4}) {
+                    const int rc = f(g, X, ldx, Y, ldy, nb, kin, vp, tw, t2, nbatch, max_dyn_smem(), s);
+                    if (rc <= 0) return rc;
+                }
+            }
             FFTPlan p4;
             if (!make_fft_plan(g.N, p4, false)) return fail(LOBPCG_ERR_UNSUPPORTED, "FFT plan");
             return fft_passes<R, df64f>(g, p4, X, ldx, Y, ldy, nb, kin, vt,
