@@ -1065,7 +1065,6 @@ __device__ void tri_bounds(const RT *__restrict__ d, const RT *__restrict__ e, i
 // (about 5 bits per round).  The FP64 divisions of the Sturm counts are the cost
 // (this GPU has few FP64 units per SM).
 constexpr int kMsLanes = 32;
-constexpr int kMsMaxN = 4096;  // FP32 pre-bracketing copies of d and e^2 (shared memory)
 // FP32 Sturm count on FP32 copies of d and e^2 (shared memory).
 __device__ __forceinline__ int sturm_count32(const float *__restrict__ d, const float *__restrict__ e2, int n, float x,
                                              float pivmin) {
@@ -1081,63 +1080,32 @@ __device__ __forceinline__ int sturm_count32(const float *__restrict__ d, const 
     return c;
 }
 
-// One warp per eigenvalue index k < m, one warp per block so that the m warps spread over
-// the SMs.  FP64 (RT = double): a few cheap FP32 rounds first narrow the bracket.  FP32
-// Sturm counts are exact for a matrix whose entries are within a few FP32 roundings of T
-// (Kahan; Demmel, Dhillon and Ren 1995), so the FP32 bracket widened by a margin well above
-// that perturbation still holds the eigenvalue; the first FP64 round checks it (its end
-// lanes evaluate the two bracket ends) and falls back to the Gershgorin bracket if not.
-template <typename RT>
-__global__ void __launch_bounds__(32)
-k_multisect(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, RT *__restrict__ theta) {
-    const int k = blockIdx.x;
+// FP64 rounds of one eigenvalue index k by a warp, from the bracket [lo, hi] (have: it may be trusted, but
+// is checked by the first round, whose end lanes evaluate its ends) or from [lo_g, hi_g].
+__device__ void multisect_fp64(int n, int k, const double *__restrict__ d, const double *__restrict__ e, bool have,
+                               double lo, double hi, double lo_g, double hi_g, double pivmin,
+                               double *__restrict__ theta) {
     const int sub = threadIdx.x;
-    if (k >= m) return;
-    RT lo, hi, tnorm, pivmin;
-    tri_bounds(d, e, n, lo, hi, tnorm, pivmin);
-    bool check = false;
-    const RT lo_g = lo, hi_g = hi;
-    if constexpr (sizeof(RT) == 8) {
-        __shared__ float ds[kMsMaxN], e2s[kMsMaxN];
-        if (n <= kMsMaxN) {
-            for (int i = sub; i < n; i += kMsLanes) {
-                ds[i] = (float)d[i];
-                e2s[i] = (i + 1 < n) ? (float)(e[i] * e[i]) : 0.f;
-            }
-            __syncwarp();
-            const float tn = (float)tnorm;
-            const float piv = FLT_MIN * fmaxf(1.f, tn * tn);
-            const float margin = 32.f * FLT_EPSILON * tn + 4.f * piv;
-            float l32 = (float)lo, h32 = (float)hi;
-            for (int it = 0; it < 8 && h32 - l32 > 4.f * margin; ++it) {  // warp-uniform
-                const float w = h32 - l32;
-                const float x = l32 + w * (float)(sub + 1) / (float)(kMsLanes + 1);
-                const int c = sturm_count32(ds, e2s, n, x, piv);
-                const unsigned mask = __ballot_sync(0xffffffffu, c <= k);
-                const int T = __popc(mask) - 1;
-                const float xlo = __shfl_sync(0xffffffffu, x, T < 0 ? 0 : T);
-                const float xhi = __shfl_sync(0xffffffffu, x, T < kMsLanes - 1 ? T + 1 : kMsLanes - 1);
-                if (T >= 0) l32 = xlo;
-                if (T < kMsLanes - 1) h32 = xhi;
-            }
-            lo = fmax(lo_g, (RT)l32 - (RT)margin);
-            hi = fmin(hi_g, (RT)h32 + (RT)margin);
-            check = true;
-        }
+    if (!have) {
+        double tnorm;
+        tri_bounds(d, e, n, lo_g, hi_g, tnorm, pivmin);
+        lo = lo_g;
+        hi = hi_g;
     }
+    bool check = have;
     for (int it = 0; it < 32; ++it) {
-        const RT w = hi - lo;
-        if (w <= 2.0 * Lim<RT>::eps() * fmax(fabs(lo), fabs(hi)) + 4.0 * pivmin) break;  // warp-uniform
-        RT x;
+        const double w = hi - lo;
+        if (w <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 4.0 * pivmin) break;  // warp-uniform
+        double x;
         if (check)  // bracket ends on the end lanes, 30 points between
-            x = (sub == 0) ? lo : (sub == kMsLanes - 1) ? hi : lo + w * (RT)sub / (RT)(kMsLanes - 1);
+            x = (sub == 0) ? lo : (sub == kMsLanes - 1) ? hi : lo + w * (double)sub / (double)(kMsLanes - 1);
         else
-            x = lo + w * (RT)(sub + 1) / (RT)(kMsLanes + 1);
+            x = lo + w * (double)(sub + 1) / (double)(kMsLanes + 1);
         const int c = sturm_count(d, e, n, x, pivmin);
         if (check) {
             check = false;
             const bool ok = __shfl_sync(0xffffffffu, c, 0) <= k && __shfl_sync(0xffffffffu, c, kMsLanes - 1) > k;
-            if (!ok) {  // the FP32 bracket missed (not expected): restart from Gershgorin
+            if (!ok) {  // the bracket missed (not expected): restart from Gershgorin
                 lo = lo_g;
                 hi = hi_g;
                 continue;
@@ -1145,12 +1113,38 @@ k_multisect(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, RT
         }
         const unsigned mask = __ballot_sync(0xffffffffu, c <= k);
         const int T = __popc(mask) - 1;  // counts are monotone in sub: lanes 0..T have c <= k
-        const RT xlo = __shfl_sync(0xffffffffu, x, T < 0 ? 0 : T);
-        const RT xhi = __shfl_sync(0xffffffffu, x, T < kMsLanes - 1 ? T + 1 : kMsLanes - 1);
+        const double xlo = __shfl_sync(0xffffffffu, x, T < 0 ? 0 : T);
+        const double xhi = __shfl_sync(0xffffffffu, x, T < kMsLanes - 1 ? T + 1 : kMsLanes - 1);
         if (T >= 0) lo = xlo;
         if (T < kMsLanes - 1) hi = xhi;
     }
     if (sub == 0) theta[k] = 0.5 * (lo + hi);
+}
+
+// FP32 (the complex64 step): one warp per eigenvalue index, one warp per block so that the m warps
+// spread over the SMs.  FP32 Sturm counts are exact for a matrix whose entries are within a few
+// FP32 roundings of T (Kahan; Demmel, Dhillon and Ren 1995); the same holds in each arithmetic
+// below, so a bracket widened by a margin well above that perturbation still holds the
+// eigenvalue in a finer one.
+__global__ void __launch_bounds__(32)
+k_multisect32(int n, int m, const float *__restrict__ d, const float *__restrict__ e, float *__restrict__ theta) {
+    const int k = blockIdx.x, sub = threadIdx.x;
+    if (k >= m) return;
+    float lo, hi, tnorm, pivmin;
+    tri_bounds(d, e, n, lo, hi, tnorm, pivmin);
+    for (int it = 0; it < 32; ++it) {
+        const float w = hi - lo;
+        if (w <= 2.f * FLT_EPSILON * fmaxf(fabsf(lo), fabsf(hi)) + 4.f * pivmin) break;  // warp-uniform
+        const float x = lo + w * (float)(sub + 1) / (float)(kMsLanes + 1);
+        const int c = sturm_count(d, e, n, x, pivmin);
+        const unsigned mask = __ballot_sync(0xffffffffu, c <= k);
+        const int T = __popc(mask) - 1;
+        const float xlo = __shfl_sync(0xffffffffu, x, T < 0 ? 0 : T);
+        const float xhi = __shfl_sync(0xffffffffu, x, T < kMsLanes - 1 ? T + 1 : kMsLanes - 1);
+        if (T >= 0) lo = xlo;
+        if (T < kMsLanes - 1) hi = xhi;
+    }
+    if (sub == 0) theta[k] = 0.5f * (lo + hi);
 }
 
 // Double-FP32 Sturm count on pair copies of d and e^2 (shared memory): the same recurrence,
@@ -1171,9 +1165,15 @@ __device__ __forceinline__ int sturm_count_df(const df64 *__restrict__ d, const 
     return c;
 }
 
-// Multisection of the FP64-class Rayleigh-Ritz step (same rounds as k_multisect): FP32 rounds
-// narrow the bracket, double-FP32 rounds finish it; the bracket bounds come from FP32 copies of
-// T with a generous pad.  Dynamic shared memory: d, e^2 as pairs, then as floats (24 n bytes).
+// Multisection with FP32 rounds, then double-FP32 rounds; the bracket bounds come from FP32 copies of
+// T with a generous pad.  The FP64-class Rayleigh-Ritz step ends there.  FINE64 (FP64 steps): the
+// double-FP32 rounds stop at the perturbation their counts are exact for, the bracket is widened by
+// it, and FP64 rounds, of which the first checks the bracket, finish: three of them instead of eight
+// (an FP64 round is the dear one: n divisions of ten instructions at 64 cycles a warp).  A matrix
+// outside the FP32 range takes FP64 rounds only.  FP64 Rayleigh-Ritz step, m = n / 3:
+//   n = 48 1.08 -> 0.97 ms, 96 2.18 -> 1.99, 200 4.80 -> 4.36.
+// Dynamic shared memory: d, e^2 as pairs, then as floats (24 n bytes).
+template <bool FINE64>
 __global__ void __launch_bounds__(32)
 k_multisect_df(int n, int m, const double *__restrict__ d, const double *__restrict__ e, double *__restrict__ theta) {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1221,9 +1221,11 @@ k_multisect_df(int n, int m, const double *__restrict__ d, const double *__restr
     const df64 lo_g(lo_f), hi_g(hi_f);
     df64 lo = fmax(lo_g, df64(l32) - df64(margin)), hi = fmin(hi_g, df64(h32) + df64(margin));
     bool check = true;
-    const float eps_df = 0x1p-45f;
+    const float eps_df = 0x1p-45f, margin_df = 0x1p-42f * tn + 4.f * piv;
+    const bool in_range = tn < 1e15f && tn > 1e-15f;
     for (int it = 0; it < 40; ++it) {
         const df64 w = hi - lo;
+        if (FINE64 && (!in_range || w.hi <= 4.f * margin_df)) break;
         if (w.hi <= 2.f * eps_df * fmaxf(fabsf(lo.hi), fabsf(hi.hi)) + 4.f * piv) break;  // warp-uniform
         df64 x;
         if (check)  // bracket ends on the end lanes, 30 points between
@@ -1247,7 +1249,12 @@ k_multisect_df(int n, int m, const double *__restrict__ d, const double *__restr
         if (T >= 0) lo = xlo;
         if (T < kMsLanes - 1) hi = xhi;
     }
-    if (sub == 0) theta[k] = (double)((lo + hi) * df64(0.5f));
+    if (!FINE64) {
+        if (sub == 0) theta[k] = (double)((lo + hi) * df64(0.5f));
+        return;
+    }
+    multisect_fp64(n, k, d, e, in_range, (double)lo - (double)margin_df, (double)hi + (double)margin_df, (double)lo_f,
+                   (double)hi_f, DBL_MIN * fmax(1.0, (double)emax2), theta);
 }
 
 // ------------------------------------------------------------------ eigenvectors (inverse iteration)
@@ -1777,20 +1784,15 @@ int heev_lowest_t(EigWork &w, int n, int m, cx<RT> *A, int lda, RT *theta, cx<RT
         k_tri_last<RT><<<1, 32, 0, s>>>(n, A, lda, dg);
         LG_TRY(check_launch("tridiag last"));
     }
-    bool ms_done = false;
     if constexpr (std::is_same<RT, double>::value) {
-        if (w.df) {  // FP64-class path: the fine rounds in double-FP32
-            const size_t smem_ms = 24 * (size_t)n;
-            if (smem_ms > 48 * 1024) LG_TRY(allow_max_dyn_smem((const void *)k_multisect_df));
-            k_multisect_df<<<m, kMsLanes, smem_ms, s>>>(n, m, dg, eg, theta);
-            LG_TRY(check_launch("multisection (double-FP32)"));
-            ms_done = true;
-        }
+        const size_t smem_ms = 24 * (size_t)n;
+        auto ms = w.df ? k_multisect_df<false> : k_multisect_df<true>;
+        if (smem_ms > 48 * 1024) LG_TRY(allow_max_dyn_smem((const void *)ms));
+        ms<<<m, kMsLanes, smem_ms, s>>>(n, m, dg, eg, theta);
+    } else {
+        k_multisect32<<<m, kMsLanes, 0, s>>>(n, m, dg, eg, theta);
     }
-    if (!ms_done) {
-        k_multisect<RT><<<m, kMsLanes, 0, s>>>(n, m, dg, eg, theta);
-        LG_TRY(check_launch("multisection"));
-    }
+    LG_TRY(check_launch("multisection"));
     const size_t smem_ii = 6 * sizeof(RT) * (size_t)n + (size_t)n;
     if (smem_ii > 48 * 1024)
         LG_TRY(allow_max_dyn_smem((const void *)k_inviter<RT>));

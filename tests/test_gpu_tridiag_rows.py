@@ -59,3 +59,17 @@ def test_diagonal_and_zero_columns():
     w, V = w.cpu().numpy(), V.cpu().numpy().T
     assert np.abs(w - np.linalg.eigvalsh(A)).max() < 1e-12 * np.abs(A).sum(1).max()
     assert np.abs(V.conj().T @ V - np.eye(200)).max() < 1e-12
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e14, 1e-14, 1e30, 1e-30])
+def test_heev_scales(scale):
+    # the multisection's FP32 and double-FP32 rounds in and out of their range
+    import torch
+    import paper_0707_3405_gb300 as lg
+    rng = np.random.default_rng(9)
+    A = _herm(rng, 90) * scale
+    w, V = lg.heev(torch.tensor(A.T.copy(), device="cuda"))
+    w, V = w.cpu().numpy(), V.cpu().numpy().T
+    nrm = np.abs(A).sum(1).max()
+    assert np.abs(w - np.linalg.eigvalsh(A)).max() < 1e-13 * nrm
+    assert np.abs(V.conj().T @ V - np.eye(90)).max() < 1e-12
