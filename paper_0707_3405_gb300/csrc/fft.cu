@@ -21,18 +21,13 @@
 // host-computed FP64 table (rounded to the compute precision).
 #include "common.cuh"
 #include "df64.cuh"
+#include "fft_two_step.cuh"
 
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
 
 namespace lg {
-
-#define LG_FFT_DF(n)                                                                                              \
-    int fft_df_apply_##n(const FFTGeom &g, const z64 *X, int ldx, z64 *Y, int ldy, int nb, const double *kin,     \
-                         const df64f *vt, const z64 *tw, cx<df64f> *T2, int nbatch, int smem_max, cudaStream_t s);
-LG_FFT_DF(1) LG_FFT_DF(2) LG_FFT_DF(3) LG_FFT_DF(4)
-#undef LG_FFT_DF
 
 bool make_fft_plan(int N, FFTPlan &p, bool allow8) {
     p.N = N;
@@ -562,11 +557,11 @@ int fft_vloc_apply(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ld
         if (fft_reg_supported(g.N)) return fft_reg_apply(g, X, ldx, Y, ldy, nb, kin, vt, T2, nbatch, s);
     } else {
         if (df) {  // FP64 data transformed in double-FP32 (the half box holds pairs of floats)
-            if (vt_pair) {  // grid edges with their own kernels (fft_df.cuh): 1 where they do not apply
-                const df64f *vp = reinterpret_cast<const df64f *>(vt_pair);
-                cx<df64f> *t2 = reinterpret_cast<cx<df64f> *>(T2);
-                for (auto f : {fft_df_apply_1, fft_df_apply_2, fft_df_apply_3, fft_df_apply_4}) {
-                    const int rc = f(g, X, ldx, Y, ldy, nb, kin, vp, tw, t2, nbatch, max_dyn_smem(), s);
+            if (vt_pair) {  // grid edges with two-step kernels: 1 where they do not apply
+                const Fft2Args<df64f, double> a{&g, X, ldx, Y, ldy, nb, kin, reinterpret_cast<const df64f *>(vt_pair), tw,
+                                                reinterpret_cast<cx<df64f> *>(T2), nbatch, max_dyn_smem(), s};
+                for (auto f : {fft2_df_1, fft2_df_2, fft2_df_3, fft2_df_4}) {
+                    const int rc = f(a);
                     if (rc <= 0) return rc;
                 }
             }
@@ -575,6 +570,11 @@ int fft_vloc_apply(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ld
             return fft_passes<R, df64f>(g, p4, X, ldx, Y, ldy, nb, kin, vt,
                                         reinterpret_cast<const df64f *>(vt_pair), tw, reinterpret_cast<cx<df64f> *>(T2),
                                        nbatch, s);
+        }
+        const Fft2Args<double, double> a{&g, X, ldx, Y, ldy, nb, kin, vt, tw, T2, nbatch, max_dyn_smem(), s};
+        for (auto f : {fft2_f64_1, fft2_f64_2, fft2_f64_3, fft2_f64_4}) {
+            const int rc = f(a);
+            if (rc <= 0) return rc;
         }
     }
     (void)vt_pair;

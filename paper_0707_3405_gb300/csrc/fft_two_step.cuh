@@ -1,4 +1,4 @@
-// Double-FP32 passes of the local potential (Sec. 4.1: Goedecker's zero-padded FFT) for grid edges
+// Double-FP32 and FP64 passes of the local potential (Sec. 4.1: Goedecker's zero-padded FFT) for grid edges
 // N = R1 R2 with both factors small enough for a thread's registers.
 //
 // Same three passes as fft.cu (A: sphere -> z-FFT -> y-FFT, B: x-FFT, V, x-FFT, C: y-FFT -> z-FFT ->
@@ -31,10 +31,33 @@
 #include <atomic>
 
 namespace lg {
-namespace fdf {
+
+// One application of the passes: S the type of the transforms and of the half box T2, R that of the bands.
+template <typename S, typename R>
+struct Fft2Args {
+    const FFTGeom *g;
+    const cx<R> *X;
+    int ldx;
+    cx<R> *Y;
+    int ldy, nb;
+    const R *kin;
+    const S *vt;        // V / N^3 as [z][x][y]
+    const cx<R> *tw;
+    cx<S> *T2;
+    int nbatch, smem_max;
+    cudaStream_t s;
+};
+
+// The passes for the grid edges of one source file each; 1 where they do not apply.
+#define LG_FFT2(n)                                   \
+    int fft2_df_##n(const Fft2Args<df64f, double> &); \
+    int fft2_f64_##n(const Fft2Args<double, double> &);
+LG_FFT2(1) LG_FFT2(2) LG_FFT2(3) LG_FFT2(4)
+#undef LG_FFT2
+
+namespace f2s {
 
 using D = df64f;
-using C = cx<df64f>;
 
 // exact product pieces of two pairs: p + e = a b up to 2^-48 |a b|
 __device__ __forceinline__ void prod(D a, D b, float &p, float &e) {
@@ -64,44 +87,62 @@ __device__ __forceinline__ D dot2_add(D c, D a, D x, D b, D y) {
     df64::fast_two_sum(s2, __fadd_rn(__fadd_rn(t, t2), __fadd_rn(c.lo, __fadd_rn(e, f))), r.hi, r.lo);
     return r;
 }
-__device__ __forceinline__ C cmul(C a, C w) { return mkc<D>(dot2(a.x, w.x, -a.y, w.y), dot2(a.x, w.y, a.y, w.x)); }
-// a conj(w)
-__device__ __forceinline__ C cmulc(C a, C w) { return mkc<D>(dot2(a.x, w.x, a.y, w.y), dot2(a.y, w.x, -a.x, w.y)); }
+// The same sums in plain arithmetic.
+template <typename R>
+__device__ __forceinline__ R dot2(R a, R x, R b, R y) { return fma(a, x, b * y); }
+template <typename R>
+__device__ __forceinline__ R dot2_add(R c, R a, R x, R b, R y) { return fma(a, x, fma(b, y, c)); }
 __device__ __forceinline__ D half(D a) { return D(0.5f * a.hi, 0.5f * a.lo); }
-template <bool INV>
-__device__ __forceinline__ C mul_i(C a) { return INV ? mkc<D>(-a.y, a.x) : mkc<D>(a.y, -a.x); }
-template <bool INV>
-__device__ __forceinline__ C twid(C a, C w) { return INV ? cmulc(a, w) : cmul(a, w); }   // w = W_N^j (forward)
+template <typename R>
+__device__ __forceinline__ R half(R a) { return R(0.5) * a; }
+
+template <typename S>
+__device__ __forceinline__ cx<S> cmul(cx<S> a, cx<S> w) {
+    return mkc<S>(dot2(a.x, w.x, -a.y, w.y), dot2(a.x, w.y, a.y, w.x));
+}
+// a conj(w)
+template <typename S>
+__device__ __forceinline__ cx<S> cmulc(cx<S> a, cx<S> w) {
+    return mkc<S>(dot2(a.x, w.x, a.y, w.y), dot2(a.y, w.x, -a.x, w.y));
+}
+template <bool INV, typename S>
+__device__ __forceinline__ cx<S> mul_i(cx<S> a) { return INV ? mkc<S>(-a.y, a.x) : mkc<S>(a.y, -a.x); }
+template <bool INV, typename S>
+__device__ __forceinline__ cx<S> twid(cx<S> a, cx<S> w) { return INV ? cmulc(a, w) : cmul(a, w); }   // w = W_N^j (forward)
 
 // ------------------------------------------------------------- small transforms in registers
 // P<R, INV>::run(v, tw): v <- DFT_R v; tw: the N-entry table, TS = N / R its stride for W_R.
-template <int R, bool INV, int N>
+template <typename S, int R, bool INV, int N>
 struct P;
-template <bool INV, int N>
-struct P<1, INV, N> {
+template <typename S, bool INV, int N>
+struct P<S, 1, INV, N> {
+    using C = cx<S>;
     static __device__ __forceinline__ void run(C (&)[1], const C *) {}
 };
-template <bool INV, int N>
-struct P<2, INV, N> {
+template <typename S, bool INV, int N>
+struct P<S, 2, INV, N> {
+    using C = cx<S>;
     static __device__ __forceinline__ void run(C (&v)[2], const C *) {
         const C a = v[0], b = v[1];
         v[0] = a + b;
         v[1] = a - b;
     }
 };
-template <bool INV, int N>
-struct P<3, INV, N> {
+template <typename S, bool INV, int N>
+struct P<S, 3, INV, N> {
+    using C = cx<S>;
     static __device__ __forceinline__ void run(C (&v)[3], const C *) {
-        const D s3 = (D)0.86602540378443864676;   // sin(2 pi / 3)
-        const C a = v[0], t1 = v[1] + v[2], t2 = mkc<D>(a.x - half(t1.x), a.y - half(t1.y));
+        const S s3 = (S)0.86602540378443864676;   // sin(2 pi / 3)
+        const C a = v[0], t1 = v[1] + v[2], t2 = mkc<S>(a.x - half(t1.x), a.y - half(t1.y));
         const C t3 = s3 * mul_i<INV>(v[1] - v[2]);
         v[0] = a + t1;
         v[1] = t2 + t3;
         v[2] = t2 - t3;
     }
 };
-template <bool INV, int N>
-struct P<4, INV, N> {
+template <typename S, bool INV, int N>
+struct P<S, 4, INV, N> {
+    using C = cx<S>;
     static __device__ __forceinline__ void run(C (&v)[4], const C *) {
         const C t0 = v[0] + v[2], t1 = v[0] - v[2], t2 = v[1] + v[3], t3 = mul_i<INV>(v[1] - v[3]);
         v[0] = t0 + t2;
@@ -110,17 +151,18 @@ struct P<4, INV, N> {
         v[3] = t1 - t3;
     }
 };
-template <bool INV, int N>
-struct P<5, INV, N> {
+template <typename S, bool INV, int N>
+struct P<S, 5, INV, N> {
+    using C = cx<S>;
     static __device__ __forceinline__ void run(C (&v)[5], const C *) {
-        const D c1 = (D)0.30901699437494742410, c2 = (D)-0.80901699437494742410;   // cos(2 pi / 5), cos(4 pi / 5)
-        const D s1 = (D)0.95105651629515357212, s2 = (D)0.58778525229247312917;    // sin(2 pi / 5), sin(4 pi / 5)
+        const S c1 = (S)0.30901699437494742410, c2 = (S)-0.80901699437494742410;   // cos(2 pi / 5), cos(4 pi / 5)
+        const S s1 = (S)0.95105651629515357212, s2 = (S)0.58778525229247312917;    // sin(2 pi / 5), sin(4 pi / 5)
         const C a = v[0], p = v[1] + v[4], q = v[2] + v[3];
         const C m = mul_i<INV>(v[1] - v[4]), k = mul_i<INV>(v[2] - v[3]);
-        const C r1 = mkc<D>(dot2_add(a.x, c1, p.x, c2, q.x), dot2_add(a.y, c1, p.y, c2, q.y));
-        const C r2 = mkc<D>(dot2_add(a.x, c2, p.x, c1, q.x), dot2_add(a.y, c2, p.y, c1, q.y));
-        const C i1 = mkc<D>(dot2(s1, m.x, s2, k.x), dot2(s1, m.y, s2, k.y));
-        const C i2 = mkc<D>(dot2(s2, m.x, -s1, k.x), dot2(s2, m.y, -s1, k.y));
+        const C r1 = mkc<S>(dot2_add(a.x, c1, p.x, c2, q.x), dot2_add(a.y, c1, p.y, c2, q.y));
+        const C r2 = mkc<S>(dot2_add(a.x, c2, p.x, c1, q.x), dot2_add(a.y, c2, p.y, c1, q.y));
+        const C i1 = mkc<S>(dot2(s1, m.x, s2, k.x), dot2(s1, m.y, s2, k.y));
+        const C i2 = mkc<S>(dot2(s2, m.x, -s1, k.x), dot2(s2, m.y, -s1, k.y));
         v[0] = a + p + q;
         v[1] = r1 + i1;
         v[4] = r1 - i1;
@@ -129,9 +171,10 @@ struct P<5, INV, N> {
     }
 };
 // 8 points; ZIN: v[5..7] are zero; NOUT: outputs 5..7 are not needed.
-template <bool INV, bool ZIN, bool NOUT>
-__device__ __forceinline__ void dft8(C (&v)[8]) {
-    const D h = (D)0.70710678118654752440;   // 1 / sqrt(2)
+template <typename S, bool INV, bool ZIN, bool NOUT>
+__device__ __forceinline__ void dft8(cx<S> (&v)[8]) {
+    using C = cx<S>;
+    const S h = (S)0.70710678118654752440;   // 1 / sqrt(2)
     // even half: 0 2 4 6, odd half: 1 3 5 7
     const C e0 = v[0] + v[4], e1 = v[0] - v[4];
     const C e2 = ZIN ? v[2] : v[2] + v[6], e3 = mul_i<INV>(ZIN ? v[2] : v[2] - v[6]);
@@ -152,9 +195,10 @@ __device__ __forceinline__ void dft8(C (&v)[8]) {
         v[7] = E3 - O3;
     }
 }
-template <bool INV, int N>
-struct P<8, INV, N> {
-    static __device__ __forceinline__ void run(C (&v)[8], const C *) { dft8<INV, false, false>(v); }
+template <typename S, bool INV, int N>
+struct P<S, 8, INV, N> {
+    using C = cx<S>;
+    static __device__ __forceinline__ void run(C (&v)[8], const C *) { dft8<S, INV, false, false>(v); }
 };
 // R = A B, coprime: n = (B n1 + A n2) mod R, k = (B (1/B mod A) k1 + A (1/A mod B) k2) mod R.
 constexpr int inv_mod(int x, int m) {
@@ -162,8 +206,9 @@ constexpr int inv_mod(int x, int m) {
         if ((x % m) * i % m == 1) return i;
     return 1;
 }
-template <int A, int B, bool INV, int N>
-__device__ __forceinline__ void pfa(C (&v)[A * B], const C *tw) {
+template <typename S, int A, int B, bool INV, int N>
+__device__ __forceinline__ void pfa(cx<S> (&v)[A * B], const cx<S> *tw) {
+    using C = cx<S>;
     constexpr int R = A * B, qa = B * inv_mod(B, A), qb = A * inv_mod(A, B);
     C t[R];   // [n1][k2]
 #pragma unroll
@@ -171,7 +216,7 @@ __device__ __forceinline__ void pfa(C (&v)[A * B], const C *tw) {
         C u[B];
 #pragma unroll
         for (int n2 = 0; n2 < B; ++n2) u[n2] = v[(B * n1 + A * n2) % R];
-        P<B, INV, N>::run(u, tw);
+        P<S, B, INV, N>::run(u, tw);
 #pragma unroll
         for (int k2 = 0; k2 < B; ++k2) t[n1 * B + k2] = u[k2];
     }
@@ -180,14 +225,15 @@ __device__ __forceinline__ void pfa(C (&v)[A * B], const C *tw) {
         C u[A];
 #pragma unroll
         for (int n1 = 0; n1 < A; ++n1) u[n1] = t[n1 * B + k2];
-        P<A, INV, N>::run(u, tw);
+        P<S, A, INV, N>::run(u, tw);
 #pragma unroll
         for (int k1 = 0; k1 < A; ++k1) v[(qa * k1 + qb * k2) % R] = u[k1];
     }
 }
 // R = A B by Cooley and Tukey, inner twiddles W_R^{n1 k2} from the table.
-template <int A, int B, bool INV, int N>
-__device__ __forceinline__ void ct(C (&v)[A * B], const C *tw) {
+template <typename S, int A, int B, bool INV, int N>
+__device__ __forceinline__ void ct(cx<S> (&v)[A * B], const cx<S> *tw) {
+    using C = cx<S>;
     constexpr int R = A * B;
     C t[R];
 #pragma unroll
@@ -195,7 +241,7 @@ __device__ __forceinline__ void ct(C (&v)[A * B], const C *tw) {
         C u[B];
 #pragma unroll
         for (int n2 = 0; n2 < B; ++n2) u[n2] = v[n1 + A * n2];
-        P<B, INV, N>::run(u, tw);
+        P<S, B, INV, N>::run(u, tw);
 #pragma unroll
         for (int k2 = 0; k2 < B; ++k2) t[n1 * B + k2] = n1 * k2 ? twid<INV>(u[k2], tw[n1 * k2 * (N / R)]) : u[k2];
     }
@@ -204,29 +250,29 @@ __device__ __forceinline__ void ct(C (&v)[A * B], const C *tw) {
         C u[A];
 #pragma unroll
         for (int n1 = 0; n1 < A; ++n1) u[n1] = t[n1 * B + k2];
-        P<A, INV, N>::run(u, tw);
+        P<S, A, INV, N>::run(u, tw);
 #pragma unroll
         for (int k1 = 0; k1 < A; ++k1) v[k2 + B * k1] = u[k1];
     }
 }
-#define LG_FDF_P(R, expr)                                                                             \
-    template <bool INV, int N>                                                                        \
-    struct P<R, INV, N> {                                                                             \
-        static __device__ __forceinline__ void run(C (&v)[R], const C *tw) { expr; }                 \
+#define LG_FFT2_P(R, expr)                                                                         \
+    template <typename S, bool INV, int N>                                                         \
+    struct P<S, R, INV, N> {                                                                       \
+        static __device__ __forceinline__ void run(cx<S> (&v)[R], const cx<S> *tw) { expr; }       \
     };
-LG_FDF_P(6, (pfa<2, 3, INV, N>(v, tw)))
-LG_FDF_P(9, (ct<3, 3, INV, N>(v, tw)))
-LG_FDF_P(10, (pfa<2, 5, INV, N>(v, tw)))
-LG_FDF_P(12, (pfa<3, 4, INV, N>(v, tw)))
-LG_FDF_P(15, (pfa<3, 5, INV, N>(v, tw)))
-LG_FDF_P(16, (ct<4, 4, INV, N>(v, tw)))
-#undef LG_FDF_P
+LG_FFT2_P(6, (pfa<S, 2, 3, INV, N>(v, tw)))
+LG_FFT2_P(9, (ct<S, 3, 3, INV, N>(v, tw)))
+LG_FFT2_P(10, (pfa<S, 2, 5, INV, N>(v, tw)))
+LG_FFT2_P(12, (pfa<S, 3, 4, INV, N>(v, tw)))
+LG_FFT2_P(15, (pfa<S, 3, 5, INV, N>(v, tw)))
+LG_FFT2_P(16, (ct<S, 4, 4, INV, N>(v, tw)))
+#undef LG_FFT2_P
 
 // The R1-point step: HALF: inputs (inverse) beyond R1 / 2 are zero, outputs (forward) beyond it unneeded.
-template <int R1, bool INV, int N, bool HALF>
-__device__ __forceinline__ void step1(C (&v)[R1], const C *tw) {
-    if constexpr (R1 == 8 && HALF) dft8<INV, INV, !INV>(v);
-    else P<R1, INV, N>::run(v, tw);
+template <typename S, int R1, bool INV, int N, bool HALF>
+__device__ __forceinline__ void step1(cx<S> (&v)[R1], const cx<S> *tw) {
+    if constexpr (R1 == 8 && HALF) dft8<S, INV, INV, !INV>(v);
+    else P<S, R1, INV, N>::run(v, tw);
 }
 
 constexpr int LB = 16;    // lines per block of pass B
@@ -234,22 +280,23 @@ constexpr int LP = 17;    // entries between positions of the line buffer (bank 
 constexpr int TH = 128;   // threads of pass B: four blocks an SM, so that one's barriers overlap the others' work
 constexpr int TP = 512;   // threads of the plane passes, whose tile leaves room for one block
 
-template <int N>
-__device__ __forceinline__ void load_tw(C *tw, const z64 *__restrict__ twg) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = mkc<D>((D)twg[i].x, (D)twg[i].y);
+template <int N, typename S, typename R>
+__device__ __forceinline__ void load_tw(cx<S> *tw, const cx<R> *__restrict__ twg) {
+    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = mkc<S>((S)twg[i].x, (S)twg[i].y);
 }
 
 // ------------------------------------------------------------- pass B
-template <int N, int R1, bool HALF>
+template <typename S, typename R, int N, int R1, bool HALF>
 __global__ void __launch_bounds__(TH, 4)
-k_db(C *__restrict__ T2, int Px, const D *__restrict__ vt, const z64 *__restrict__ twg) {
+k_2b(cx<S> *__restrict__ T2, int Px, const S *__restrict__ vt, const cx<R> *__restrict__ twg) {
+    using C = cx<S>;
     constexpr int R2 = N / R1;
     __shared__ C tw[N];
-    __shared__ C S[N * LP];
+    __shared__ C L[N * LP];
     const int y0 = blockIdx.x * LB, z = blockIdx.y;
     const size_t NN = (size_t)N * N;
     C *base = T2 + (size_t)blockIdx.z * Px * NN + (size_t)z * N + y0;
-    const C zero = mkc<D>(D(0), D(0));
+    const C zero = mkc<S>(S(0), S(0));
     const int ny = min(LB, N - y0);
     load_tw<N>(tw, twg);
     __syncthreads();
@@ -262,24 +309,24 @@ k_db(C *__restrict__ T2, int Px, const D *__restrict__ vt, const z64 *__restrict
             const int px = a + R2 * b;
             v[b] = (HALF && b > R1 / 2) ? zero : px < Px ? base[(size_t)px * NN + l] : zero;
         }
-        step1<R1, true, N, HALF>(v, tw);
+        step1<S, R1, true, N, HALF>(v, tw);
 #pragma unroll
-        for (int k = 0; k < R1; ++k) S[(a + R2 * k) * LP + l] = k ? cmulc(v[k], tw[a * k]) : v[k];
+        for (int k = 0; k < R1; ++k) L[(a + R2 * k) * LP + l] = k ? cmulc(v[k], tw[a * k]) : v[k];
     }
     __syncthreads();
     for (int it = threadIdx.x; it < R1 * LB; it += TH) {
         const int l = it % LB, k1 = it / LB;
         if (l >= ny) continue;
-        const D *vx = vt + (size_t)z * NN + y0 + l;   // [z][x][y]
+        const S *vx = vt + (size_t)z * NN + y0 + l;   // [z][x][y]
         C v[R2];
 #pragma unroll
-        for (int a = 0; a < R2; ++a) v[a] = S[(a + R2 * k1) * LP + l];
-        P<R2, true, N>::run(v, tw);
+        for (int a = 0; a < R2; ++a) v[a] = L[(a + R2 * k1) * LP + l];
+        P<S, R2, true, N>::run(v, tw);
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) v[k2] = vx[(size_t)(k1 + R1 * k2) * N] * v[k2];
-        P<R2, false, N>::run(v, tw);
+        P<S, R2, false, N>::run(v, tw);
 #pragma unroll
-        for (int a = 0; a < R2; ++a) S[(a + R2 * k1) * LP + l] = a ? cmul(v[a], tw[a * k1]) : v[a];
+        for (int a = 0; a < R2; ++a) L[(a + R2 * k1) * LP + l] = a ? cmul(v[a], tw[a * k1]) : v[a];
     }
     __syncthreads();
     for (int it = threadIdx.x; it < R2 * LB; it += TH) {
@@ -287,8 +334,8 @@ k_db(C *__restrict__ T2, int Px, const D *__restrict__ vt, const z64 *__restrict
         if (l >= ny) continue;
         C v[R1];
 #pragma unroll
-        for (int k = 0; k < R1; ++k) v[k] = S[(a + R2 * k) * LP + l];
-        step1<R1, false, N, HALF>(v, tw);
+        for (int k = 0; k < R1; ++k) v[k] = L[(a + R2 * k) * LP + l];
+        step1<S, R1, false, N, HALF>(v, tw);
 #pragma unroll
         for (int b = 0; b < R1; ++b) {
             const int px = a + R2 * b;
@@ -300,26 +347,27 @@ k_db(C *__restrict__ T2, int Px, const D *__restrict__ vt, const z64 *__restrict
 // ------------------------------------------------------------- pass A
 // One block per (band, x-plane).  Tile A[z][py] (pitch P1, odd).  After the z-FFT, slot k2 + R2 k1 of a row
 // holds z = k1 + R1 k2.  Dynamic shared memory: tw, tile, line buffer.
-template <int N, int R1, bool HALF>
+template <typename S, typename R, int N, int R1, bool HALF>
 __global__ void __launch_bounds__(TP, 1)
-k_da(const z64 *__restrict__ X, int ldx, C *__restrict__ T2, int Px, int Py, const int *__restrict__ plane_begin,
-     const int2 *__restrict__ yrange, const int *__restrict__ gmap, const z64 *__restrict__ twg, int lbs) {
+k_2a(const cx<R> *__restrict__ X, int ldx, cx<S> *__restrict__ T2, int Px, int Py, const int *__restrict__ plane_begin,
+     const int2 *__restrict__ yrange, const int *__restrict__ gmap, const cx<R> *__restrict__ twg, int lbs) {
+    using C = cx<S>;
     constexpr int R2 = N / R1;
     const int LB = 1 << lbs, LP = LB | 1;   // lines of a chunk
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P1 = Py | 1;
-    C *tw = reinterpret_cast<C *>(smem_raw), *A = tw + N, *S = A + (size_t)N * P1;
+    C *tw = reinterpret_cast<C *>(smem_raw), *A = tw + N, *L = A + (size_t)N * P1;
     const int px = blockIdx.x, bd = blockIdx.y;
-    const z64 *Xb = X + (size_t)bd * ldx;
-    const C zero = mkc<D>(D(0), D(0));
+    const cx<R> *Xb = X + (size_t)bd * ldx;
+    const C zero = mkc<S>(S(0), S(0));
     load_tw<N>(tw, twg);
     for (int i = threadIdx.x; i < N * P1; i += TP) A[i] = zero;
     __syncthreads();
     const int g1 = plane_begin[px + 1];
     for (int g = plane_begin[px] + threadIdx.x; g < g1; g += TP) {
         const int m = gmap[g], py = m / N, iz = m - py * N;
-        const z64 x = Xb[g];
-        A[iz * P1 + py] = mkc<D>((D)x.x, (D)x.y);
+        const cx<R> x = Xb[g];
+        A[iz * P1 + py] = mkc<S>((S)x.x, (S)x.y);
     }
     __syncthreads();
     const int2 yr = yrange[px];
@@ -329,7 +377,7 @@ k_da(const z64 *__restrict__ X, int ldx, C *__restrict__ T2, int Px, int Py, con
         C v[R1];
 #pragma unroll
         for (int b = 0; b < R1; ++b) v[b] = A[(a + R2 * b) * P1 + py];
-        P<R1, true, N>::run(v, tw);
+        P<S, R1, true, N>::run(v, tw);
 #pragma unroll
         for (int k = 0; k < R1; ++k) A[(a + R2 * k) * P1 + py] = k ? cmulc(v[k], tw[a * k]) : v[k];
     }
@@ -339,7 +387,7 @@ k_da(const z64 *__restrict__ X, int ldx, C *__restrict__ T2, int Px, int Py, con
         C v[R2];
 #pragma unroll
         for (int a = 0; a < R2; ++a) v[a] = A[(a + R2 * k1) * P1 + py];
-        P<R2, true, N>::run(v, tw);
+        P<S, R2, true, N>::run(v, tw);
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) A[(k2 + R2 * k1) * P1 + py] = v[k2];
     }
@@ -356,9 +404,9 @@ k_da(const z64 *__restrict__ X, int ldx, C *__restrict__ T2, int Px, int Py, con
                 const int py = a + R2 * b;
                 v[b] = (HALF && b > R1 / 2) ? zero : py < Py ? A[(s0 + l) * P1 + py] : zero;
             }
-            step1<R1, true, N, HALF>(v, tw);
+            step1<S, R1, true, N, HALF>(v, tw);
 #pragma unroll
-            for (int k = 0; k < R1; ++k) S[(a + R2 * k) * LP + l] = k ? cmulc(v[k], tw[a * k]) : v[k];
+            for (int k = 0; k < R1; ++k) L[(a + R2 * k) * LP + l] = k ? cmulc(v[k], tw[a * k]) : v[k];
         }
         __syncthreads();
         for (int it = threadIdx.x; it < R1 * LB; it += TP) {   // neighbouring threads on neighbouring y
@@ -367,8 +415,8 @@ k_da(const z64 *__restrict__ X, int ldx, C *__restrict__ T2, int Px, int Py, con
             const int sl = s0 + l, z = sl / R2 + R1 * (sl % R2);
             C v[R2];
 #pragma unroll
-            for (int a = 0; a < R2; ++a) v[a] = S[(a + R2 * k1) * LP + l];
-            P<R2, true, N>::run(v, tw);
+            for (int a = 0; a < R2; ++a) v[a] = L[(a + R2 * k1) * LP + l];
+            P<S, R2, true, N>::run(v, tw);
 #pragma unroll
             for (int k2 = 0; k2 < R2; ++k2) out[(size_t)z * N + k1 + R1 * k2] = v[k2];
         }
@@ -378,16 +426,17 @@ k_da(const z64 *__restrict__ X, int ldx, C *__restrict__ T2, int Px, int Py, con
 
 // ------------------------------------------------------------- pass C
 // One block per (band, x-plane), pass A backwards: slot b + R1 a of a row holds the z coefficient a + R2 b.
-template <int N, int R1, bool HALF>
+template <typename S, typename R, int N, int R1, bool HALF>
 __global__ void __launch_bounds__(TP, 1)
-k_dc(const C *__restrict__ T2, z64 *__restrict__ Y, int ldy, const z64 *__restrict__ X, int ldx,
-     const double *__restrict__ kin, int Px, int Py, const int *__restrict__ plane_begin,
-     const int2 *__restrict__ yrange, const int *__restrict__ gmap, const z64 *__restrict__ twg, int lbs) {
+k_2c(const cx<S> *__restrict__ T2, cx<R> *__restrict__ Y, int ldy, const cx<R> *__restrict__ X, int ldx,
+     const R *__restrict__ kin, int Px, int Py, const int *__restrict__ plane_begin,
+     const int2 *__restrict__ yrange, const int *__restrict__ gmap, const cx<R> *__restrict__ twg, int lbs) {
+    using C = cx<S>;
     constexpr int R2 = N / R1;
     const int LB = 1 << lbs, LP = LB | 1;   // lines of a chunk
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P1 = Py | 1;
-    C *tw = reinterpret_cast<C *>(smem_raw), *A = tw + N, *S = A + (size_t)N * P1;
+    C *tw = reinterpret_cast<C *>(smem_raw), *A = tw + N, *L = A + (size_t)N * P1;
     const int px = blockIdx.x, bd = blockIdx.y;
     load_tw<N>(tw, twg);
     __syncthreads();
@@ -400,9 +449,9 @@ k_dc(const C *__restrict__ T2, z64 *__restrict__ Y, int ldy, const z64 *__restri
             C v[R2];
 #pragma unroll
             for (int k2 = 0; k2 < R2; ++k2) v[k2] = in[(size_t)(z0 + l) * N + k1 + R1 * k2];
-            P<R2, false, N>::run(v, tw);
+            P<S, R2, false, N>::run(v, tw);
 #pragma unroll
-            for (int a = 0; a < R2; ++a) S[(a + R2 * k1) * LP + l] = a ? cmul(v[a], tw[a * k1]) : v[a];
+            for (int a = 0; a < R2; ++a) L[(a + R2 * k1) * LP + l] = a ? cmul(v[a], tw[a * k1]) : v[a];
         }
         __syncthreads();
         for (int it = threadIdx.x; it < R2 * LB; it += TP) {
@@ -410,8 +459,8 @@ k_dc(const C *__restrict__ T2, z64 *__restrict__ Y, int ldy, const z64 *__restri
             if (l >= nl) continue;
             C v[R1];
 #pragma unroll
-            for (int k = 0; k < R1; ++k) v[k] = S[(a + R2 * k) * LP + l];
-            step1<R1, false, N, HALF>(v, tw);
+            for (int k = 0; k < R1; ++k) v[k] = L[(a + R2 * k) * LP + l];
+            step1<S, R1, false, N, HALF>(v, tw);
 #pragma unroll
             for (int b = 0; b < R1; ++b) {
                 const int py = a + R2 * b;
@@ -427,7 +476,7 @@ k_dc(const C *__restrict__ T2, z64 *__restrict__ Y, int ldy, const z64 *__restri
         C v[R2];
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) v[k2] = A[(k1 + R1 * k2) * P1 + py];
-        P<R2, false, N>::run(v, tw);
+        P<S, R2, false, N>::run(v, tw);
 #pragma unroll
         for (int a = 0; a < R2; ++a) A[(k1 + R1 * a) * P1 + py] = a ? cmul(v[a], tw[a * k1]) : v[a];
     }
@@ -437,68 +486,69 @@ k_dc(const C *__restrict__ T2, z64 *__restrict__ Y, int ldy, const z64 *__restri
         C v[R1];
 #pragma unroll
         for (int k = 0; k < R1; ++k) v[k] = A[(k + R1 * a) * P1 + py];
-        P<R1, false, N>::run(v, tw);
+        P<S, R1, false, N>::run(v, tw);
 #pragma unroll
         for (int b = 0; b < R1; ++b) A[(b + R1 * a) * P1 + py] = v[b];
     }
     __syncthreads();
-    z64 *Yb = Y + (size_t)bd * ldy;
-    const z64 *Xb = X + (size_t)bd * ldx;
+    cx<R> *Yb = Y + (size_t)bd * ldy;
+    const cx<R> *Xb = X + (size_t)bd * ldx;
     const int g1 = plane_begin[px + 1];
     for (int g = plane_begin[px] + threadIdx.x; g < g1; g += TP) {
         const int m = gmap[g], py = m / N, iz = m - py * N;
         C v = A[(iz / R2 + R1 * (iz % R2)) * P1 + py];
         if (kin) {
-            const D t = (D)kin[g];
-            const z64 x = Xb[g];
-            v = v + t * mkc<D>((D)x.x, (D)x.y);
+            const S t = (S)kin[g];
+            const cx<R> x = Xb[g];
+            v = v + t * mkc<S>((S)x.x, (S)x.y);
         }
-        Yb[g] = mkc((double)v.x, (double)v.y);
+        Yb[g] = mkc<R>((R)v.x, (R)v.y);
     }
 }
 
 // Lines of a chunk of the plane passes (a power of two, its logarithm) for the shared memory at hand; -1: the
 // plane tile does not fit.
-inline int chunk_log2(const FFTGeom &g, int smem_max) {
+template <typename S>
+int chunk_log2(const FFTGeom &g, int smem_max) {
     for (int l = 5; l >= 1; --l)
-        if (sizeof(C) * (size_t)g.N * (1 + (g.Py | 1) + ((1 << l) | 1)) <= (size_t)smem_max) return l;
+        if (sizeof(cx<S>) * (size_t)g.N * (1 + (g.Py | 1) + ((1 << l) | 1)) <= (size_t)smem_max) return l;
     return -1;
 }
 
 // 1: the geometry does not fit (the caller's general passes take it).
-template <int N, int R1>
-int run(const FFTGeom &g, const z64 *X, int ldx, z64 *Y, int ldy, int nb, const double *kin, const D *vt, const z64 *tw,
-        C *T2, int nbatch, int smem_max, cudaStream_t s) {
-    const int lbs = chunk_log2(g, smem_max);
+template <typename S, typename R, int N, int R1>
+int run(const Fft2Args<S, R> &a) {
+    const FFTGeom &g = *a.g;
+    const int lbs = chunk_log2<S>(g, a.smem_max);
     if (lbs < 0) return 1;
-    const size_t sm = sizeof(C) * (size_t)N * (1 + (g.Py | 1) + ((1 << lbs) | 1));
+    const size_t sm = sizeof(cx<S>) * (size_t)N * (1 + (g.Py | 1) + ((1 << lbs) | 1));
     const bool half = g.Px <= N / 2 + 1 && g.Py <= N / 2 + 1;
     static std::atomic<bool> attr{false};
     if (!attr.load()) {
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_da<N, R1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_dc<N, R1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_da<N, R1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
-        LG_CUDA_TRY(cudaFuncSetAttribute(k_dc<N, R1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+        const void *fns[] = {(const void *)k_2a<S, R, N, R1, true>, (const void *)k_2c<S, R, N, R1, true>,
+                             (const void *)k_2a<S, R, N, R1, false>, (const void *)k_2c<S, R, N, R1, false>};
+        for (const void *f : fns)
+            LG_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a.smem_max));
         attr.store(true);
     }
     auto passes = [&](auto ka, auto kb, auto kc) -> int {
-        for (int b0 = 0; b0 < nb; b0 += nbatch) {
-            const int nbb = std::min(nbatch, nb - b0);
-            const z64 *Xb = X + (size_t)b0 * ldx;
-            z64 *Yb = Y + (size_t)b0 * ldy;
-            ka<<<dim3(g.Px, nbb), TP, sm, s>>>(Xb, ldx, T2, g.Px, g.Py, g.plane_begin, g.plane_yrange, g.gmap, tw, lbs);
-            LG_TRY(check_launch("fft pass A (double-FP32)"));
-            kb<<<dim3((N + LB - 1) / LB, N, nbb), TH, 0, s>>>(T2, g.Px, vt, tw);
-            LG_TRY(check_launch("fft pass B (double-FP32)"));
-            kc<<<dim3(g.Px, nbb), TP, sm, s>>>(T2, Yb, ldy, Xb, ldx, kin, g.Px, g.Py, g.plane_begin, g.plane_yrange,
-                                              g.gmap, tw, lbs);
-            LG_TRY(check_launch("fft pass C (double-FP32)"));
+        for (int b0 = 0; b0 < a.nb; b0 += a.nbatch) {
+            const int nbb = std::min(a.nbatch, a.nb - b0);
+            const cx<R> *Xb = a.X + (size_t)b0 * a.ldx;
+            cx<R> *Yb = a.Y + (size_t)b0 * a.ldy;
+            ka<<<dim3(g.Px, nbb), TP, sm, a.s>>>(Xb, a.ldx, a.T2, g.Px, g.Py, g.plane_begin, g.plane_yrange, g.gmap, a.tw, lbs);
+            LG_TRY(check_launch("fft pass A (two-step)"));
+            kb<<<dim3((N + LB - 1) / LB, N, nbb), TH, 0, a.s>>>(a.T2, g.Px, a.vt, a.tw);
+            LG_TRY(check_launch("fft pass B (two-step)"));
+            kc<<<dim3(g.Px, nbb), TP, sm, a.s>>>(a.T2, Yb, a.ldy, Xb, a.ldx, a.kin, g.Px, g.Py, g.plane_begin,
+                                                g.plane_yrange, g.gmap, a.tw, lbs);
+            LG_TRY(check_launch("fft pass C (two-step)"));
         }
         return LOBPCG_OK;
     };
-    if (half) return passes(k_da<N, R1, true>, k_db<N, R1, true>, k_dc<N, R1, true>);
-    return passes(k_da<N, R1, false>, k_db<N, R1, false>, k_dc<N, R1, false>);
+    if (half) return passes(k_2a<S, R, N, R1, true>, k_2b<S, R, N, R1, true>, k_2c<S, R, N, R1, true>);
+    return passes(k_2a<S, R, N, R1, false>, k_2b<S, R, N, R1, false>, k_2c<S, R, N, R1, false>);
 }
 
-}  // namespace fdf
+}  // namespace f2s
 }  // namespace lg
