@@ -1424,19 +1424,20 @@ static int create_impl(lobpcg_ctx *c, const lobpcg_cell *cell, int nk, const dou
     c->cell = *cell;
     c->nk = nk;
     c->nproj = nproj;
-    // potential: [x][y][z] -> [z][x][y] (FP32 register FFT: [y][x][z]), scaled by 1/N^3
+    // potential: [x][y][z] -> [z][x][y] (FP32 register passes: [y][x][z]), scaled by 1/N^3
     // (the forward FFT's normalisation)
     std::vector<double> vt(N3);
     std::vector<float> vt32(N3);
     const double inv = 1.0 / (double)N3;
     const bool reg32 = fft_reg_supported(N);
+    const bool yxz = reg32 && !fft2_f32_edge(N);
     if (reg32) LG_TRY(fft_reg_prepare());
     for (int x = 0; x < N; ++x)
         for (int y = 0; y < N; ++y)
             for (int z = 0; z < N; ++z) {
                 const double v = vloc_r[((size_t)x * N + y) * N + z] * inv;
                 vt[((size_t)z * N + x) * N + y] = v;
-                vt32[reg32 ? ((size_t)y * N + x) * N + z : ((size_t)z * N + x) * N + y] = (float)v;
+                vt32[yxz ? ((size_t)y * N + x) * N + z : ((size_t)z * N + x) * N + y] = (float)v;
             }
     LG_TRY(upload(c, &c->vt64, vt.data(), N3));
     {   // the same table as (hi, lo) FP32 pairs for the double-FP32 passes

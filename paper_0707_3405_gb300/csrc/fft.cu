@@ -548,13 +548,32 @@ template int fft_density<float>(const FFTGeom &, const FFTPlan &, const c32 *, i
 template int fft_density<double>(const FFTGeom &, const FFTPlan &, const z64 *, int, int, const z64 *,
                                  const double *, const float *, double, double *, z64 *, int, cudaStream_t, bool);
 
+// FP32 edges of the two-step passes: those without register passes, and those whose lane would hold 24 or more
+// points of a line there (three or fewer blocks an SM).  GB300, us, 128 bands, the other passes / two-step:
+//   no register passes: 40 406 / 90, 54 1534 / 171, 60 1410 / 225, 80 2885 / 463, 90 5081 / 702, 100 5491 / 935,
+//   108 8282 / 1174; from 24 points: 96 746 / 718, 120 1761 / 1433, 128 2126 / 2119 (one band 50.4 / 41.7),
+//   160 6236 / 3904; below: 24 27 / 39, 36 55 / 80, 48 92 / 117, 64 210 / 228, 72 323 / 373.
+bool fft2_f32_edge(int N) {
+    for (int n : {40, 54, 60, 80, 90, 96, 100, 108, 120, 128, 160})
+        if (n == N) return true;
+    return false;
+}
+
 template <typename R>
 int fft_vloc_apply(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx, cx<R> *Y, int ldy, int nb,
                    const R *kin, const R *vt, const cx<R> *tw, cx<R> *T2, int nbatch, cudaStream_t s, bool df,
                    const float2 *vt_pair) {
     if (nb <= 0) return LOBPCG_OK;
     if constexpr (std::is_same<R, float>::value) {
-        if (fft_reg_supported(g.N)) return fft_reg_apply(g, X, ldx, Y, ldy, nb, kin, vt, T2, nbatch, s);
+        if (fft2_f32_edge(g.N)) {
+            const Fft2Args<float, float> a{&g, X, ldx, Y, ldy, nb, kin, vt, tw, T2, nbatch, max_dyn_smem(), s};
+            for (auto f : {fft2_f32_1, fft2_f32_2, fft2_f32_3, fft2_f32_4}) {
+                const int rc = f(a);
+                if (rc <= 0) return rc;
+            }
+        } else if (fft_reg_supported(g.N)) {
+            return fft_reg_apply(g, X, ldx, Y, ldy, nb, kin, vt, T2, nbatch, s);
+        }
     } else {
         if (df) {  // FP64 data transformed in double-FP32 (the half box holds pairs of floats)
             if (vt_pair) {  // grid edges with two-step kernels: 1 where they do not apply
@@ -571,6 +590,7 @@ int fft_vloc_apply(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ld
                                         reinterpret_cast<const df64f *>(vt_pair), tw, reinterpret_cast<cx<df64f> *>(T2),
                                        nbatch, s);
         }
+        // GB300, H on 64 bands of the 72^3 cell in FP64: 8.5 ms with the passes below, 6.6 with these
         const Fft2Args<double, double> a{&g, X, ldx, Y, ldy, nb, kin, vt, tw, T2, nbatch, max_dyn_smem(), s};
         for (auto f : {fft2_f64_1, fft2_f64_2, fft2_f64_3, fft2_f64_4}) {
             const int rc = f(a);

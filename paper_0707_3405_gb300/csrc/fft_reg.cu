@@ -694,8 +694,7 @@ int fft_reg_apply(const FFTGeom &g, const C *X, int ldx, C *Y, int ldy, int nb, 
 #define LG_REG_CASE(n) \
     case n: return run_reg<n>(g, X, ldx, Y, ldy, nb, kin, vr, T2, nbatch, s);
         LG_REG_CASE(8) LG_REG_CASE(12) LG_REG_CASE(16) LG_REG_CASE(20) LG_REG_CASE(24) LG_REG_CASE(36)
-        LG_REG_CASE(48) LG_REG_CASE(64) LG_REG_CASE(72) LG_REG_CASE(96) LG_REG_CASE(120) LG_REG_CASE(128)
-        LG_REG_CASE(160)
+        LG_REG_CASE(48) LG_REG_CASE(64) LG_REG_CASE(72)   // longer edges: fft2_f32_edge
 #undef LG_REG_CASE
         default: return fail(LOBPCG_ERR_UNSUPPORTED, "no register FFT for this grid");
     }

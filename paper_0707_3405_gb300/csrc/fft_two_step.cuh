@@ -1,4 +1,4 @@
-// Double-FP32 and FP64 passes of the local potential (Sec. 4.1: Goedecker's zero-padded FFT) for grid edges
+// Double-FP32, FP64 and FP32 passes of the local potential (Sec. 4.1: Goedecker's zero-padded FFT) for grid edges
 // N = R1 R2 with both factors small enough for a thread's registers.
 //
 // Same three passes as fft.cu (A: sphere -> z-FFT -> y-FFT, B: x-FFT, V, x-FFT, C: y-FFT -> z-FFT ->
@@ -21,7 +21,12 @@
 //     are renormalised (19 instead of 25 operations per two-term sum).
 // What bounds it: FP32 issue.  Measured on a GB300, 9 bands of the 120^3 cell a launch, us, against the
 // shared-memory passes with one exchange and two barriers per radix (4, 2, 5, 3): pass A 227 -> 122,
-// B 675 -> 295, C 288 -> 155; H on 128 bands with 432 projectors 20.7 -> 12.1 ms.
+// B 675 -> 295, C 288 -> 155; H on 128 bands with 432 projectors 20.7 -> 12.1 ms.  FP64 is bound by its
+// units: 64 bands of the 72^3 cell, pass A 540 -> 390, B 1620 -> 1000, C 614 -> 405.  FP32, 19 bands of the
+// 120^3 cell against the register passes (fft_reg.cu): A 67 -> 53, B 119 -> 92 (issuing 41 % of the cycles, the
+// shared-memory pipe 68 % busy, 200 MB of DRAM), C 71 -> 61; both twiddle products of pass B in its second step
+// (one read instead of two), five or seven blocks an SM, 16 lines a block, 256 threads or 16-line chunks in the
+// plane passes: 2 to 5 % slower.
 #pragma once
 
 #include "common.cuh"
@@ -29,6 +34,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 namespace lg {
 
@@ -51,7 +57,8 @@ struct Fft2Args {
 // The passes for the grid edges of one source file each; 1 where they do not apply.
 #define LG_FFT2(n)                                   \
     int fft2_df_##n(const Fft2Args<df64f, double> &); \
-    int fft2_f64_##n(const Fft2Args<double, double> &);
+    int fft2_f64_##n(const Fft2Args<double, double> &); \
+    int fft2_f32_##n(const Fft2Args<float, float> &);
 LG_FFT2(1) LG_FFT2(2) LG_FFT2(3) LG_FFT2(4)
 #undef LG_FFT2
 
@@ -275,10 +282,18 @@ __device__ __forceinline__ void step1(cx<S> (&v)[R1], const cx<S> *tw) {
     else P<S, R1, INV, N>::run(v, tw);
 }
 
-constexpr int LB = 16;    // lines per block of pass B
-constexpr int LP = 17;    // entries between positions of the line buffer (bank spread)
-constexpr int TH = 128;   // threads of pass B: four blocks an SM, so that one's barriers overlap the others' work
-constexpr int TP = 512;   // threads of the plane passes, whose tile leaves room for one block
+// Blocks: FP32 lines are half as long in bytes and registers, so pass B takes a warp's width of lines (twiddle
+// reads are then broadcasts) and the plane passes share an SM in pairs.
+template <typename S>
+struct Shape {
+    static constexpr bool F32 = std::is_same<S, float>::value;
+    static constexpr int LB = F32 ? 32 : 16;   // lines per block of pass B
+    static constexpr int LP = LB + 1;          // entries between positions of the line buffer (bank spread)
+    static constexpr int NB = F32 ? 6 : 4;     // blocks of pass B an SM: one's barriers overlap the others' work
+    static constexpr int NP = F32 ? 2 : 1;     // blocks of the plane passes, as many as their tile leaves room for
+};
+constexpr int TH = 128;   // threads of pass B
+constexpr int TP = 512;   // threads of the plane passes
 
 template <int N, typename S, typename R>
 __device__ __forceinline__ void load_tw(cx<S> *tw, const cx<R> *__restrict__ twg) {
@@ -287,10 +302,11 @@ __device__ __forceinline__ void load_tw(cx<S> *tw, const cx<R> *__restrict__ twg
 
 // ------------------------------------------------------------- pass B
 template <typename S, typename R, int N, int R1, bool HALF>
-__global__ void __launch_bounds__(TH, 4)
+__global__ void __launch_bounds__(TH, Shape<S>::NB)
 k_2b(cx<S> *__restrict__ T2, int Px, const S *__restrict__ vt, const cx<R> *__restrict__ twg) {
     using C = cx<S>;
     constexpr int R2 = N / R1;
+    constexpr int LB = Shape<S>::LB, LP = Shape<S>::LP;
     __shared__ C tw[N];
     __shared__ C L[N * LP];
     const int y0 = blockIdx.x * LB, z = blockIdx.y;
@@ -348,7 +364,7 @@ k_2b(cx<S> *__restrict__ T2, int Px, const S *__restrict__ vt, const cx<R> *__re
 // One block per (band, x-plane).  Tile A[z][py] (pitch P1, odd).  After the z-FFT, slot k2 + R2 k1 of a row
 // holds z = k1 + R1 k2.  Dynamic shared memory: tw, tile, line buffer.
 template <typename S, typename R, int N, int R1, bool HALF>
-__global__ void __launch_bounds__(TP, 1)
+__global__ void __launch_bounds__(TP, Shape<S>::NP)
 k_2a(const cx<R> *__restrict__ X, int ldx, cx<S> *__restrict__ T2, int Px, int Py, const int *__restrict__ plane_begin,
      const int2 *__restrict__ yrange, const int *__restrict__ gmap, const cx<R> *__restrict__ twg, int lbs) {
     using C = cx<S>;
@@ -427,7 +443,7 @@ k_2a(const cx<R> *__restrict__ X, int ldx, cx<S> *__restrict__ T2, int Px, int P
 // ------------------------------------------------------------- pass C
 // One block per (band, x-plane), pass A backwards: slot b + R1 a of a row holds the z coefficient a + R2 b.
 template <typename S, typename R, int N, int R1, bool HALF>
-__global__ void __launch_bounds__(TP, 1)
+__global__ void __launch_bounds__(TP, Shape<S>::NP)
 k_2c(const cx<S> *__restrict__ T2, cx<R> *__restrict__ Y, int ldy, const cx<R> *__restrict__ X, int ldx,
      const R *__restrict__ kin, int Px, int Py, const int *__restrict__ plane_begin,
      const int2 *__restrict__ yrange, const int *__restrict__ gmap, const cx<R> *__restrict__ twg, int lbs) {
@@ -538,7 +554,7 @@ int run(const Fft2Args<S, R> &a) {
             cx<R> *Yb = a.Y + (size_t)b0 * a.ldy;
             ka<<<dim3(g.Px, nbb), TP, sm, a.s>>>(Xb, a.ldx, a.T2, g.Px, g.Py, g.plane_begin, g.plane_yrange, g.gmap, a.tw, lbs);
             LG_TRY(check_launch("fft pass A (two-step)"));
-            kb<<<dim3((N + LB - 1) / LB, N, nbb), TH, 0, a.s>>>(a.T2, g.Px, a.vt, a.tw);
+            kb<<<dim3((N + Shape<S>::LB - 1) / Shape<S>::LB, N, nbb), TH, 0, a.s>>>(a.T2, g.Px, a.vt, a.tw);
             LG_TRY(check_launch("fft pass B (two-step)"));
             kc<<<dim3(g.Px, nbb), TP, sm, a.s>>>(a.T2, Yb, a.ldy, Xb, a.ldx, a.kin, g.Px, g.Py, g.plane_begin,
                                                 g.plane_yrange, g.gmap, a.tw, lbs);
