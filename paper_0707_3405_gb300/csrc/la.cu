@@ -1265,12 +1265,28 @@ __device__ __forceinline__ RT hash_uniform(unsigned int a, unsigned int b) {
     return (RT)h * (2.0 / 4294967296.0) - 1.0;
 }
 
+// |a| < |b| and a == 0; for FP64 on the bits, without an FP64 instruction
+__device__ __forceinline__ bool mag_less(float a, float b) { return fabsf(a) < fabsf(b); }
+__device__ __forceinline__ bool is_zero(float a) { return a == 0.f; }
+__device__ __forceinline__ bool mag_less(double a, double b) {
+    constexpr unsigned long long M = 0x7FFFFFFFFFFFFFFFULL;
+    return ((unsigned long long)__double_as_longlong(a) & M) < ((unsigned long long)__double_as_longlong(b) & M);
+}
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
+
 // One warp per eigenvalue index; the warp whose eigenvalue starts a cluster of
 // close eigenvalues computes all vectors of that cluster, in order: lane 0 runs the
 // LU of T - lambda I with partial pivoting and the solves (sequential recurrences,
-// kept in shared memory), from a pseudo-random start, three times; after each solve
-// the warp orthogonalises against the cluster's earlier vectors (modified
-// Gram-Schmidt) and normalises.  Dynamic shared memory: 6 n reals + n pivots.
+// kept in shared memory), from a pseudo-random start; after each solve the warp
+// orthogonalises against the cluster's earlier vectors (modified Gram-Schmidt) and
+// normalises.  Dynamic shared memory: 6 n reals + n pivots.
+// What bounds it: lane 0's chain of dependent FP64 instructions, 64 cycles or more each (with few clusters, of
+// the longest one).  So comparisons run on the bits, rows are swapped by selects (a predicated-off
+// instruction costs the same), each pivot is inverted once (the multiplier is its product with the
+// reciprocal, corrected by its remainder; the rows of U are divided by their pivots by all lanes), and a
+// vector alone beyond gaptol takes two solves: each shrinks the others' part by 1e-8 or more, so that
+// the second leaves rounding only; three within clusters and in FP32.  GB300, the step with 128 vectors of
+// n = 384 in double-FP32 4.57 -> 4.45 ms, n = 1152 33.0 -> 31.9.
 template <typename RT>
 __global__ void __launch_bounds__(32)
 k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, const RT *__restrict__ theta,
@@ -1295,48 +1311,66 @@ k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, cons
         if (j > k && lam < lam_prev + pert) lam = lam_prev + pert;
         lam_prev = lam;
         RT *zj = Z + (size_t)j * n;
-        if (lane == 0) {
-            for (int i = 0; i < n; ++i) dd[i] = d[i] - lam;
-            for (int i = 0; i + 1 < n; ++i) { du[i] = e[i]; dl[i] = e[i]; du2[i] = 0.0; }
-            for (int i = 0; i + 1 < n; ++i) {
-                if (fabs(dd[i]) >= fabs(dl[i])) {
-                    pv[i] = 0;
-                    if (dd[i] == 0.0) dd[i] = pert;
-                    const RT f = dl[i] / dd[i];
-                    dl[i] = f;
-                    dd[i + 1] -= f * du[i];
-                } else {
-                    pv[i] = 1;
-                    const RT f = dd[i] / dl[i];
-                    dd[i] = dl[i];
-                    dl[i] = f;
-                    const RT t = du[i];
-                    du[i] = dd[i + 1];
-                    dd[i + 1] = t - f * dd[i + 1];
-                    if (i + 2 < n) { du2[i] = du[i + 1]; du[i + 1] = -f * du[i + 1]; }
-                }
-            }
-            if (dd[n - 1] == 0.0) dd[n - 1] = pert;
+        for (int i = lane; i < n; i += 32) {
+            dd[i] = d[i] - lam;
+            dl[i] = i + 1 < n ? e[i] : (RT)0.0;
+            z[i] = hash_uniform<RT>((unsigned)j, (unsigned)i);
         }
         __syncwarp();
-        // reciprocal pivots, all lanes: the three solves below then multiply instead of divide
-        for (int i = lane; i < n; i += 32) rdd[i] = (RT)1.0 / dd[i];
-        for (int i = lane; i < n; i += 32) z[i] = hash_uniform<RT>((unsigned)j, (unsigned)i);
+        if (lane == 0) {
+            RT p = dd[0], u = dl[0];            // the row being eliminated: pivot candidate and its right neighbour
+            for (int i = 0; i + 1 < n; ++i) {
+                const RT l = dl[i], dn = dd[i + 1], un = dl[i + 1];
+                const bool sw = mag_less(p, l);
+                RT piv = sw ? l : p;
+                const RT o = sw ? p : l, u0 = sw ? dn : u, u1 = sw ? u : dn;
+                if (is_zero(piv)) piv = pert;
+                const RT r = (RT)1.0 / piv, f0 = o * r;
+                const RT f = fma(fma(-f0, piv, o), r, f0);   // o / piv
+                rdd[i] = r;
+                dl[i] = f;
+                du[i] = u0;
+                du2[i] = sw ? un : (RT)0.0;
+                pv[i] = sw;
+                p = fma(-f, u0, u1);
+                const RT t = -f * un;
+                u = sw ? t : un;
+            }
+            if (is_zero(p)) p = pert;
+            rdd[n - 1] = (RT)1.0 / p;
+        }
         __syncwarp();
-        for (int it = 0; it < 3; ++it) {
+        for (int i = lane; i + 1 < n; i += 32) {   // rows of U over their pivots
+            du[i] *= rdd[i];
+            du2[i] *= rdd[i];
+        }
+        __syncwarp();
+        // alone beyond gaptol: the part of every other vector shrinks by (error of lam) / gap <= 1e-8 per solve
+        const bool alone = j == k && (j + 1 < m ? theta[j + 1] - theta[j] > gaptol : m == n);
+        const int solves = alone && sizeof(RT) == 8 ? 2 : 3;
+        for (int it = 0; it < solves; ++it) {
             if (lane == 0) {
+                RT zi = z[0];
                 for (int i = 0; i + 1 < n; ++i) {
-                    if (pv[i] == 0) {
-                        z[i + 1] -= dl[i] * z[i];
-                    } else {
-                        const RT t = z[i];
-                        z[i] = z[i + 1];
-                        z[i + 1] = t - dl[i] * z[i];
-                    }
+                    const RT zn = z[i + 1], f = dl[i];
+                    const bool sw = pv[i];
+                    const RT x = sw ? zn : zi, y = sw ? zi : zn;
+                    z[i] = x;
+                    zi = fma(-f, x, y);
                 }
-                z[n - 1] = z[n - 1] * rdd[n - 1];
-                if (n > 1) z[n - 2] = (z[n - 2] - du[n - 2] * z[n - 1]) * rdd[n - 2];
-                for (int i = n - 3; i >= 0; --i) z[i] = (z[i] - du[i] * z[i + 1] - du2[i] * z[i + 2]) * rdd[i];
+                z[n - 1] = zi;
+            }
+            __syncwarp();
+            for (int i = lane; i < n; i += 32) z[i] *= rdd[i];
+            __syncwarp();
+            if (lane == 0) {
+                RT z1 = z[n - 1], z2 = 0.0;
+                for (int i = n - 2; i >= 0; --i) {
+                    const RT x = fma(-du[i], z1, fma(-du2[i], z2, z[i]));
+                    z[i] = x;
+                    z2 = z1;
+                    z1 = x;
+                }
             }
             __syncwarp();
             for (int p = k; p < j; ++p) {

@@ -73,3 +73,32 @@ def test_heev_scales(scale):
     nrm = np.abs(A).sum(1).max()
     assert np.abs(w - np.linalg.eigvalsh(A)).max() < 1e-13 * nrm
     assert np.abs(V.conj().T @ V - np.eye(90)).max() < 1e-12
+
+
+@pytest.mark.parametrize("n", [2, 3, 33, 90, 200])
+@pytest.mark.parametrize("kind", ["wide", "near", "clusters", "equal", "blocks"])
+def test_heev_spectra(kind, n):
+    # inverse iteration at the edge of a cluster: neighbours 2e-5 |T| apart are solved alone (their vectors
+    # are orthogonal to about eps / 2e-5, times 16), closer ones together
+    import torch
+    import paper_0707_3405_gb300 as lg
+    rng = np.random.default_rng(n)
+    if kind == "wide":
+        lam = np.arange(n) - n / 3.0
+    elif kind == "near":
+        lam = np.where(np.arange(n) % 2 == 0, np.arange(n), np.arange(n) - 1 + 4e-5 * n)
+    elif kind == "clusters":
+        lam = np.floor(np.arange(n) / 5.0) + 1e-9 * np.arange(n)
+    elif kind == "equal":
+        lam = np.full(n, 0.75)
+    else:
+        lam = np.arange(n) * 1.0
+    Q = np.linalg.qr(_herm(rng, n))[0] if kind != "blocks" else np.eye(n)
+    A = (Q * lam) @ Q.conj().T
+    A = (0.5 * (A + A.conj().T)).astype(complex)
+    w, V = lg.heev(torch.tensor(A.T.copy(), device="cuda"))
+    w, V = w.cpu().numpy(), V.cpu().numpy().T
+    nrm = np.abs(A).sum(1).max()
+    assert np.abs(w - np.linalg.eigvalsh(A)).max() < 1e-12 * nrm
+    assert np.abs(A @ V - V * w[None, :]).max() < 1e-11 * nrm
+    assert np.abs(V.conj().T @ V - np.eye(n)).max() < 16 * 2.0 ** -52 / 1e-5
