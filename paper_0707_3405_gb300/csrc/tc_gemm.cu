@@ -15,8 +15,8 @@
 //   D = A B:    [re, -im, ...] and [im, re, ...] of B's column.
 //
 // One persistent CTA per SM takes every gridDim-th item (an output tile, and for A^H B a part of
-// the reduction, which is split over the GPU).  Eight warps load FP32 from HBM two stages ahead
-// into registers, split it and store hi / lo into 64-byte-swizzled K-major shared tiles of a
+// the reduction, which is split over the GPU).  Sixteen warps in four groups, one per ring slot, load FP32
+// from HBM ahead into registers, split it and store hi / lo into 64-byte-swizzled K-major shared tiles of a
 // 4-stage ring (8 complex K a stage); one warp issues a stage's six MMAs of M = 128, N = 2 NT and
 // commits them to the stage's mbarrier; four warps read the accumulator of the finished item from
 // TMEM, which holds two, and write it out while the next item runs.  FP32 partial tiles of a split

@@ -4,6 +4,7 @@
 // the FP64 residual norms of the convergence test, precision casts and
 // row scalings.
 #include "common.cuh"
+#include "df64.cuh"
 
 #include <cstring>
 
@@ -38,6 +39,8 @@ __device__ void block_sum2(double &a, double &b) {
 // Two sums per column over the plane waves, split over chunks of rows so that the FP64 work of
 // a few columns spreads over the whole GPU (one block per column would leave it to that block's
 // SM, whose FP64 units are few); the chunk partials are added in a fixed order (reproducible).
+// FP64 issue bounds them: four chained FMAs an element instead of six to eight operations took the Rayleigh
+// quotients of 57925 x 64 from 64 to 46 us on a GB300.
 enum ColOp { kEkin = 0, kRayleigh = 1, kDiag = 2, kResid = 3 };
 constexpr int kMaxChunks = 32;
 
@@ -53,19 +56,19 @@ k_colsum2(int npw, int chunk, const z64 *__restrict__ X, int ldx, const z64 *__r
     double a = 0.0, b = 0.0;
     for (int g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
         const z64 xv = x[g];
-        const double xx = abs2(xv);
         if (OP == kEkin) {
+            const double xx = abs2(xv);
             a += kin[g] * xx;
             b += xx;
         } else if (OP == kResid) {
             const z64 hv = h[g];
             const double p = hv.x - th * xv.x, q = hv.y - th * xv.y;
-            a += p * p + q * q;
-            b += xx;
+            a = fma(q, q, fma(p, p, a));
+            b = fma(xv.y, xv.y, fma(xv.x, xv.x, b));
         } else {
             const z64 hv = h[g];
-            a += xx;
-            b += xv.x * hv.x + xv.y * hv.y;
+            a = fma(xv.y, xv.y, fma(xv.x, xv.x, a));
+            b = fma(xv.y, hv.y, fma(xv.x, hv.x, b));
         }
     }
     block_sum2(a, b);
@@ -205,15 +208,34 @@ __global__ void k_residual32(int npw, const z64 *__restrict__ X, int ldx, const 
 }
 
 // W = K(R) (Teter-Payne-Allan, x = T(q)/Ekin_j) on FP32 columns.
+__device__ __noinline__ float teter_fp64(double t0, double e0) {
+    const double t = t0 / e0, p = 27.0 + t * (18.0 + t * (12.0 + 8.0 * t)), t2 = t * t;
+    return (float)(p / (p + 16.0 * t2 * t2));
+}
+// K(t / e) rounded to FP32 from double-FP32 arithmetic, in x = t / e up to 1 and in x = e / t beyond (numerator and
+// denominator over x^4), which stays in FP32's range; FP64 where a divisor does not.
+__device__ __forceinline__ float teter32(double t0, double e0) {
+    const df64 t(t0), e(e0);
+    const bool low = t.hi <= e.hi;
+    const df64 num = low ? t : e, den = low ? e : t;
+    if (!(den.hi > 1e-30f && den.hi < 1e30f)) return teter_fp64(t0, e0);
+    const df64 x = num / den;
+    df64 p = ((df64(low ? 8.f : 27.f) * x + df64(low ? 12.f : 18.f)) * x + df64(low ? 18.f : 12.f)) * x +
+             df64(low ? 27.f : 8.f);
+    const df64 x2 = x * x, x4 = x2 * x2, px = p * x;
+    if (!low) p = px;
+    const df64 q = low ? df64(16.f * x4.hi, 16.f * x4.lo) : df64(16.f);
+    return (p / (p + q)).hi;
+}
+
+// W = K(R), FP32.  In FP64 the quotient's 20 instructions of 64 cycles a warp bound it: 57925 x 64, GB300,
+// 124 -> 35 us with pairs (memory: 9).
 __global__ void k_precond32(int npw, const c32 *__restrict__ R, int ldr, const double *__restrict__ kin,
                             const double *__restrict__ ekin, c32 *__restrict__ W, int ldw) {
     const int j = blockIdx.y;
-    const double ie = 1.0 / ekin[j];
+    const double e = ekin[j];
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < npw; g += gridDim.x * blockDim.x) {
-        const double t = kin[g] * ie;
-        const double p = 27.0 + t * (18.0 + t * (12.0 + 8.0 * t));
-        const double t2 = t * t;
-        const float k = (float)(p / (p + 16.0 * t2 * t2));
+        const float k = teter32(kin[g], e);
         const c32 r = R[(size_t)j * ldr + g];
         W[(size_t)j * ldw + g] = mkc<float>(k * r.x, k * r.y);
     }
