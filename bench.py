@@ -428,9 +428,9 @@ FP32_INSTR_PER_S = 152 * 128 * 2.07e9
 DF32_INSTR_PER_CMAC = 48.0
 TF32_PER_BF16 = 1.1 / 2.25        # nominal dense TF32 / BF16 tensor rates
 OZ_PAIRS = 21                     # digit-slice products per real product of the FP64-class tensor-core GEMM
-# Dominant kernel of the mixed solve on the benchmark cell (launch list in profiles/): the 3xTF32
-# A B of the block updates, k_tc_nn<128> (14% of device time), timed here at a block update's
-# shape; the FP64-class tensor GEMMs (22% as a family) are reported beside it under kernels.
+# Largest contraction of the mixed solve on the benchmark cell (launch list in profiles/): the 3xTF32
+# A B of the block updates, k_tc_nn<128> (12% of device time), timed here at a block update's
+# shape; the FP64-class tensor GEMMs (20% as a family) are reported beside it under kernels.
 DOMINANT = "update_3xtf32"
 
 
@@ -548,7 +548,7 @@ def kernel_rooflines(w, npw, nbands, pk, reps=3):
             px = int(mil[:, 0].max() - mil[:, 0].min() + 1)
             by = m * (4.0 * 8 * px * w.N * w.N + 3.0 * 8 * s.npw(0) + 4.0 * s.npw(0)) + 4.0 * w.N ** 3
             out["fft_c64"] = {
-                "kernel": f"k_ra<{w.N}> + k_rb<{w.N}> + k_rc<{w.N}>", "shape": [m, s.npw(0), w.N], "bound": "hbm",
+                "kernel": "FP32 FFT passes A + B + C", "shape": [m, s.npw(0), w.N], "bound": "hbm",
                 "unit": "GB/s", "ms": t * 1e3, "achieved": by / t / 1e9, "peak": hbm, "frac": by / t / 1e9 / hbm,
                 "band_applies_per_s": m / t, "work_per_launch": f"{by:.4g} algorithmic bytes",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
@@ -561,8 +561,8 @@ def kernel_rooflines(w, npw, nbands, pk, reps=3):
 
 # DRAM bytes per launch (read + write) from one ncu capture, by kernel entry and shape; valid only
 # while the kernel is unchanged since the capture (the summary names the command).
-TRAFFIC = {("fp64class_gemm", (113081, 1152, 1152)): (1.905e10, "profiles/fp64class_tensor_gemm_traffic_gamma120.md"),
-           ("update_3xtf32", (113081, 128, 256)): (3.16e8, "profiles/tc_nn_3xtf32_update_gamma120.md")}
+TRAFFIC = {("fp64class_gemm", (113081, 1152, 1152)): (1.884e10, "profiles/fp64class_tensor_gemm_traffic_gamma120.md"),
+           ("update_3xtf32", (113081, 128, 256)): (3.04e8, "profiles/tc_nn_3xtf32_update_gamma120.md")}
 
 
 def roofline_of(kr, dominant=DOMINANT):
