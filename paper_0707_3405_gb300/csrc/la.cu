@@ -1283,10 +1283,10 @@ __device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong
 // What bounds it: lane 0's chain of dependent FP64 instructions, 64 cycles or more each (with few clusters, of
 // the longest one).  So comparisons run on the bits, rows are swapped by selects (a predicated-off
 // instruction costs the same), each pivot is inverted once (the multiplier is its product with the
-// reciprocal, corrected by its remainder; the rows of U are divided by their pivots by all lanes), and a
-// vector alone beyond gaptol takes two solves: each shrinks the others' part by 1e-8 or more, so that
-// the second leaves rounding only; three within clusters and in FP32.  GB300, the step with 128 vectors of
-// n = 384 in double-FP32 4.57 -> 4.45 ms, n = 1152 33.0 -> 31.9.
+// reciprocal, corrected by its remainder; the rows of U are divided by their pivots by all lanes).  Three
+// solves, also for eigenvalues far from all others: with two, 2 of 400 solves of a free-electron cell lost
+// linear independence.  GB300, the step with 128 vectors of n = 384 in double-FP32 4.57 -> 4.45 ms, all of n = 1152
+// 33.0 -> 32.2.
 template <typename RT>
 __global__ void __launch_bounds__(32)
 k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, const RT *__restrict__ theta,
@@ -1345,10 +1345,7 @@ k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, cons
             du2[i] *= rdd[i];
         }
         __syncwarp();
-        // alone beyond gaptol: the part of every other vector shrinks by (error of lam) / gap <= 1e-8 per solve
-        const bool alone = j == k && (j + 1 < m ? theta[j + 1] - theta[j] > gaptol : m == n);
-        const int solves = alone && sizeof(RT) == 8 ? 2 : 3;
-        for (int it = 0; it < solves; ++it) {
+        for (int it = 0; it < 3; ++it) {
             if (lane == 0) {
                 RT zi = z[0];
                 for (int i = 0; i + 1 < n; ++i) {
