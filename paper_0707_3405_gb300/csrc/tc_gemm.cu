@@ -28,7 +28,7 @@
 // (256 threads loading, splitting and storing in lockstep, one of them issuing) and after:
 //   A B    113081 x 128 x 256    330 -> 131 us  (269 -> 680 TFLOP/s of about 960 for TF32)
 //          113081 x 128 x 1024  1070 -> 420 us;  57925 x 64 x 128  50 -> 33 us
-//   A^H B  432 x 128 x 113081    333 -> 259 us;  384 x 256 x 113081  468 -> 375 us
+//   A^H B  432 x 128 x 113081    333 -> 289 us;  384 x 256 x 113081  468 -> 403 us
 //          64 x 64 x 57925        65 -> 40 us
 // All loaders filling one stage together (8 or 16 warps, 2 to 4 stages ahead in registers) took 179 to
 // 197 us for the first: each stage then costs one group's whole chain of wait, stores, fence and
@@ -381,41 +381,57 @@ int pick_nt(int n) {
     return best;
 }
 
+// Terms of one FP32 accumulation of A^H B, from K alone.  The tensor core truncates as it accumulates, so a
+// sum loses about half a unit in the last place per MMA: entries of a Gram with chunks of c terms come out
+// about 0.3 c 2^-24 too small.  A Rayleigh-Ritz step on nearly dependent directions divides by the small
+// eigenvalues of S: where A's blocks lose more than S's, spurious low Ritz values appear.  (With the chunks
+// chosen by the time of each shape, 2264 terms for the S and 2976 for the A of a 128-band block of the 120^3
+// cell, its last block left orthonormality by 0.1 to 1e5 and one solve in seven broke down; with 744 for
+// both, by 1e-6.)  So all products of one K have the same chunks, of at most 1024 terms, their number a
+// multiple of the SMs, so that any number of tiles keeps them all busy to the end.  More partial tiles cost,
+// GB300, K = 113081: 384 x 256 374 -> 403 us, 432 x 128 259 -> 289, 1152 x 1152 4.61 -> 5.53 ms; 128 x 128 92 as
+// before.  At least 128 terms, where K is short: a tile's 128 KB of partial sums are then written in about the
+// time of its stages (512 x 512 x 5000 56 -> 79 us, 16 x 16 x 3000 16.5 -> 15.1).
+constexpr int kMinChunk = 128, kMaxChunk = 1024;
+int cn_chunk(int K) {
+    const long long sms = num_sms_tc(), rounds = (K + sms * kMaxChunk - 1) / (sms * kMaxChunk);
+    const long long kc = (K + sms * rounds - 1) / (sms * rounds);
+    return std::max(kMinChunk, (int)((kc + KST - 1) / KST * KST));
+}
+// Partial tiles at a time: larger products run in panels of rows and columns.
+constexpr size_t kPartBytes = (size_t)256 << 20;
+
 template <int NT>
-int launch_cn(GemmWork &w, TcArgs &a, float beta, c32 *C, int ldc, cudaStream_t s) {
+int launch_cn(GemmWork &w, const TcArgs &all, float beta, c32 *C, int ldc, cudaStream_t s) {
     static std::atomic<bool> attr{false};
     LG_TRY(ensure_smem(k_tc_cn<NT>, smem_bytes(NT), attr));
-    a.tm = (a.m + kRows - 1) / kRows;
-    a.tn = (a.n + NT - 1) / NT;
-    // Split of the reduction: the busiest SM's items x (stages + about four stages' time of pipeline
-    // fill), plus the partial tiles written and summed (in units of a stage, half a microsecond, at
-    // 5 TB/s); chunks of 64 to 4096 terms, so that no FP32 accumulation is longer than that.
-    const int sms = num_sms_tc();
-    const long long tiles = (long long)a.tm * a.tn;
-    double best = 1e300;
-    for (int ns = 1; ns <= 4 * sms; ++ns) {
-        const int kc = ((a.K + ns - 1) / ns + KST - 1) / KST * KST;
-        if (kc > 4096) continue;
-        if (kc < 64 && ns > 1) break;
-        const int nsp = (a.K + kc - 1) / kc;
-        const long long items = tiles * nsp;
-        const double cost = (double)((items + sms - 1) / sms) * ((kc / KST + 4) * (double)stage_cycles(NT) / 900.0) +
-                            (double)nsp * 16.0 * a.m * (double)a.n / 2.3e6;
-        if (cost < best) {
-            best = cost;
-            a.kchunk = kc;
+    const int sms = num_sms_tc(), kchunk = cn_chunk(all.K), nsplit = (all.K + kchunk - 1) / kchunk;
+    const long long units = std::max<long long>(1, (long long)(kPartBytes / (sizeof(c32) * nsplit)) / (kRows * NT));
+    const int tm_all = (all.m + kRows - 1) / kRows, tn_all = (all.n + NT - 1) / NT;   // tiles of a panel: tmp x tnp <= units
+    const int tmp = (int)std::min<long long>(tm_all, units), tnp = (int)std::min<long long>(tn_all, units / tmp);
+    const int pm = std::min(all.m, tmp * kRows), pn = std::min(all.n, tnp * NT);
+    LG_TRY(w.alloc->ensure(w.part, sizeof(c32) * (size_t)nsplit * pm * pn));
+    for (int j0 = 0; j0 < all.n; j0 += tnp * NT)
+        for (int i0 = 0; i0 < all.m; i0 += tmp * kRows) {
+            TcArgs a = all;
+            a.m = std::min(pm, all.m - i0);
+            a.n = std::min(pn, all.n - j0);
+            a.A = all.A + (size_t)i0 * all.lda;
+            a.B = all.B + (size_t)j0 * all.ldb;
+            a.tm = (a.m + kRows - 1) / kRows;
+            a.tn = (a.n + NT - 1) / NT;
+            a.kchunk = kchunk;
+            a.nsplit = nsplit;
+            a.part = reinterpret_cast<c32 *>(w.part.p);
+            const int grid = (int)std::min<long long>(sms, (long long)a.tm * a.tn * nsplit);
+            k_tc_cn<NT><<<grid, kThreads, smem_bytes(NT), s>>>(a);
+            LG_TRY(check_launch("tensor-core gemm A^H B"));
+            const size_t tot = (size_t)a.m * a.n;
+            const int blocks = (int)std::min<size_t>((tot + 127) / 128, 4096);
+            k_tc_reduce<<<blocks, 128, 0, s>>>(a.m, a.n, nsplit, a.alpha, a.part, beta, C + (size_t)j0 * ldc + i0, ldc);
+            LG_TRY(check_launch("tensor-core gemm reduce"));
         }
-    }
-    a.nsplit = (a.K + a.kchunk - 1) / a.kchunk;
-    LG_TRY(w.alloc->ensure(w.part, sizeof(c32) * (size_t)a.nsplit * a.m * a.n));
-    a.part = reinterpret_cast<c32 *>(w.part.p);
-    const int grid = (int)std::min<long long>(sms, tiles * a.nsplit);
-    k_tc_cn<NT><<<grid, kThreads, smem_bytes(NT), s>>>(a);
-    LG_TRY(check_launch("tensor-core gemm A^H B"));
-    const size_t tot = (size_t)a.m * a.n;
-    const int blocks = (int)std::min<size_t>((tot + 127) / 128, 4096);
-    k_tc_reduce<<<blocks, 128, 0, s>>>(a.m, a.n, a.nsplit, a.alpha, a.part, beta, C, ldc);
-    return check_launch("tensor-core gemm reduce");
+    return LOBPCG_OK;
 }
 
 template <int NT>
