@@ -138,7 +138,10 @@ struct alignas(8) df64 {
     // Three quotient digits from one reciprocal r of b.hi: each digit is the remainder's high part times
     // r, and the remainder a - q b stays a pair (the high parts' difference is exact: q b.hi is within
     // a few units in the last place of what it is subtracted from).  A third of the instructions of
-    // three FP32 divisions with double-word remainders, to the same few units of 2^-48.
+    // three FP32 divisions with double-word remainders, to the same few units of 2^-48, for |b| in
+    // [2^-126, 2^126] and a remainder that FP32 holds (|a| >= 2^-100).  Smaller |b|: the reciprocal is infinite and
+    // the quotient not a number, which callers keep away from (reflectors scale their column, Sturm
+    // counts replace small pivots).
     friend __device__ __forceinline__ df64 operator/(df64 a, df64 b) {
         const float r = __frcp_rn(b.hi);
         const float q1 = __fmul_rn(a.hi, r);

@@ -371,26 +371,56 @@ __global__ void k_set_dropped_diag(int n, cx<RT> *__restrict__ A, const int *__r
 }
 
 // ------------------------------------------------------------------ tridiagonalisation
+// Range of a column: the sums of squares below keep their type's precision for |x|^2 in [lo, hi]
+// (double-FP32: the low part of a square is 2^-48 of it, and FP32 ends at 2^-149); a column outside is
+// brought to about one by a power of two f, whose inverse is a normal number.
+template <typename RT> struct ColRange {
+    using F = RT;
+    static __device__ __forceinline__ bool ok(RT t) {
+        return sizeof(RT) == 8 ? t >= (RT)0x1p-900 && t <= (RT)0x1p900 : t >= (RT)0x1p-96 && t <= (RT)0x1p96;
+    }
+};
+template <> struct ColRange<df64> {
+    using F = float;
+    static __device__ __forceinline__ bool ok(df64 t) { return t.hi >= 0x1p-96f && t.hi <= 0x1p96f; }
+};
+__device__ __forceinline__ float col_factor(float m) { return scalbnf(1.f, min(126, max(-100, -ilogbf(m)))); }
+__device__ __forceinline__ double col_factor(double m) { return scalbn(1.0, min(1000, max(-900, -ilogb(m)))); }
+__device__ __forceinline__ float scaled(float a, float f) { return a * f; }
+__device__ __forceinline__ double scaled(double a, double f) { return a * f; }
+__device__ __forceinline__ df64 scaled(df64 a, float f) { return df64(a.hi * f, a.lo * f); }
+template <typename RT>
+__device__ __forceinline__ cx<RT> scaled(cx<RT> a, typename ColRange<RT>::F f) {
+    return mkc<RT>(scaled(a.x, f), scaled(a.y, f));
+}
+__device__ __forceinline__ float high(float a) { return a; }
+__device__ __forceinline__ double high(double a) { return a; }
+__device__ __forceinline__ float high(df64 a) { return a.hi; }
+
 // Reflector of x = A[i+1:n, i] in the LAPACK larfg convention:
 //   H = I - tau v v^H, v[0] = 1, H^H x = beta e_1 with beta real.
 template <typename RT>
 struct Refl {
     cx<RT> tau;
     RT beta;
-    cx<RT> scal;  // v[r] = x[r] * scal for r >= 1
+    cx<RT> scal;                         // v[r] = (x[r] pre) scal for r >= 1
+    typename ColRange<RT>::F pre;        // a power of two; 0: x is out of range (reflector_rescaled)
+    __device__ __forceinline__ cx<RT> of(cx<RT> x) const { return (pre != 1 ? scaled<RT>(x, pre) : x) * scal; }
 };
 
 // Reflector from alpha = x[0] and s = sum_{r>=1} |x[r]|^2 (LAPACK larfg convention).
 template <typename RT>
 __device__ __forceinline__ Refl<RT> reflector_from(cx<RT> alpha, RT s) {
     Refl<RT> R;
-    if (s == 0.0 && alpha.y == 0.0) {
+    const RT t = abs2(alpha) + s;
+    R.pre = ColRange<RT>::ok(t) ? 1 : 0;
+    if (R.pre == 0 || (s == 0.0 && alpha.y == 0.0)) {
         R.tau = mkc<RT>(0.0, 0.0);
         R.beta = alpha.x;
         R.scal = mkc<RT>(0.0, 0.0);
         return R;
     }
-    const RT beta = -copysign(sqrt(abs2(alpha) + s), alpha.x);
+    const RT beta = -copysign(sqrt(t), alpha.x);
     R.beta = beta;
     R.tau = mkc<RT>((beta - alpha.x) / beta, -alpha.y / beta);
     const cx<RT> den = mkc<RT>(alpha.x - beta, alpha.y);
@@ -399,12 +429,55 @@ __device__ __forceinline__ Refl<RT> reflector_from(cx<RT> alpha, RT s) {
     return R;
 }
 
+// The reflector of a column of L entries whose |x|^2 is out of range (zero, nearly decoupled or huge columns): as
+// above on x times a power of two.  Every thread of the block calls it, and gets the result; sh holds 32
+// entries.  (Without it a double-FP32 column of norm 5e-20 or less, whose |den|^2 has no FP32
+// reciprocal, made the whole eigen-decomposition not a number, and columns below 1e-15 lost digits.)
+template <typename RT, bool CG, typename PT>
+__device__ __noinline__ Refl<RT> reflector_rescaled(const cx<PT> *col, int L, RT *sh) {
+    using F = typename ColRange<RT>::F;
+    F m = 0;                             // largest part, or not a number where one is
+    auto larger = [&m](F a) { m = a > m || a != a ? a : m; };
+    for (int r = threadIdx.x; r < L; r += blockDim.x) {
+        const cx<RT> x = CG ? ldcg_as<RT>(col + r) : ld_as<RT>(col + r);
+        larger(fabs(high(x.x)));
+        larger(fabs(high(x.y)));
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) larger(__shfl_xor_sync(0xffffffffu, m, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = RT(m);
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) larger(high(sh[w]));
+    const cx<RT> alpha = CG ? ldcg_as<RT>(col) : ld_as<RT>(col);
+    if (m == 0) {
+        Refl<RT> R = reflector_from<RT>(mkc<RT>(0.0, 0.0), RT(0.0));
+        R.pre = 1;
+        return R;
+    }
+    const F f = col_factor(m);
+    RT s = 0.0;
+    for (int r = 1 + threadIdx.x; r < L; r += blockDim.x)
+        s += abs2(scaled<RT>(CG ? ldcg_as<RT>(col + r) : ld_as<RT>(col + r), f));
+    s = block_sum(s, sh);
+    Refl<RT> R = reflector_from<RT>(scaled<RT>(alpha, f), s);
+    if (R.pre == 0) {                    // infinite or not a number: so is the result
+        const RT t = abs2(scaled<RT>(alpha, f)) + s, nan = t - t;
+        R.beta = nan;
+        R.tau = R.scal = mkc<RT>(nan, nan);
+    }
+    R.beta = scaled(R.beta, 1 / f);
+    R.pre = f;
+    return R;
+}
+
 template <typename RT, bool CG = false, typename PT = RT>
 __device__ Refl<RT> make_reflector(const cx<PT> *__restrict__ col, int L, RT *sh) {
     RT s = 0.0;
     for (int r = 1 + threadIdx.x; r < L; r += blockDim.x) s += abs2(CG ? ldcg_as<RT>(col + r) : ld_as<RT>(col + r));
     s = block_sum(s, sh);
-    return reflector_from<RT>(CG ? ldcg_as<RT>(col) : ld_as<RT>(col), s);
+    const Refl<RT> R = reflector_from<RT>(CG ? ldcg_as<RT>(col) : ld_as<RT>(col), s);
+    return R.pre != 0 ? R : reflector_rescaled<RT, CG, PT>(col, L, sh);
 }
 
 // Block sum whose cross-warp step is one warp's shuffle tree (a fixed order): for large
@@ -435,7 +508,8 @@ __device__ Refl<RT> make_reflector_bc(const cx<PT> *__restrict__ col, int L, RT 
     s = block_sum_tree(s, sh);
     if (threadIdx.x == 0) *rb = reflector_from<RT>(ld_as<RT>(col), s);
     __syncthreads();
-    return *rb;
+    const Refl<RT> R = *rb;
+    return R.pre != 0 ? R : reflector_rescaled<RT, false, PT>(col, L, sh);
 }
 
 // Step i, part 1: reflector (every block, redundantly) and y = A22 v by 32x32 tiles;
@@ -455,7 +529,7 @@ k_tri_step1(int n, int i, cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ 
     const int tr = blockIdx.x, tc = blockIdx.y;
     const int tid = threadIdx.x;
     if (tr == 0 && tc == 0) {
-        for (int r = tid; r < L; r += blockDim.x) Hv[(size_t)i * n + i + 1 + r] = (r == 0) ? mkc<RT>(1.0, 0.0) : col[r] * R.scal;
+        for (int r = tid; r < L; r += blockDim.x) Hv[(size_t)i * n + i + 1 + r] = (r == 0) ? mkc<RT>(1.0, 0.0) : R.of(col[r]);
         if (tid == 0) {
             taus[i] = R.tau;
             dg[i] = A[(size_t)i * lda + i].x;
@@ -465,7 +539,7 @@ k_tri_step1(int n, int i, cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ 
     // v entries of this column tile
     if (tid < 32) {
         const int c = tc * 32 + tid;
-        vs[tid] = (c < L) ? ((c == 0) ? mkc<RT>(1.0, 0.0) : col[c] * R.scal) : mkc<RT>(0.0, 0.0);
+        vs[tid] = (c < L) ? ((c == 0) ? mkc<RT>(1.0, 0.0) : R.of(col[c])) : mkc<RT>(0.0, 0.0);
     }
     __syncthreads();
     const int rl = tid & 31, cg = tid >> 5;  // 32 rows x 8 column groups of 4
@@ -506,7 +580,7 @@ k_tri_step1(int n, int i, cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ 
         for (int c = 0; c < ncb; ++c) {
             y = y + ldcg_cx(ypart + (size_t)c * n + rr);
         }
-        const cx<RT> v = (rr == 0) ? mkc<RT>(1.0, 0.0) : col[rr] * R.scal;
+        const cx<RT> v = (rr == 0) ? mkc<RT>(1.0, 0.0) : R.of(col[rr]);
         // conj(v) * y
         dre += v.x * y.x + v.y * y.y;
         dim += v.x * y.y - v.y * y.x;
@@ -517,7 +591,7 @@ k_tri_step1(int n, int i, cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ 
     const RT t2 = 0.5 * abs2(R.tau) * dre;
     __syncthreads();
     for (int rr = tid; rr < L; rr += blockDim.x) {
-        const cx<RT> v = (rr == 0) ? mkc<RT>(1.0, 0.0) : col[rr] * R.scal;
+        const cx<RT> v = (rr == 0) ? mkc<RT>(1.0, 0.0) : R.of(col[rr]);
         const cx<RT> y = wv[rr];
         wv[rr] = R.tau * y - t2 * v;
     }
@@ -595,7 +669,7 @@ k_tri_coop(int n, cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv, cx<R
         const int tl = (L + 31) / 32, ntiles = tl * tl;
         const cx<RT> *col = A + (size_t)i * lda + i + 1;
         const Refl<RT> R = make_reflector<RT, true>(col, L, sh);
-        for (int r = tid; r < L; r += blockDim.x) vsh[r] = (r == 0) ? mkc<RT>(1.0, 0.0) : ldcg_cx(col + r) * R.scal;
+        for (int r = tid; r < L; r += blockDim.x) vsh[r] = (r == 0) ? mkc<RT>(1.0, 0.0) : R.of(ldcg_cx(col + r));
         if (blockIdx.x == 0) {
             for (int r = tid; r < L; r += blockDim.x) Hv[(size_t)i * n + i + 1 + r] = vsh[r];
             if (tid == 0) {
@@ -716,7 +790,7 @@ k_tri_cluster(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__
     // reflector 0 from column 0 of A, d[0]
     Refl<CT> R = make_reflector_bc<CT, RT>(A + 1, n - 1, sh, &rb);
     for (int r = tid; r < n; r += blockDim.x)
-        vb[r] = (r < 1) ? zero : (r == 1 ? mkc<CT>(1.0, 0.0) : ld_as<CT>(A + r) * R.scal);
+        vb[r] = (r < 1) ? zero : (r == 1 ? mkc<CT>(1.0, 0.0) : R.of(ld_as<CT>(A + r)));
     if (q == 0 && tid == 0) dg[0] = A[0].x;
     __syncthreads();
     // y_0 = A[J,J] v_0 and column 1 on the owned rows of J = [1, n), sent to every CTA
@@ -762,7 +836,7 @@ k_tri_cluster(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__
         if (i + 2 >= n) break;  // last column: nothing left to transform
         const Refl<CT> Rn = make_reflector_bc<CT>(x + i + 2, n - i - 2, sh, &rb);
         for (int r = tid; r < n; r += blockDim.x)
-            vn[r] = (r < i + 2) ? zero : (r == i + 2 ? mkc<CT>(1.0, 0.0) : x[r] * Rn.scal);
+            vn[r] = (r < i + 2) ? zero : (r == i + 2 ? mkc<CT>(1.0, 0.0) : Rn.of(x[r]));
         __syncthreads();
         // rank-2 update of the owned rows of the trailing block [i+2, n)^2, times v_{i+1}
         const int c2 = i + 2, nxt = 1 - par;
@@ -833,14 +907,16 @@ __device__ __forceinline__ CT light_total(const CT *sh) {
 template <typename CT>
 __device__ __forceinline__ Refl<CT> reflector_warp(cx<CT> alpha, CT s) {
     Refl<CT> R;
-    if (s == CT(0.0) && alpha.y == CT(0.0)) {
+    const CT t = abs2(alpha) + s;
+    R.pre = ColRange<CT>::ok(t) ? 1 : 0;
+    if (R.pre == 0 || (s == CT(0.0) && alpha.y == CT(0.0))) {
         R.tau = mkc<CT>(0.0, 0.0);
         R.beta = alpha.x;
         R.scal = mkc<CT>(0.0, 0.0);
         return R;
     }
     const int lane = threadIdx.x & 31;
-    const CT beta = -copysign(sqrt(abs2(alpha) + s), alpha.x);
+    const CT beta = -copysign(sqrt(t), alpha.x);
     const cx<CT> den = mkc<CT>(alpha.x - beta, alpha.y);
     const CT num = (lane & 3) == 0 ? beta - alpha.x : (lane & 3) == 2 ? den.x : (lane & 3) == 1 ? -alpha.y : -den.y;
     const CT quo = num / ((lane & 2) ? abs2(den) : beta);
@@ -892,7 +968,7 @@ k_tri_rows(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv
            RT *__restrict__ dg, RT *__restrict__ eg, cx<RT> *__restrict__ xch_st, unsigned int *count, int *err) {
     static_assert(sizeof(cx<CT>) == sizeof(cx<RT>), "the compute type keeps the storage size");
     extern __shared__ __align__(16) unsigned char dsm[];
-    __shared__ CT sh[2][16], dots;
+    __shared__ CT sh[2][16], dots;   // (reflector_rescaled takes sh as 32 entries)
     __shared__ cx<CT> part[512 / 32], al;
     __shared__ Refl<CT> rs;
     const int G = gridDim.x, q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, nw = blockDim.x >> 5;
@@ -912,7 +988,8 @@ k_tri_rows(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv
     for (int r = 2 + tid; r < n; r += blockDim.x) sq = light_add<CT>(sq, abs2(ld_as<CT>(A + r)));
     light_partial(sq, sh[0]);
     Refl<CT> R = reflector_warp<CT>(ld_as<CT>(A + 1), light_total(sh[0]));
-    for (int r = tid; r < n; r += blockDim.x) v[r] = (r < 1) ? zero : (r == 1 ? mkc<CT>(1.0, 0.0) : ld_as<CT>(A + r) * R.scal);
+    if (R.pre == 0) R = reflector_rescaled<CT, false, RT>(A + 1, n - 1, sh[0]);
+    for (int r = tid; r < n; r += blockDim.x) v[r] = (r < 1) ? zero : (r == 1 ? mkc<CT>(1.0, 0.0) : R.of(ld_as<CT>(A + r)));
     if (q == 0 && tid == 0) dg[0] = A[0].x;
     __syncthreads();
     for (int i = -1; i + 1 < n; ++i) {
@@ -966,7 +1043,8 @@ k_tri_rows(int n, const cx<RT> *__restrict__ A, int lda, cx<RT> *__restrict__ Hv
             }
             __syncthreads();
             R = rs;
-            for (int r = c2 + tid; r < n; r += blockDim.x) x[r] = r == c2 ? mkc<CT>(1.0, 0.0) : x[r] * R.scal;
+            if (R.pre == 0) R = reflector_rescaled<CT, false, CT>(x + c2, n - c2, sh[0]);
+            for (int r = c2 + tid; r < n; r += blockDim.x) x[r] = r == c2 ? mkc<CT>(1.0, 0.0) : R.of(x[r]);
             vn = x;
             __syncthreads();
         }
