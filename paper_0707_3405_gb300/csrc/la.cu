@@ -1381,6 +1381,10 @@ k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, cons
     // elsewhere orthogonality is ~ eps |T| / gap (LAPACK uses 1e-3 |T| for single precision)
     const RT gaptol = (sizeof(RT) == 4 ? (RT)1e-3 : (RT)1e-5) * fmax(tnorm, Lim<RT>::tiny());
     const RT pert = 10.0 * Lim<RT>::eps() * fmax(tnorm, Lim<RT>::tiny());
+    // pivots below a hundredth of a rounding of |T| are raised to it: where lam is a decoupled diagonal entry
+    // to the last bit, the pivot is the coupling itself, and the solution its inverse squared, which overflowed
+    // (a zero vector)
+    const RT low = pert * (RT)1e-3;
     if (k > 0 && theta[k] - theta[k - 1] <= gaptol) return;  // not a cluster start
     RT lam_prev = -Lim<RT>::big();
     for (int j = k; j < m; ++j) {
@@ -1402,7 +1406,7 @@ k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, cons
                 const bool sw = mag_less(p, l);
                 RT piv = sw ? l : p;
                 const RT o = sw ? p : l, u0 = sw ? dn : u, u1 = sw ? u : dn;
-                if (is_zero(piv)) piv = pert;
+                piv = is_zero(piv) ? pert : mag_less(piv, low) ? copysign(low, piv) : piv;
                 const RT r = (RT)1.0 / piv, f0 = o * r;
                 const RT f = fma(fma(-f0, piv, o), r, f0);   // o / piv
                 rdd[i] = r;
@@ -1414,7 +1418,7 @@ k_inviter(int n, int m, const RT *__restrict__ d, const RT *__restrict__ e, cons
                 const RT t = -f * un;
                 u = sw ? t : un;
             }
-            if (is_zero(p)) p = pert;
+            p = is_zero(p) ? pert : mag_less(p, low) ? copysign(low, p) : p;
             rdd[n - 1] = (RT)1.0 / p;
         }
         __syncwarp();
