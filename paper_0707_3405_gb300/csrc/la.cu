@@ -1271,12 +1271,18 @@ k_multisect_df(int n, int m, const double *__restrict__ d, const double *__restr
     __syncwarp();
     // Gershgorin bracket in FP32, padded well above its rounding
     float lo_f = FLT_MAX, hi_f = -FLT_MAX, emax2 = 0.f;
+    bool finite = true;
     for (int i = 0; i < n; ++i) {
         float r = 0.f;
         if (i > 0) r += sqrtf(e2s[i - 1]);
         if (i < n - 1) { r += sqrtf(e2s[i]); emax2 = fmaxf(emax2, e2s[i]); }
         lo_f = fminf(lo_f, ds[i] - r);
         hi_f = fmaxf(hi_f, ds[i] + r);
+        finite = finite && fabsf(ds[i]) + r <= FLT_MAX;
+    }
+    if (!FINE64 && !finite) {   // the minima, maxima and counts would pass over what is not a number
+        if (sub == 0) theta[k] = nan("");
+        return;
     }
     const float tn = fmaxf(fabsf(lo_f), fabsf(hi_f));
     const float piv = FLT_MIN * fmaxf(1.f, fmaxf(emax2, tn * tn));
