@@ -43,6 +43,7 @@
 #include "tc.cuh"
 
 #include <algorithm>
+#include <cfloat>
 
 namespace lg {
 
@@ -320,8 +321,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_cn(TcArgs a) { tc_body<true,
 template <int NT>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_nn(TcArgs a) { tc_body<false, NT>(a); }
 
-// C = alpha (sum of the partial tiles, in split order) + beta C.  The sum is a double-FP32 pair (TwoSum):
-// FP64 additions would cost 64 cycles a warp each.
+// One entry of k_tc_reduce in FP64, for sums that leave the FP32 range on the way.
+__device__ __noinline__ c32 tc_reduce_fp64(const c32 *part, size_t tot, int nsplit, float alpha, float beta, c32 c) {
+    double re = 0.0, im = 0.0;
+    for (int z = 0; z < nsplit; ++z) {
+        re += part[(size_t)z * tot].x;
+        im += part[(size_t)z * tot].y;
+    }
+    re *= alpha;
+    im *= alpha;
+    if (beta != 0.f) {
+        re += (double)beta * c.x;
+        im += (double)beta * c.y;
+    }
+    return mkc((float)re, (float)im);
+}
+
+// C = alpha (sum of the partial tiles, in split order) + beta C.  The sum is a double-FP32 pair (TwoSum), its
+// products with alpha and beta are exact, and the result is rounded once: FP64 arithmetic would cost 64
+// cycles a warp and instruction.
 __global__ void k_tc_reduce(int m, int n, int nsplit, float alpha, const c32 *__restrict__ part, float beta,
                             c32 *C, int ldc) {
     const size_t tot = (size_t)m * n;
@@ -339,11 +357,16 @@ __global__ void k_tc_reduce(int m, int n, int nsplit, float alpha, const c32 *__
             add(rh, rl, v.x);
             add(ih, il, v.y);
         }
-        c32 v = mkc(fmaf(alpha, rh, alpha * rl), fmaf(alpha, ih, alpha * il));
-        if (beta != 0.f) {
-            const c32 c = C[(size_t)j * ldc + i];
-            v = mkc(fmaf(beta, c.x, v.x), fmaf(beta, c.y, v.y));
-        }
+        const c32 c = beta != 0.f ? C[(size_t)j * ldc + i] : mkc(0.f, 0.f);
+        auto out = [alpha, beta](float h, float l, float x) {
+            const float p = __fmul_rn(alpha, h), q = __fmul_rn(beta, x);
+            float s, t;
+            df64::two_sum(p, q, s, t);
+            t = __fadd_rn(t, __fadd_rn(__fmaf_rn(alpha, h, -p), __fmaf_rn(beta, x, -q)));
+            return __fadd_rn(s, __fmaf_rn(alpha, l, t));
+        };
+        c32 v = mkc(out(rh, rl, c.x), out(ih, il, c.y));
+        if (!(fabsf(v.x) <= FLT_MAX && fabsf(v.y) <= FLT_MAX)) v = tc_reduce_fp64(part + e, tot, nsplit, alpha, beta, c);
         C[(size_t)j * ldc + i] = v;
     }
 }
