@@ -50,7 +50,8 @@ __device__ __forceinline__ double pair_to_double(float hi, float lo) {
 // The pair of an FP64 number, hi = x rounded to nearest and lo = x - hi likewise, in integer arithmetic
 // for the same reason (and with no FP64 instruction in a rare branch: predicated off it costs the
 // same): the 53-bit mantissa is cut into 24 bits, rounded, and the signed rest.  Numbers whose low
-// part would leave the FP32 range are brought into it by 2^64 or 2^-64; below 2^-138 they are zero.
+// part would leave the FP32 range are brought into it by 2^64 or 2^-64; below 2^-138, where hi is subnormal, lo
+// is zero.
 __device__ __forceinline__ void double_to_pair(double x, float &hi, float &lo) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);   // (folds for constants)
     const uint32_t top = (uint32_t)(b >> 32), sign = top & 0x80000000u;
@@ -62,7 +63,8 @@ __device__ __forceinline__ void double_to_pair(double x, float &hi, float &lo) {
     const int ml = (int)(uint32_t)((uint32_t)m - (mh << 29));                       // in [-2^28, 2^28], mod 2^32
     hi = __uint_as_float((((uint32_t)(e + 126) << 23) + mh) | sign) * fac;           // the leading one adds the exponent
     lo = (float)ml * __uint_as_float(((uint32_t)(e - 52 + 127) << 23) | sign) * fac;
-    if (e < -74) hi = lo = 0.f;
+    if (e < -74) lo = 0.f;
+    if (e < -86) hi = 0.f;   // below half of FP32's smallest number
     if (e > 126) {   // beyond FP32's range, infinite or not a number
         const bool nan = e0 == 1024 && (b & 0xFFFFFFFFFFFFFULL) != 0;
         hi = __uint_as_float((nan ? 0x7FC00000u : 0x7F800000u) | sign);
