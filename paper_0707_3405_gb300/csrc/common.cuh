@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/lobpcg_gb300.h"
+#include "device_once.h"
 
 namespace lg {
 
@@ -80,6 +81,11 @@ const char *global_error();
                                                    cudaGetErrorString(_e));                 \
         }                                                                                   \
     } while (0)
+
+inline int current_device() {
+    int dev = -1;
+    return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
 
 #define LG_TRY(...)                                  \
     do {                                             \

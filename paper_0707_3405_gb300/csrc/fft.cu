@@ -464,13 +464,14 @@ int fft_passes(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ldx, c
     const size_t sm_ac = smem_ac<R>(g, zc);
     const int yc = 16;
     const size_t sm_b = sizeof(cx<R>) * ((size_t)N + (size_t)yc * (N + 1));
-    static std::atomic<bool> attr_set{false};
-    if (!attr_set.load()) {
+    static DeviceOnce attr_set;
+    const int dev = current_device();
+    if (!attr_set.done(dev)) {
         const int lim = max_dyn_smem();
         LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_a<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
         LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_b<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
         LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_c<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        attr_set.store(true);
+        attr_set.mark(dev);
     }
     const int ny0m = ((g.ny0 % N) + N) % N;
     const int nx0m = ((g.nx0 % N) + N) % N;
@@ -500,12 +501,13 @@ int density_passes(const FFTGeom &g, const FFTPlan &plan, const cx<R> *X, int ld
     const size_t sm_ac = smem_ac<R>(g, zc);
     const int yc = 16;
     const size_t sm_d = sizeof(cx<CT>) * ((size_t)N + (size_t)yc * (N + 1)) + sizeof(CT) * (size_t)yc * N;
-    static std::atomic<bool> attr_set{false};
-    if (!attr_set.load()) {
+    static DeviceOnce attr_set;
+    const int dev = current_device();
+    if (!attr_set.done(dev)) {
         const int lim = max_dyn_smem();
         LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_a<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
         LG_CUDA_TRY(cudaFuncSetAttribute(k_pass_d<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        attr_set.store(true);
+        attr_set.mark(dev);
     }
     if (sm_d > (size_t)max_dyn_smem()) return fail(LOBPCG_ERR_UNSUPPORTED, "density pass exceeds shared memory");
     const int ny0m = ((g.ny0 % N) + N) % N;

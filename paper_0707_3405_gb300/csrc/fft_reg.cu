@@ -585,11 +585,11 @@ int run_reg(const FFTGeom &g, const C *X, int ldx, C *Y, int ldy, int nb, const 
     constexpr int LPW = 32 / RP<N>::T;
     constexpr int NZC = (N + LPW - 1) / LPW;
     const size_t sm = tile_bytes(N, g.Py);
-    // dynamic shared-memory ceiling: the device maximum, set once (process-wide attribute)
-    static std::atomic<bool> attr{false};
-    if (!attr.load()) {
-        int dev = 0, smem_max = 0;
-        LG_CUDA_TRY(cudaGetDevice(&dev));
+    // dynamic shared-memory ceiling: the device maximum, set once (for each device)
+    static DeviceOnce attr;
+    const int dev = current_device();
+    if (!attr.done(dev)) {
+        int smem_max = 0;
         LG_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         if (sm > (size_t)smem_max) return fail(LOBPCG_ERR_UNSUPPORTED, "FFT plane tile exceeds shared memory");
         cudaFuncAttributes fa, fc;
@@ -599,7 +599,7 @@ int run_reg(const FFTGeom &g, const C *X, int ldx, C *Y, int ldy, int nb, const 
                                          smem_max - (int)fa.sharedSizeBytes));
         LG_CUDA_TRY(cudaFuncSetAttribute(k_rc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          smem_max - (int)fc.sharedSizeBytes));
-        attr.store(true);
+        attr.mark(dev);
     }
     const int ny0m = ((g.ny0 % N) + N) % N;
     const int nx0m = ((g.nx0 % N) + N) % N;
@@ -627,10 +627,10 @@ int run_reg_density(const FFTGeom &g, const C *X, int ldx, int nb, const float *
     constexpr int NZC = (N + LPW - 1) / LPW;
     const size_t sm = tile_bytes(N, g.Py);
     const size_t smd = sizeof(float) * (size_t)VS * 32 * kWarps;
-    static std::atomic<bool> attr{false};
-    if (!attr.load()) {
-        int dev = 0, smem_max = 0;
-        LG_CUDA_TRY(cudaGetDevice(&dev));
+    static DeviceOnce attr;
+    const int dev = current_device();
+    if (!attr.done(dev)) {
+        int smem_max = 0;
         LG_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         if (sm > (size_t)smem_max || smd > (size_t)smem_max)
             return fail(LOBPCG_ERR_UNSUPPORTED, "FFT plane tile exceeds shared memory");
@@ -641,7 +641,7 @@ int run_reg_density(const FFTGeom &g, const C *X, int ldx, int nb, const float *
                                          smem_max - (int)fa.sharedSizeBytes));
         LG_CUDA_TRY(cudaFuncSetAttribute(k_rd<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          smem_max - (int)fd.sharedSizeBytes));
-        attr.store(true);
+        attr.mark(dev);
     }
     const int ny0m = ((g.ny0 % N) + N) % N;
     const int nx0m = ((g.nx0 % N) + N) % N;

@@ -539,13 +539,14 @@ int run(const Fft2Args<S, R> &a) {
     if (lbs < 0) return 1;
     const size_t sm = sizeof(cx<S>) * (size_t)N * (1 + (g.Py | 1) + ((1 << lbs) | 1));
     const bool half = g.Px <= N / 2 + 1 && g.Py <= N / 2 + 1;
-    static std::atomic<bool> attr{false};
-    if (!attr.load()) {
+    static DeviceOnce attr;
+    const int dev = current_device();
+    if (!attr.done(dev)) {
         const void *fns[] = {(const void *)k_2a<S, R, N, R1, true>, (const void *)k_2c<S, R, N, R1, true>,
                              (const void *)k_2a<S, R, N, R1, false>, (const void *)k_2c<S, R, N, R1, false>};
         for (const void *f : fns)
             LG_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a.smem_max));
-        attr.store(true);
+        attr.mark(dev);
     }
     auto passes = [&](auto ka, auto kb, auto kc) -> int {
         for (int b0 = 0; b0 < a.nb; b0 += a.nbatch) {

@@ -586,14 +586,12 @@ __global__ void k_oz_finish_cn(int m, int n, int nsplit, const double *__restric
 }
 
 int ensure_attr() {
-    static std::atomic<bool> done0{false}, done1{false};
-    if (!done0.load()) {
+    static DeviceOnce once;
+    const int dev = current_device();
+    if (!once.done(dev)) {
         LG_CUDA_TRY(cudaFuncSetAttribute(k_oz_mma<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
-        done0.store(true);
-    }
-    if (!done1.load()) {
         LG_CUDA_TRY(cudaFuncSetAttribute(k_oz_mma<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
-        done1.store(true);
+        once.mark(dev);
     }
     return LOBPCG_OK;
 }

@@ -372,10 +372,11 @@ __global__ void k_tc_reduce(int m, int n, int nsplit, float alpha, const c32 *__
 }
 
 template <typename Kern>
-int ensure_smem(Kern kern, size_t bytes, std::atomic<bool> &done) {
-    if (!done.load()) {
+int ensure_smem(Kern kern, size_t bytes, DeviceOnce &once) {
+    const int dev = current_device();
+    if (!once.done(dev)) {
         LG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-        done.store(true);
+        once.mark(dev);
     }
     return LOBPCG_OK;
 }
@@ -426,7 +427,7 @@ constexpr size_t kPartBytes = (size_t)256 << 20;
 
 template <int NT>
 int launch_cn(GemmWork &w, const TcArgs &all, float beta, c32 *C, int ldc, cudaStream_t s) {
-    static std::atomic<bool> attr{false};
+    static DeviceOnce attr;
     LG_TRY(ensure_smem(k_tc_cn<NT>, smem_bytes(NT), attr));
     const int sms = num_sms_tc(), kchunk = cn_chunk(all.K), nsplit = (all.K + kchunk - 1) / kchunk;
     const long long units = std::max<long long>(1, (long long)(kPartBytes / (sizeof(c32) * nsplit)) / (kRows * NT));
@@ -459,7 +460,7 @@ int launch_cn(GemmWork &w, const TcArgs &all, float beta, c32 *C, int ldc, cudaS
 
 template <int NT>
 int launch_nn(TcArgs &a, cudaStream_t s) {
-    static std::atomic<bool> attr{false};
+    static DeviceOnce attr;
     LG_TRY(ensure_smem(k_tc_nn<NT>, smem_bytes(NT), attr));
     a.tm = (a.m + kRows - 1) / kRows;
     a.tn = (a.n + NT - 1) / NT;
