@@ -424,15 +424,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
                 if (++s == kRing) { s = 0; ph ^= 1; }
             }
         }
-        if (late) {
-            if (el) {
-                *abort_flag = 1;
-                atomicExch(&g_oz_err, 1);
-            }
-            // wait (bounded) for the last stages' MMAs before the CTA frees its TMEM
-            const int nst = nc * kChunkStages;
-            if (nst > 0) mbar_wait(&empty[(nst - 1) % kRing], (uint32_t)(((nst - 1) / kRing) & 1));
+        if (late && el) {
+            *abort_flag = 1;
+            atomicExch(&g_oz_err, 1);
         }
+        // wait (bounded) for the last stage's MMAs: its arrival follows that of the last level, which is all the
+        // epilogue waits for, and neither it nor an MMA may outlive the CTA's shared memory and TMEM
+        const int nst = nc * kChunkStages;
+        if (nst > 0) mbar_wait(&empty[(nst - 1) % kRing], (uint32_t)(((nst - 1) / kRing) & 1));
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns kCols (w / 4) ..
         const int wq = warp & 3, h = warp >> 2;
