@@ -147,10 +147,10 @@ int lobpcg_k_heev(int n, const void *A, double *w, void *V, void *stream);
 int lobpcg_k_set_gemm_mode(int mode);
 
 /*
- * Poll limit of the waits inside the complex64 tensor-core GEMMs on the current
+ * Poll limit of the waits inside the tensor-core GEMMs on the current
  * device: before a warp refills a shared-memory stage it waits, at most `polls`
- * times, for the MMAs that read it.  polls < 0 restores the default (2^26 polls,
- * seconds).  A wait that runs out sets a device flag, which
+ * times, for the MMAs that read it.  polls < 0 restores the default (2^21 polls,
+ * about 8 seconds).  A wait that runs out sets a device flag, which
  * lobpcg_k_check_timeouts and every solve sweep turn into LOBPCG_ERR_TIMEOUT,
  * and is repeated once with the default limit, so that the kernel still ends
  * with its work drained and its tensor memory freed.  This exists so that tests

@@ -276,9 +276,10 @@ int oz_gemm_cn(GemmWork &w, int m, int n, int K, double alpha, const z64 *A, int
                double beta, z64 *C, int ldc, cudaStream_t s, bool lower);
 int oz_gemm_nn(GemmWork &w, int M, int n, int k, double alpha, const z64 *A, int lda, const z64 *B, int ldb,
                double beta, const z64 *C, int ldc, z64 *D, int ldd, cudaStream_t s);
+int oz_set_spin_limit(long long polls);
 int oz_check_error();   // LOBPCG_ERR_TIMEOUT if a wait inside oz_gemm ran out (clears the flag)
 // Complex64 products on the tensor cores (3xTF32 split operands, FP32 accumulation):
-// C = alpha A^H B + beta C (K split over the GPU, FP64 partial sums) and
+// C = alpha A^H B + beta C (K split over the GPU, FP32 partial tiles summed as pairs) and
 // D = alpha A B + beta C.  gemm_cn<float> / gemm_nn<float> route here for long
 // reductions / tall products unless the GEMM mode says otherwise.
 int tc_gemm_cn(GemmWork &w, int m, int n, int K, float alpha, const c32 *A, int lda, const c32 *B, int ldb,

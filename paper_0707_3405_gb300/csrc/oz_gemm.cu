@@ -48,8 +48,9 @@
 // levels of the one before it, and an item while the output of the one before it, are still read.
 // Long reductions (A^H B) are split over the GPU and cut into K slabs that bound the digit
 // scratch; FP64 partial tiles are summed in a fixed order (reproducible).  Every mbarrier wait is
-// bounded; a wait that runs out sets a device flag (read by oz_check_error), and the CTA waits
-// (bounded) for its copies and MMAs in flight, frees its TMEM and returns.
+// bounded; one that runs out sets a device flag (read by oz_check_error), the CTA's warps leave their
+// loops, and it waits (bounded) for its copies and MMAs in flight, frees its TMEM and returns.  (The
+// producer's first wait for a stage, whose limit tests lower, is repeated with the full limit.)
 //
 // What bounds it: the tensor cores would take 36 cycles an MMA (the left slice held in the
 // collector, the right one read at 128 bytes a cycle), 6000 a chunk; issue, the waits for the
@@ -86,7 +87,6 @@ constexpr int kStageA = kSlices * kTileA;    // 48 KB
 constexpr int kStageB = kSlices * kTileB;    // 24 KB
 constexpr int kStageBytes = kStageA + kStageB;
 constexpr int kRing = 3;
-constexpr long long kMmaSpin = 1 << 18;      // polls of one wait of the MMA warp (milliseconds)
 constexpr int kEpiWarps = 16;
 constexpr int kCols = TQ / (kEpiWarps / 4);  // columns of a tile row that one epilogue warp folds
 constexpr int kThreads = 32 * (kEpiWarps + 2);   // + producer warp + MMA warp
@@ -99,7 +99,11 @@ constexpr int kRowsPlain = 0;   // one row (re, im)                     left of 
 constexpr int kRowsCnB = 1;     // two rows (re, im), (im, -re)         right of A^H B
 constexpr int kRowsNnA = 2;     // two rows (re, -im), (im, re)         left of A B
 
+constexpr long long kMmaSpin = 1 << 15;      // polls of one wait of the MMA warp (an eighth of a second)
+
 __device__ int g_oz_err = 0;
+// Poll limit of the producer's first wait for a stage (lowered only by tests of the timeout path).
+__device__ long long g_oz_spin = kSpinLimit;
 
 // Byte offset of BF16 element (r, c) (c < 32) in a 64-byte-swizzled K-major tile:
 // the 16-byte chunk c / 8 of row r sits at chunk position (c / 8) ^ ((r / 2) % 4).
@@ -379,6 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
     if (warp == kEpiWarps) {
         // ---- producer: one bulk copy per factor per stage
         if (lane == 0) {
+            const long long spin = g_oz_spin;
             int g = 0;
             for (int it = it0; it < nit && !*abort_flag; it += step) {
                 const OzItem w = oz_item(a, it);
@@ -386,9 +391,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
                 const unsigned char *gB = a.Bt + ((size_t)w.qt * a.KS + (size_t)w.c0 * kChunkStages) * kStageB;
                 for (int t = 0; t < w.nch * kChunkStages && !*abort_flag; ++t, ++g) {
                     const int s = g % kRing;
-                    if (g >= kRing && !mbar_wait(&empty[s], (uint32_t)((g / kRing - 1) & 1))) {
-                        *abort_flag = 1;
-                        break;
+                    const uint32_t par = (uint32_t)((g / kRing - 1) & 1);
+                    if (g >= kRing && !mbar_wait(&empty[s], par, spin)) {
+                        atomicExch(&g_oz_err, 1);
+                        if (!mbar_wait(&empty[s], par)) {
+                            *abort_flag = 1;
+                            break;
+                        }
                     }
                     unsigned char *sA = base + s * kStageBytes, *sB = sA + kStageA;
                     mbar_expect_tx(&full[s], kStageBytes);
@@ -400,11 +409,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
             for (int h = max(0, g - kRing); h < g; ++h) mbar_wait(&full[h % kRing], (uint32_t)((h / kRing) & 1));
         }
     } else if (warp == kEpiWarps + 1) {
-        // ---- MMA issuer: the whole warp, one elected lane issuing.  Nothing in its loop depends on how
-        // a wait ended, its limit included: a branch or a predicate that does makes the compiler give
-        // up uniform registers (80 cycles an MMA instead of 45).  A wait that runs out (kMmaSpin polls,
-        // so that even a CTA whose every wait runs out ends within seconds) is recorded, the rest is
-        // issued on whatever the ring holds, and the error flag discards the result.
+        // ---- MMA issuer: the whole warp, one elected lane issuing.  Nothing in a chunk depends on how
+        // a wait ended: a branch or a predicate that does, or a look at the abort flag between the polls of a
+        // wait, makes the compiler give up uniform registers (80 cycles an MMA instead of 45, the whole kernel
+        // 20 % slower).  A wait that runs out is recorded, the rest of the chunk is issued on whatever the
+        // ring holds, and the error flag discards the result; the abort flag, which the other warps raise when
+        // theirs run out, is looked at before every chunk.
         const uint32_t el = elect_one();
         const uint32_t d0 = (uint32_t)make_desc_sw64(uniform(smem_u32(base)));
         bool late = false;
@@ -412,7 +422,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
         uint32_t ph = 0;                     // and its phase
         int nc = 0;                          // chunks of all this CTA's items
         for (int it = it0; it < nit; it += step) nc += max(0, min(a.nchunks - it / a.tiles * a.cps, a.cps));
-        for (int ci = 0; ci < nc; ++ci) {
+        int ci = 0;
+        for (; ci < nc; ++ci) {
+            if (uniform((uint32_t)*abort_flag)) break;
             const int u0 = kLevels * ci;     // level L of chunk ci is the (u0 + L)-th level of the CTA
             for (int st = 0; st < kChunkStages; ++st) {
                 late |= !mbar_wait(&full[s], ph, kMmaSpin);
@@ -430,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_mma(OzArgs a) {
         }
         // wait (bounded) for the last stage's MMAs: its arrival follows that of the last level, which is all the
         // epilogue waits for, and neither it nor an MMA may outlive the CTA's shared memory and TMEM
-        const int nst = nc * kChunkStages;
+        const int nst = ci * kChunkStages;
         if (nst > 0) mbar_wait(&empty[(nst - 1) % kRing], (uint32_t)(((nst - 1) / kRing) & 1));
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns kCols (w / 4) ..
@@ -752,6 +764,12 @@ int oz_gemm_nn(GemmWork &w, int M, int n, int k, double alpha, const z64 *A, int
         k_oz_mma<1><<<std::min(num_sms(), a.tiles), kThreads, kSmem, s>>>(a);
         LG_TRY(check_launch("FP64-class tensor-core GEMM A B"));
     }
+    return LOBPCG_OK;
+}
+
+int oz_set_spin_limit(long long polls) {
+    const long long v = polls < 0 ? kSpinLimit : polls;
+    LG_CUDA_TRY(cudaMemcpyToSymbol(g_oz_spin, &v, sizeof(v)));
     return LOBPCG_OK;
 }
 

@@ -4,7 +4,7 @@
 // stored row after row; rows are grouped by 8 into 512-byte atoms (tile base 512-byte aligned),
 // and the 16-byte chunk c of row r sits at chunk position c ^ ((r / 2) % 4).
 //
-// Every wait in here is bounded: a wait that runs out sets *err and returns.
+// Every wait in here is bounded: a wait that runs out returns false, which its caller reports.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -13,7 +13,7 @@
 namespace lg {
 namespace tc {
 
-constexpr long long kSpinLimit = 1LL << 26;   // ~ seconds of polling at most
+constexpr long long kSpinLimit = 1LL << 21;   // polls of one wait: about 8 s (the hardware suspends each for 4 us)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -153,6 +153,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, long 
         if (ok) return true;
     }
     return false;
+}
+
+// A wait that does not tell how it ended (for warps that issue MMAs, whose code should not depend on it): the first
+// of a CTA that runs out sets *quit (shared memory, zeroed before), which ends the others at their next poll.
+__device__ __forceinline__ void mbar_wait_quit(uint64_t *mbar, uint32_t parity, volatile int *quit) {
+    long long it = 0;
+    for (; it < kSpinLimit; ++it) {
+        if (mbar_wait(mbar, parity, 1) || *quit) break;
+    }
+    if (it == kSpinLimit) *quit = 1;
 }
 
 // 32 lanes x 16 consecutive 32-bit columns of TMEM into registers (one warp), which hold the values

@@ -34,10 +34,10 @@
 // 197 us for the first: each stage then costs one group's whole chain of wait, stores, fence and
 // signal, which the slot groups overlap.
 //
-// Every mbarrier wait is bounded.  A loader's wait that runs out raises a device flag (read by
-// tc_check_error), is repeated with the full limit, and the CTA carries on, so that it always ends
-// with its copies and MMAs done and its TMEM freed; the MMA warp's and the readers' waits raise the
-// flag and go on without what they waited for.
+// Every mbarrier wait is bounded.  A loader's first wait for its slot, whose limit tests lower, raises a device flag
+// (read by tc_check_error) and is repeated with the full limit.  When that or another wait runs out, the flag is
+// raised, the other waits end at their next poll, and every warp goes on without what it waited for, so that the
+// CTA ends with its copies and MMAs done and its TMEM freed.
 #include "common.cuh"
 #include "df64.cuh"
 #include "tc.cuh"
@@ -57,7 +57,6 @@ constexpr int KST = 8;       // complex K per stage: 16 floats = one 64-byte sha
 constexpr int ROWB = 64;     // bytes per shared row
 constexpr int kRing = 4;
 constexpr int kRows = 128;   // vectors of the left factor per tile (MMA M)
-constexpr long long kPipeSpin = 1 << 18;   // polls of one wait of the MMA and reader warps (milliseconds)
 
 __device__ int g_tc_err = 0;
 // Poll limit of the loaders' first wait for a stage (lowered only by tests of the timeout path).
@@ -129,6 +128,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
     uint64_t *full = reinterpret_cast<uint64_t *>(base + kRing * STAGE);
     uint64_t *empty = full + kRing, *accf = empty + kRing, *acce = accf + 2;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + 2);
+    volatile int *quit = reinterpret_cast<volatile int *>(tslot + 1);
     const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
     if (warp == kLoaders) tmem_alloc(tslot, TCOLS);
     if (tid == 0) {
@@ -140,6 +140,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
             mbar_init(&accf[b], 1);
             mbar_init(&acce[b], kReaders);
         }
+        *quit = 0;
     }
     fence_before_sync();
     __syncthreads();
@@ -191,9 +192,9 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
         unsigned char *sAh = base + s * STAGE, *sAl = sAh + A_BYTES, *sBh = sAl + A_BYTES, *sBl = sBh + B_BYTES;
         if (more) load();
         for (uint32_t n = 0; more; ++n) {                  // n-th filling of the slot
-            if (n > 0 && !mbar_wait(&empty[s], (n - 1) & 1u, spin)) {
+            if (n > 0 && !mbar_wait(&empty[s], (n - 1) & 1u, *quit ? 1 : spin)) {
                 atomicExch(&g_tc_err, 1);
-                mbar_wait(&empty[s], (n - 1) & 1u);
+                mbar_wait_quit(&empty[s], (n - 1) & 1u, quit);
             }
             if (CN) {
 #pragma unroll
@@ -233,7 +234,6 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
         const uint32_t el = elect_one();
         constexpr uint32_t HI = (uint32_t)(make_desc_sw64(0) >> 32), IDESC = make_idesc_tf32(kRows, ACC);
         const uint32_t d0 = (uint32_t)make_desc_sw64(uniform(smem_u32(base)));
-        bool late = false;
         int s = 0, g = 0;
         uint32_t ph = 0;
         int q = 0;                                         // items so far
@@ -242,9 +242,9 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
             const int nst = (min(a.K, kbeg + a.kchunk) - kbeg + KST - 1) / KST;
             const int b = q & 1;
             const uint32_t dt = tmem + (uint32_t)(b * ACC);
-            if (q >= 2) late |= !mbar_wait(&acce[b], (uint32_t)((q / 2 - 1) & 1), kPipeSpin);
+            if (q >= 2) mbar_wait_quit(&acce[b], (uint32_t)((q / 2 - 1) & 1), quit);
             for (int t = 0; t < nst; ++t, ++g) {
-                late |= !mbar_wait(&full[s], ph, kPipeSpin);
+                mbar_wait_quit(&full[s], ph, quit);
                 __syncwarp();
                 fence_after_sync();
                 const uint32_t ah = d0 + ((uint32_t)(s * STAGE) >> 4), bh = ah + ((2 * A_BYTES) >> 4);
@@ -260,7 +260,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
             }
             mma_commit_warp(el, &accf[b]);
         }
-        if (late && el) atomicExch(&g_tc_err, 1);
+        if (*quit && el) atomicExch(&g_tc_err, 1);
         // every MMA is done before the CTA frees its TMEM
         if (g > 0) mbar_wait(&empty[(g - 1) % kRing], (uint32_t)(((g - 1) / kRing) & 1));
     } else {
@@ -272,7 +272,7 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
             const TcItem w = tc_item<NT>(a, it);
             const int b = q & 1, i = w.i0 + r, nj = min(NT, a.n - w.j0);
             const bool row_ok = i < a.m;
-            late |= !mbar_wait(&accf[b], (uint32_t)((q / 2) & 1), kPipeSpin);
+            late |= !mbar_wait(&accf[b], (uint32_t)((q / 2) & 1));
             __syncwarp();
             fence_after_sync();
             const uint32_t t0 = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * ACC);
@@ -531,10 +531,11 @@ int *device_wait_flag() {
 int tc_set_spin_limit(long long polls) {
     const long long v = polls < 0 ? kSpinLimit : polls;
     LG_CUDA_TRY(cudaMemcpyToSymbol(g_tc_spin, &v, sizeof(v)));
-    return LOBPCG_OK;
+    return oz_set_spin_limit(polls);
 }
 
 int tc_check_error() {
+    const int oz = oz_check_error();   // (both flags are read and cleared)
     int h = 0;
     LG_CUDA_TRY(cudaMemcpyFromSymbol(&h, g_tc_err, sizeof(int)));
     if (h) {
@@ -543,7 +544,7 @@ int tc_check_error() {
         return fail(LOBPCG_ERR_TIMEOUT,
                     "a bounded device wait ran out (tensor-core GEMM mbarrier or tridiagonalisation grid barrier)");
     }
-    return oz_check_error();
+    return oz;
 }
 
 }  // namespace lg
