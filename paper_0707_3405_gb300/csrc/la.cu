@@ -1368,8 +1368,8 @@ __device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong
 // the longest one).  So comparisons run on the bits, rows are swapped by selects (a predicated-off
 // instruction costs the same), each pivot is inverted once (the multiplier is its product with the
 // reciprocal, corrected by its remainder; the rows of U are divided by their pivots by all lanes).  Three
-// solves, also for eigenvalues far from all others: with two, 2 of 400 solves of a free-electron cell lost
-// linear independence.  GB300, the step with 128 vectors of n = 384 in double-FP32 4.57 -> 4.45 ms, all of n = 1152
+// solves for every vector: two for eigenvalues far from all others take 1 % off the step at n = 1152 and
+// nothing below.  GB300, the step with 128 vectors of n = 384 in double-FP32 4.57 -> 4.45 ms, all of n = 1152
 // 33.0 -> 32.2.
 template <typename RT>
 __global__ void __launch_bounds__(32)
@@ -1779,7 +1779,7 @@ int launch_tri_rows(EigWork &w, int n, const cx<RT> *A, int lda, cx<RT> *Hv, cx<
     done = true;
     return LOBPCG_OK;
 }
-// One cluster's barrier is cheaper than the grid's, its 8 or 16 SMs' arithmetic dearer: 1.48 against
+// One cluster's barrier is cheaper than the grid's, its eight SMs' arithmetic dearer: 1.48 against
 // 1.52 ms at n = 128 (double-FP32 step, m = n / 3), 2.50 against 2.26 at n = 192; FP64 3.10 / 3.03, 5.45 / 4.51.
 constexpr int kTriClusterMaxN = 128;
 constexpr int kWyChunks = 8;   // row chunks of the back-transformation's Gram partials
