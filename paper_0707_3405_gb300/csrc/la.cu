@@ -1785,7 +1785,8 @@ constexpr int kTriClusterMaxN = 128;
 constexpr int kWyChunks = 8;   // row chunks of the back-transformation's Gram partials
 
 // T factors, then the blocked application; NV eigenvectors per CTA, as many as keep about
-// 128 CTAs or more (each CTA reads every reflector once).
+// 128 CTAs or more (each CTA reads every reflector once) and fit its shared memory (8 up to n = 1752,
+// 4 up to 3568).
 template <typename RT, typename CT>
 int backtransform_wy(int n, int m, const cx<CT> *Hv, const cx<CT> *taus, cx<CT> *Tf, cx<CT> *Gp, const RT *Z,
                      cx<RT> *V, int ldv, cudaStream_t s) {
@@ -1795,7 +1796,10 @@ int backtransform_wy(int n, int m, const cx<CT> *Hv, const cx<CT> *taus, cx<CT> 
     LG_TRY(check_launch("back-transform Gram partials"));
     k_wy_t<CT><<<nblk, 256, 0, s>>>(n, nch, Gp, taus, Tf);
     LG_TRY(check_launch("back-transform T factors"));
-    const int NV = m >= 8 * 128 ? 8 : m >= 4 * 128 ? 4 : m >= 2 * 128 ? 2 : 1;
+    int NV = m >= 8 * 128 ? 8 : m >= 4 * 128 ? 4 : m >= 2 * 128 ? 2 : 1;
+    int smem_max = 0;
+    LG_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, current_device()));
+    while (NV > 1 && sizeof(cx<CT>) * (size_t)NV * (n + 2 * kWy) > (size_t)smem_max) NV /= 2;
     const size_t smem = sizeof(cx<CT>) * (size_t)NV * n;
     const int grid = (m + NV - 1) / NV;
     auto run = [&](auto kern) -> int {
