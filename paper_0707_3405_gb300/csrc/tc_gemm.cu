@@ -188,13 +188,18 @@ __device__ __forceinline__ void tc_body(const TcArgs &a) {
                 rb[q] = (j < a.n && k < lw.kend) ? __ldg(reinterpret_cast<const float2 *>(a.B + (size_t)j * a.ldb + k)) : zero;
             }
         };
-        const long long spin = g_tc_spin;
+        // the first polls (a millisecond) do not look at *quit, which would cost a shared-memory read a stage (2 %)
+        const long long spin = g_tc_spin, first = min(spin, 256LL);
         unsigned char *sAh = base + s * STAGE, *sAl = sAh + A_BYTES, *sBh = sAl + A_BYTES, *sBl = sBh + B_BYTES;
         if (more) load();
         for (uint32_t n = 0; more; ++n) {                  // n-th filling of the slot
-            if (n > 0 && !mbar_wait(&empty[s], (n - 1) & 1u, *quit ? 1 : spin)) {
-                atomicExch(&g_tc_err, 1);
-                mbar_wait_quit(&empty[s], (n - 1) & 1u, quit);
+            if (n > 0 && !mbar_wait(&empty[s], (n - 1) & 1u, first)) {
+                bool ok = false;
+                for (long long p = first; p < spin && !ok && !*quit; ++p) ok = mbar_wait(&empty[s], (n - 1) & 1u, 1);
+                if (!ok) {
+                    atomicExch(&g_tc_err, 1);
+                    mbar_wait_quit(&empty[s], (n - 1) & 1u, quit);
+                }
             }
             if (CN) {
 #pragma unroll
