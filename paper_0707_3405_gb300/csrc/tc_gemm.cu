@@ -26,7 +26,7 @@
 // rows kept in the collector, 64 KB of shared-memory reads beside the loaders' 48 KB of stores, 896
 // cycles of shared-memory bandwidth.  Measured on a GB300 (tensor rate: 3 x 8 m n K flops), before
 // (256 threads loading, splitting and storing in lockstep, one of them issuing) and after:
-//   A B    113081 x 128 x 256    330 -> 131 us  (269 -> 680 TFLOP/s of about 960 for TF32)
+//   A B    113081 x 128 x 256    330 -> 134 us  (269 -> 664 TFLOP/s of about 960 for TF32)
 //          113081 x 128 x 1024  1070 -> 420 us;  57925 x 64 x 128  50 -> 33 us
 //   A^H B  432 x 128 x 113081    333 -> 289 us;  384 x 256 x 113081  468 -> 403 us
 //          64 x 64 x 57925        65 -> 40 us
